@@ -15,7 +15,7 @@
 #include "adasd_cluster.cuh"
 #include "adasd_spec.cuh"
 #include "adasd_draft.cuh"
-#include "adasd_vanilla.cuh"
+#include "adasd_stream.cuh"
 #include "adasd_modes.cuh"
 
 using namespace adasd;
@@ -26,17 +26,14 @@ struct adasd_ctx {
     Scratch sc;
     std::vector<void*> allocs;
     int sm_count;
-    // warp-specialised verification kernel, one configuration per mode (AdaSD, vanilla);
-    // iter == 0 means not usable for this V / dtype
+    // warp-specialised verification kernel; iter == 0 means not usable for this V / dtype
     struct Fast {
         int iter;             // iterations per warp and row (template parameter)
         int cs;               // CTAs per cluster
         int smem;             // dynamic shared memory per CTA
         ClusterGeom geom;
-    } fast[2];
+    } fast;
     bool draft_stream;        // the streaming draft kernel is usable for this V / dtype
-    bool lse_stream;          // ... and so is the row log-sum-exp kernel of the vanilla mode
-    bool sample_stream;       // ... and its sampling kernel (the vocabulary fits its chunk tables)
     bool cut_hist;            // the one-pass cutoff kernel got its 128 KB of shared memory
     // adjusted distribution (adasd_set_warpers) and the per-row cutoffs a call works out
     float temperature;
@@ -45,6 +42,9 @@ struct adasd_ctx {
     float* cut_t;             // [B,Kmax+1]
     float* cut_d;             // [B,Kmax]
     float* cut_row;           // [B] draft step
+    float4* seg;              // [B (2 Kmax + 1)][2^seg_bits]: row statistics of the vanilla and greedy modes by segment
+    uint32_t* stream_next;    // items its warps have drawn (0 between launches)
+    int seg_bits, stream_it;  // ... of which there are 2^seg_bits; iterations of a chunk
     bool cuts_on() const { return (top_k > 0 && top_k < cfg.V) || top_p < 1.f; }
     bool warp_on() const { return cuts_on() || temperature != 1.f; }
 };
@@ -207,7 +207,7 @@ int fast_static_smem_iter(int iter) {
 // elements only.
 template <int MODE>
 void fast_setup_mode(adasd_ctx* c, size_t smem_optin) {
-    adasd_ctx::Fast& f = c->fast[MODE];
+    adasd_ctx::Fast& f = c->fast;
     f.iter = 0;
     const int V = c->cfg.V;
     if (c->cfg.dtype != ADASD_BF16 || (V & 7) != 0 || V < 8192) return;
@@ -235,11 +235,8 @@ void fast_setup_mode(adasd_ctx* c, size_t smem_optin) {
 }
 void fast_setup(adasd_ctx* c, size_t smem_optin) {
     fast_setup_mode<MODE_ADASD>(c, smem_optin);
-    fast_setup_mode<MODE_VANILLA>(c, smem_optin);
     // streaming draft kernel: bf16 rows of a multiple of 8 logits, two 4 KB buffers per warp
     c->draft_stream = false;
-    c->lse_stream = false;
-    c->sample_stream = false;
     c->cut_hist = cudaFuncSetAttribute(row_cutoff_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kHistWords * 4) == cudaSuccess;
     if (!c->cut_hist) cudaGetLastError();
@@ -257,21 +254,77 @@ void fast_setup(adasd_ctx* c, size_t smem_optin) {
             c->draft_stream = true;
         else
             cudaGetLastError();
-        if (cudaFuncSetAttribute(row_lse_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kLW * 2 * kLChunkBytes) == cudaSuccess &&
-            cudaFuncSetAttribute(row_lse_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kLW * 2 * kLChunkBytes) == cudaSuccess)
-            c->lse_stream = true;
-        else
-            cudaGetLastError();
-        if (V <= kVMaxV) {
-            if (cudaFuncSetAttribute(vanilla_sample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     kVW * 4 * kVChunkBytes) == cudaSuccess)
-                c->sample_stream = true;
-            else
-                cudaGetLastError();
-        }
     }
+}
+
+// Chunk length and segments of a row in the vanilla and greedy modes.  Chunks of 8 iterations (4 KB)
+// where every warp of the grid gets two of them, else of 2; segments of at least two chunks while that
+// gives the warps six items each (half as long measured 33 instead of 31.8 us on 544 rows of 128256),
+// shorter ones only where warps would have nothing to do.
+void stream_setup(adasd_ctx* c) {
+    const int N = c->cfg.dtype == ADASD_BF16 ? 8 : 4, NU = (c->cfg.V + N - 1) / N;
+    const long long rows = (long long)c->cfg.B * (2 * c->cfg.Kmax + 1), warps = 2LL * c->sm_count * kRW;
+    const int nc8 = (NU + 255) / 256;
+    c->stream_it = rows * nc8 >= 2 * warps ? 8 : 2;
+    const int NC = c->stream_it == 8 ? nc8 : (NU + 63) / 64;
+    int bits = 0;
+    while ((2 << bits) <= std::min(kMaxSegs, NC) &&
+           ((rows << bits) < warps || ((rows << bits) < 6 * warps && (NC >> bits) >= 4)))
+        ++bits;
+    c->seg_bits = bits;
+}
+
+template <typename T, bool ALIGNED, int IT>
+cudaError_t stream_prepare_it() {
+    cudaError_t e = cudaFuncSetAttribute(row_stream_kernel<T, ALIGNED, OP_LSE, false, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(row_stream_kernel<T, ALIGNED, OP_LSE, true, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(row_stream_kernel<T, ALIGNED, OP_ARGMAX, false, IT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRSmem);
+    return e;
+}
+template <typename T, bool ALIGNED>
+cudaError_t stream_prepare(int it) { return it == 8 ? stream_prepare_it<T, ALIGNED, 8>() : stream_prepare_it<T, ALIGNED, 2>(); }
+
+// Launch with programmatic stream serialisation: the kernel may become resident while the one ahead of
+// it is still running (it waits before it reads what that one wrote).
+template <typename K, typename... Args>
+int launch_pdl(K kernel, int grid, int threads, int smem, int cs, cudaStream_t stream, const Args&... args) {
+    cudaLaunchConfig_t lc;
+    memset(&lc, 0, sizeof(lc));
+    lc.gridDim = dim3((unsigned)grid, 1, 1);
+    lc.blockDim = dim3((unsigned)threads, 1, 1);
+    lc.dynamicSmemBytes = (size_t)smem;
+    lc.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)cs;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    lc.attrs = attr;
+    lc.numAttrs = cs > 1 ? 2 : 1;
+    CUDA_TRY(cudaLaunchKernelEx(&lc, kernel, args...));
+    return ADASD_OK;
+}
+
+template <typename T, bool ALIGNED, int IT>
+int launch_stream_it(adasd_ctx* c, const StreamParams& p, int op, cudaStream_t stream) {
+    const long long rows = (long long)p.B * (p.zd ? 2 * p.Kmax + 1 : p.Kmax + 1);
+    const int grid = (int)std::min<long long>(((rows << p.seg_bits) + kRW - 1) / kRW, 2LL * c->sm_count);
+    if (op == OP_ARGMAX) return launch_pdl(row_stream_kernel<T, ALIGNED, OP_ARGMAX, false, IT>, grid, kRThreads, kRSmem, 1, stream, p);
+    return c->warp_on() ? launch_pdl(row_stream_kernel<T, ALIGNED, OP_LSE, true, IT>, grid, kRThreads, kRSmem, 1, stream, p)
+                        : launch_pdl(row_stream_kernel<T, ALIGNED, OP_LSE, false, IT>, grid, kRThreads, kRSmem, 1, stream, p);
+}
+template <typename T, bool ALIGNED>
+int launch_stream(adasd_ctx* c, const StreamParams& p, int op, cudaStream_t stream) {
+    return c->stream_it == 8 ? launch_stream_it<T, ALIGNED, 8>(c, p, op, stream) : launch_stream_it<T, ALIGNED, 2>(c, p, op, stream);
+}
+int launch_stream(adasd_ctx* c, const StreamParams& p, int op, bool aligned, cudaStream_t stream) {
+    if (c->cfg.dtype == ADASD_BF16)
+        return aligned ? launch_stream<__nv_bfloat16, true>(c, p, op, stream) : launch_stream<__nv_bfloat16, false>(c, p, op, stream);
+    return aligned ? launch_stream<float, true>(c, p, op, stream) : launch_stream<float, false>(c, p, op, stream);
 }
 
 // CTAs per row for the streaming draft kernel: enough to fill the SMs, and few enough chunks
@@ -291,7 +344,7 @@ int draft_stream_p(const adasd_ctx* c) {
 template <int ITER, int MODE, bool WARPED>
 int fast_launch(adasd_ctx* c, const VerifyParams& p, cudaStream_t stream) {
     const long long positions = (long long)p.B * (p.Kmax + 1);
-    const adasd_ctx::Fast& f = c->fast[MODE];
+    const adasd_ctx::Fast& f = c->fast;
     ClusterGeom gq = f.geom;
     if (positions < gq.ncl) gq.ncl = (int)positions;
     cudaLaunchConfig_t lc;
@@ -319,11 +372,11 @@ template <int MODE>
 int fast_launch_iter(adasd_ctx* c, const VerifyParams& p, cudaStream_t stream) {
     if (c->warp_on()) {
 #define CALL(I) fast_launch<I, MODE, true>(c, p, stream)
-        ADASD_ITER_SWITCH(c->fast[MODE].iter, CALL, ADASD_ERR_SHAPE)
+        ADASD_ITER_SWITCH(c->fast.iter, CALL, ADASD_ERR_SHAPE)
 #undef CALL
     }
 #define CALL(I) fast_launch<I, MODE, false>(c, p, stream)
-    ADASD_ITER_SWITCH(c->fast[MODE].iter, CALL, ADASD_ERR_SHAPE)
+    ADASD_ITER_SWITCH(c->fast.iter, CALL, ADASD_ERR_SHAPE)
 #undef CALL
 }
 
@@ -411,53 +464,21 @@ int launch_cutoffs(adasd_ctx* ctx, const void* z, long long seq_stride, long lon
     return ADASD_OK;
 }
 
+// ... of the rows of a verification round
+int launch_round_cutoffs(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
+    if (!ctx->cuts_on()) return ADASD_OK;
+    if (int rc = launch_cutoffs(ctx, p.zt, p.t_seq, p.t_row, p.Kmax + 1, 1, p.draft_len, nullptr, ctx->cut_t, stream)) return rc;
+    return launch_cutoffs(ctx, p.zd, p.d_seq, p.d_row, p.Kmax, 0, p.draft_len, nullptr, ctx->cut_d, stream);
+}
+
 template <int MODE>
 int launch_verify(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
     const long long positions = (long long)p.B * (p.Kmax + 1);
     const int cs = pick_cluster(ctx, positions);
     const bool vec = vec_ok(p.zd, ctx->cfg.dtype, {p.d_seq, p.d_row}) &&
                      vec_ok(p.zt, ctx->cfg.dtype, {p.t_seq, p.t_row});
-    if (ctx->cuts_on()) {
-        if (int rc = launch_cutoffs(ctx, p.zt, p.t_seq, p.t_row, p.Kmax + 1, 1, p.draft_len, nullptr, ctx->cut_t, stream))
-            return rc;
-        if (int rc = launch_cutoffs(ctx, p.zd, p.d_seq, p.d_row, p.Kmax, 0, p.draft_len, nullptr, ctx->cut_d, stream))
-            return rc;
-    }
-    if (vec && ctx->fast[MODE].iter > 0) {
-        // Vanilla mode with enough rows to fill the GPU: log-sum-exps of all rows in one light
-        // streaming pass, the accept test per sequence, then the sampling of one position per
-        // sequence.  With fewer rows than CTA slots of the streaming pass: everything in the one
-        // cluster kernel.
-        const long long rows = (long long)p.B * (2 * p.Kmax + 1);
-        if (MODE == MODE_VANILLA && ctx->lse_stream && ctx->sample_stream && rows >= 2LL * ctx->sm_count) {
-            LseParams lp;
-            memset(&lp, 0, sizeof(lp));
-            lp.zd = p.zd;
-            lp.zt = p.zt;
-            lp.d_seq = p.d_seq;
-            lp.d_row = p.d_row;
-            lp.t_seq = p.t_seq;
-            lp.t_row = p.t_row;
-            lp.draft_len = p.draft_len;
-            lp.lse_d = p.sc.lse_d;
-            lp.lse_t = p.sc.lse_t;
-            lp.status = p.st.status;
-            lp.B = p.B;
-            lp.V = p.V;
-            lp.Kmax = p.Kmax;
-            lp.c1 = p.c1;
-            lp.cut_t = p.cut_t;
-            lp.cut_d = p.cut_d;
-            if (ctx->warp_on()) row_lse_kernel<true><<<2 * ctx->sm_count, kLW * 32, kLW * 2 * kLChunkBytes, stream>>>(lp);
-            else row_lse_kernel<false><<<2 * ctx->sm_count, kLW * 32, kLW * 2 * kLChunkBytes, stream>>>(lp);
-            CUDA_TRY(cudaGetLastError());
-            vanilla_accept_kernel<<<(p.B + 3) / 4, 128, 0, stream>>>(p, p.sc.only_pos);     // one warp per sequence
-            CUDA_TRY(cudaGetLastError());
-            // one CTA per sequence streams the row pair of its one position
-            vanilla_sample_kernel<<<p.B, kVW * 32, kVW * 4 * kVChunkBytes, stream>>>(p, p.sc.only_pos);
-            CUDA_TRY(cudaGetLastError());
-            return ADASD_OK;
-        }
+    if (int rc = launch_round_cutoffs(ctx, p, stream)) return rc;
+    if (vec && ctx->fast.iter > 0) {
         return fast_launch_iter<MODE>(ctx, p, stream);
     }
     if (ctx->cfg.dtype == ADASD_BF16) {
@@ -468,7 +489,7 @@ int launch_verify(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
                : launch_cluster(verify_kernel<float, false, MODE>, p, positions, cs, stream);
 }
 
-// The most probable token of every needed row (greedy drafting and greedy verification).
+// The most probable token of every active draft row (greedy drafting).
 int launch_argmax(adasd_ctx* ctx, const ArgmaxParams& a, cudaStream_t stream) {
     const long long rows = (long long)a.B * a.R;
     const unsigned grid = (unsigned)std::min<long long>(rows, 4LL * ctx->sm_count);
@@ -605,21 +626,26 @@ int adasd_create(adasd_ctx** out, const adasd_config* cfg) {
     ALLOC(t.dist, B * K);
     ALLOC(t.p_acc, B * K);
     ALLOC(t.y, B * (K + 1));
-    ALLOC(t.van_flag, B * K);
-    ALLOC(t.van_tok, B * (K + 1));
     ALLOC(t.ticket, B);
-    ALLOC(t.only_pos, B);
     ALLOC(t.q_items, B);
     ALLOC(t.q_ctl, 4);
     ALLOC(c->cut_t, B * (K + 1));
     ALLOC(c->cut_d, B * K);
     ALLOC(c->cut_row, B);
+    ALLOC(c->stream_next, 1);
+    stream_setup(c);
+    ALLOC(c->seg, (B * (2 * K + 1)) << c->seg_bits);
 #undef ALLOC
     c->temperature = 1.f;
     c->top_k = 0;
     c->top_p = 1.f;
     if (rc == ADASD_OK && cudaMemset(t.q_items, 0xFF, B * sizeof(int32_t)) != cudaSuccess) rc = ADASD_ERR_CUDA;
     if (rc == ADASD_OK) fast_setup(c, prop.sharedMemPerBlockOptin);
+    if (rc == ADASD_OK) {
+        const cudaError_t e1 = cfg->dtype == ADASD_BF16 ? stream_prepare<__nv_bfloat16, true>(c->stream_it) : stream_prepare<float, true>(c->stream_it);
+        const cudaError_t e2 = cfg->dtype == ADASD_BF16 ? stream_prepare<__nv_bfloat16, false>(c->stream_it) : stream_prepare<float, false>(c->stream_it);
+        if (e1 != cudaSuccess || e2 != cudaSuccess) rc = ADASD_ERR_CUDA;
+    }
     if (rc == ADASD_OK && cudaDeviceSynchronize() != cudaSuccess) rc = ADASD_ERR_CUDA;
     if (rc != ADASD_OK) {
         for (void* q : c->allocs) cudaFree(q);
@@ -827,7 +853,44 @@ int adasd_vanilla_verify(adasd_ctx* ctx, const void* draft_logits_dev,
     p.accept_len = accept_len_dev;
     p.next_token = next_token_dev;
     p.alpha_out = alpha_out_dev;
-    return launch_verify<MODE_VANILLA>(ctx, p, (cudaStream_t)stream);
+    cudaStream_t st = (cudaStream_t)stream;
+    const bool aligned = vec_ok(p.zd, ctx->cfg.dtype, {p.d_seq, p.d_row}) && vec_ok(p.zt, ctx->cfg.dtype, {p.t_seq, p.t_row});
+    if ((rc = launch_round_cutoffs(ctx, p, st))) return rc;
+    StreamParams sp;
+    memset(&sp, 0, sizeof(sp));
+    sp.zd = p.zd;
+    sp.zt = p.zt;
+    sp.d_seq = p.d_seq;
+    sp.d_row = p.d_row;
+    sp.t_seq = p.t_seq;
+    sp.t_row = p.t_row;
+    sp.draft_len = p.draft_len;
+    sp.seg = ctx->seg;
+    sp.status = ctx->st.status;
+    sp.next = ctx->stream_next;
+    sp.B = p.B;
+    sp.V = p.V;
+    sp.Kmax = p.Kmax;
+    sp.seg_bits = ctx->seg_bits;
+    sp.c1 = p.c1;
+    sp.cut_t = p.cut_t;
+    sp.cut_d = p.cut_d;
+    if ((rc = launch_stream(ctx, sp, OP_LSE, aligned, st))) return rc;
+    VanillaParams vp;
+    vp.v = p;
+    vp.seg = ctx->seg;
+    vp.next = ctx->stream_next;
+    vp.seg_bits = ctx->seg_bits;
+    // CTAs per sequence: until the SMs carry two each, as long as a warp keeps an iteration or two
+    const int NI = (ctx->cfg.V / (ctx->cfg.dtype == ADASD_BF16 ? 8 : 4) + 31) / 32;
+    int S = 1;
+    while (S < kVMaxS && (long long)p.B * S * 2 <= 4LL * ctx->sm_count && NI >= 2 * S * kVWarps) S *= 2;
+    const int grid = p.B * S;
+    if (ctx->cfg.dtype == ADASD_BF16)
+        return aligned ? launch_pdl(vanilla_finish_kernel<__nv_bfloat16, true>, grid, kVThreads, 0, S, st, vp)
+                       : launch_pdl(vanilla_finish_kernel<__nv_bfloat16, false>, grid, kVThreads, 0, S, st, vp);
+    return aligned ? launch_pdl(vanilla_finish_kernel<float, true>, grid, kVThreads, 0, S, st, vp)
+                   : launch_pdl(vanilla_finish_kernel<float, false>, grid, kVThreads, 0, S, st, vp);
 }
 
 int adasd_greedy_verify(adasd_ctx* ctx, const void* target_logits_dev, int64_t t_seq_stride,
@@ -843,22 +906,34 @@ int adasd_greedy_verify(adasd_ctx* ctx, const void* target_logits_dev, int64_t t
     if (int rc = check_strides(ctx, t_seq_stride, t_row_stride)) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     const int B = ctx->cfg.B, K = ctx->cfg.Kmax;
-    ArgmaxParams a;
-    memset(&a, 0, sizeof(a));
-    a.z = target_logits_dev;
-    a.seq_stride = t_seq_stride;
-    a.row_stride = t_row_stride;
-    a.draft_len = draft_len_dev;
-    a.out = ctx->sc.van_tok;                 // [B, Kmax + 1] scratch of the comparison modes
-    a.status = ctx->st.status;
-    a.B = B;
-    a.R = K + 1;
-    a.V = ctx->cfg.V;
-    if (int rc = launch_argmax(ctx, a, st)) return rc;
-    greedy_accept_kernel<<<(B + 127) / 128, 128, 0, st>>>(draft_tokens_dev, ctx->sc.van_tok, draft_len_dev,
-                                                        accept_len_dev, next_token_dev, argmax_out_dev, B, K);
-    CUDA_TRY(cudaGetLastError());
-    return ADASD_OK;
+    StreamParams sp;
+    memset(&sp, 0, sizeof(sp));
+    sp.zt = target_logits_dev;
+    sp.t_seq = t_seq_stride;
+    sp.t_row = t_row_stride;
+    sp.draft_len = draft_len_dev;
+    sp.seg = ctx->seg;
+    sp.status = ctx->st.status;
+    sp.next = ctx->stream_next;
+    sp.B = B;
+    sp.V = ctx->cfg.V;
+    sp.Kmax = K;
+    sp.seg_bits = ctx->seg_bits;
+    sp.c1 = kLog2e;
+    const bool aligned = vec_ok(target_logits_dev, ctx->cfg.dtype, {t_seq_stride, t_row_stride});
+    if (int rc = launch_stream(ctx, sp, OP_ARGMAX, aligned, st)) return rc;
+    GreedyParams g;
+    g.seg = ctx->seg;
+    g.x = draft_tokens_dev;
+    g.draft_len = draft_len_dev;
+    g.accept_len = accept_len_dev;
+    g.next_token = next_token_dev;
+    g.argmax_out = argmax_out_dev;
+    g.status = ctx->st.status;
+    g.next = ctx->stream_next;
+    g.Kmax = K;
+    g.seg_bits = ctx->seg_bits;
+    return launch_pdl(greedy_finish_kernel, B, kGThreads, 0, 1, st, g);
 }
 
 int adasd_gen_only_update(adasd_ctx* ctx, const float* H_draft_dev, const int32_t* draft_len_dev,

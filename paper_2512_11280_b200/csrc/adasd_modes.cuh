@@ -1,12 +1,9 @@
 // Greedy decoding (Sec. 2.1.3) and the Gen-Only ablation variant (Sec. 5).
 //
-//  * row_argmax_kernel: the most probable token of every needed logit row, x = argmax_v z_v
+//  * row_argmax_kernel: the most probable token of every active draft row, x = argmax_v z_v
 //    (Sec. 2.1.1, deterministic selection), the lowest index among equal maxima.  One CTA per
 //    row at a time, rows dealt round robin to a grid that fills the SMs; any V, dtype and
 //    stride (16-byte loads where the row allows them).
-//  * greedy_accept_kernel: candidate x_i is accepted only if it equals argmax p_i; the scan
-//    stops at the first mismatch and the token after the accepted prefix is the target's own
-//    choice there (the bonus row's after a full match).
 //  * gen_only_update_kernel: the feedback of the generation component alone: the entropy of
 //    the candidate that vanilla verification rejected joins L_E^R, T_G = mean(L_E^R).
 #pragma once
@@ -93,28 +90,6 @@ __global__ void __launch_bounds__(kAThreads) row_argmax_kernel(ArgmaxParams p) {
         }
         __syncthreads();
     }
-}
-
-// One thread per sequence: longest prefix of candidates that equal the target's choice.
-__global__ void greedy_accept_kernel(const int32_t* __restrict__ x, const int32_t* __restrict__ am,
-                                     const int32_t* __restrict__ draft_len, int32_t* accept_len,
-                                     int32_t* next_token, int32_t* argmax_user, int B, int Kmax) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= B) return;
-    const int K1 = Kmax + 1;
-    int kt = draft_len ? draft_len[b] : Kmax;
-    kt = max(0, min(kt, Kmax));
-    int w = kt;
-    for (int i = 0; i < kt; ++i) {
-        if (x[(size_t)b * Kmax + i] != am[(size_t)b * K1 + i]) {
-            w = i;
-            break;
-        }
-    }
-    accept_len[b] = w;
-    next_token[b] = am[(size_t)b * K1 + w];
-    if (argmax_user)
-        for (int i = 0; i <= kt; ++i) argmax_user[(size_t)b * K1 + i] = am[(size_t)b * K1 + i];
 }
 
 // One thread per sequence: L_E^R += H(q) of the candidate vanilla verification rejected.

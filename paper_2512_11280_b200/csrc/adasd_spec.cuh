@@ -44,7 +44,7 @@
 // through the rest of the protocol, so the kernel always ends.
 #pragma once
 
-#include "adasd_cluster.cuh"
+#include "adasd_async.cuh"
 
 namespace adasd {
 
@@ -115,24 +115,6 @@ struct __align__(16) SpecShared {
     float td[3][ADASD_KMAX_LIMIT], tH[3][ADASD_KMAX_LIMIT];   // scratch of the three tail workers of a CTA
 };
 
-// ---- mbarrier helpers with explicit scopes -----------------------------------------------
-__device__ __forceinline__ void mbar_arrive_cta(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-// shared::cluster address of `p` (an address in this CTA's shared memory) as seen in CTA `cta`
-__device__ __forceinline__ uint32_t mapa_u32(const void* p, uint32_t cta) {
-    uint32_t r;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(cta));
-    return r;
-}
-// 16 bytes into another CTA's shared memory; their arrival is counted (complete_tx) on a
-// barrier of THAT CTA, so the receiver needs no fence and the sender no second message
-__device__ __forceinline__ void st_async_v4(uint32_t remote_addr, float4 v, uint32_t remote_bar) {
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];"
-                 ::"r"(remote_addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(remote_bar)
-                 : "memory");
-}
-
 __device__ __forceinline__ void st_cluster_u32(uint32_t remote_addr, uint32_t v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote_addr), "r"(v) : "memory");
 }
@@ -144,15 +126,6 @@ __device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t remote_addr) {
 __device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 
 // ---- tensor memory as a scratchpad ---------------------------------------------------------
-// Allocation and release are warp-wide; the address lands in shared memory.
-__device__ __forceinline__ void tmem_alloc(uint32_t* smem_dst, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_dst)), "r"(ncols)
-                 : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
-}
 // 16 consecutive columns of this thread's lane: a[0..7] then b[0..7]
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const float (&a)[8], const float (&b)[8]) {
     asm volatile(
@@ -166,7 +139,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&a)[8]) {
                  ::"r"(taddr), "f"(a[0]), "f"(a[1]), "f"(a[2]), "f"(a[3]), "f"(a[4]), "f"(a[5]), "f"(a[6]), "f"(a[7])
                  : "memory");
 }
-__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // The loads are asynchronous: the registers hold the values only after tmem_wait_ld, which
 // takes them as operands so that nothing that uses them can be scheduled ahead of the wait.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&a)[8], float (&b)[8]) {
@@ -183,30 +155,12 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&a)[8]) {
                  : "r"(taddr)
                  : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld(float (&a)[8], float (&b)[8]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]),
-                   "+f"(b[0]), "+f"(b[1]), "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7])
-                 :
-                 : "memory");
-}
 __device__ __forceinline__ void tmem_wait_ld(float (&a)[8]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7])
                  :
                  : "memory");
 }
-__device__ __forceinline__ float rcp_approx(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ double warp_sum_f64(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    return v;
-}
-
 // The published scalars of one position from the CTAs' statistics (lane c holds CTA c) and the
 // warps' pass-C sums, worked out in float64 by the whole tail warp.  In fp32 the totals
 // (entropies of up to 17 bits, log2 of sums of up to 2^17) carry errors of about 1e-6 each, which
