@@ -14,7 +14,7 @@
 #include "adasd_rows.cuh"
 #include "adasd_cluster.cuh"
 #include "adasd_spec.cuh"
-#include "adasd_draft.cuh"
+#include "adasd_draft_stream.cuh"
 #include "adasd_stream.cuh"
 #include "adasd_modes.cuh"
 
@@ -33,7 +33,8 @@ struct adasd_ctx {
         int smem;             // dynamic shared memory per CTA
         ClusterGeom geom;
     } fast;
-    bool draft_stream;        // the streaming draft kernel is usable for this V / dtype
+    int draft_p, draft_nw, draft_it;      // draft step: CTAs per row, warps per CTA, iterations of a chunk
+    bool draft_early;         // ... the next call's CTAs may be set up while one runs
     bool cut_hist;            // the one-pass cutoff kernel got its 128 KB of shared memory
     // adjusted distribution (adasd_set_warpers) and the per-row cutoffs a call works out
     float temperature;
@@ -235,26 +236,9 @@ void fast_setup_mode(adasd_ctx* c, size_t smem_optin) {
 }
 void fast_setup(adasd_ctx* c, size_t smem_optin) {
     fast_setup_mode<MODE_ADASD>(c, smem_optin);
-    // streaming draft kernel: bf16 rows of a multiple of 8 logits, two 4 KB buffers per warp
-    c->draft_stream = false;
     c->cut_hist = cudaFuncSetAttribute(row_cutoff_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kHistWords * 4) == cudaSuccess;
     if (!c->cut_hist) cudaGetLastError();
-    const int V = c->cfg.V;
-    if (c->cfg.dtype == ADASD_BF16 && (V & 7) == 0 && V >= 8192 &&
-        (V >> 3) <= kDMaxP * kDW * kDMaxChunks * kDChunkUnits) {
-        if (cudaFuncSetAttribute(draft_stream_kernel<kDW, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kDW * 2 * kDChunkBytes) == cudaSuccess &&
-            cudaFuncSetAttribute(draft_stream_kernel<kDWBig, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kDWBig * 2 * kDChunkBytes) == cudaSuccess &&
-            cudaFuncSetAttribute(draft_stream_kernel<kDW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kDW * 2 * kDChunkBytes) == cudaSuccess &&
-            cudaFuncSetAttribute(draft_stream_kernel<kDWBig, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kDWBig * 2 * kDChunkBytes) == cudaSuccess)
-            c->draft_stream = true;
-        else
-            cudaGetLastError();
-    }
 }
 
 // Chunk length and segments of a row in the vanilla and greedy modes.  Chunks of 8 iterations (4 KB)
@@ -287,7 +271,8 @@ template <typename T, bool ALIGNED>
 cudaError_t stream_prepare(int it) { return it == 8 ? stream_prepare_it<T, ALIGNED, 8>() : stream_prepare_it<T, ALIGNED, 2>(); }
 
 // Launch with programmatic stream serialisation: the kernel may become resident while the one ahead of
-// it is still running (it waits before it reads what that one wrote).
+// it is still running (it waits before it reads what that one wrote).  cs: CTAs per cluster; 0: the kernel
+// uses no cluster.  (A kernel that uses cluster-scope instructions gets the attribute even for clusters of one.)
 template <typename K, typename... Args>
 int launch_pdl(K kernel, int grid, int threads, int smem, int cs, cudaStream_t stream, const Args&... args) {
     cudaLaunchConfig_t lc;
@@ -304,7 +289,7 @@ int launch_pdl(K kernel, int grid, int threads, int smem, int cs, cudaStream_t s
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 1;
     lc.attrs = attr;
-    lc.numAttrs = cs > 1 ? 2 : 1;
+    lc.numAttrs = cs > 0 ? 2 : 1;
     CUDA_TRY(cudaLaunchKernelEx(&lc, kernel, args...));
     return ADASD_OK;
 }
@@ -313,9 +298,9 @@ template <typename T, bool ALIGNED, int IT>
 int launch_stream_it(adasd_ctx* c, const StreamParams& p, int op, cudaStream_t stream) {
     const long long rows = (long long)p.B * (p.zd ? 2 * p.Kmax + 1 : p.Kmax + 1);
     const int grid = (int)std::min<long long>(((rows << p.seg_bits) + kRW - 1) / kRW, 2LL * c->sm_count);
-    if (op == OP_ARGMAX) return launch_pdl(row_stream_kernel<T, ALIGNED, OP_ARGMAX, false, IT>, grid, kRThreads, kRSmem, 1, stream, p);
-    return c->warp_on() ? launch_pdl(row_stream_kernel<T, ALIGNED, OP_LSE, true, IT>, grid, kRThreads, kRSmem, 1, stream, p)
-                        : launch_pdl(row_stream_kernel<T, ALIGNED, OP_LSE, false, IT>, grid, kRThreads, kRSmem, 1, stream, p);
+    if (op == OP_ARGMAX) return launch_pdl(row_stream_kernel<T, ALIGNED, OP_ARGMAX, false, IT>, grid, kRThreads, kRSmem, 0, stream, p);
+    return c->warp_on() ? launch_pdl(row_stream_kernel<T, ALIGNED, OP_LSE, true, IT>, grid, kRThreads, kRSmem, 0, stream, p)
+                        : launch_pdl(row_stream_kernel<T, ALIGNED, OP_LSE, false, IT>, grid, kRThreads, kRSmem, 0, stream, p);
 }
 template <typename T, bool ALIGNED>
 int launch_stream(adasd_ctx* c, const StreamParams& p, int op, cudaStream_t stream) {
@@ -327,18 +312,69 @@ int launch_stream(adasd_ctx* c, const StreamParams& p, int op, bool aligned, cud
     return aligned ? launch_stream<float, true>(c, p, op, stream) : launch_stream<float, false>(c, p, op, stream);
 }
 
-// CTAs per row for the streaming draft kernel: enough to fill the SMs, and few enough chunks
-// per warp for its tables
-int draft_stream_p(const adasd_ctx* c) {
-    const int NU = c->cfg.V >> 3;
+// ---- draft step: configuration and launch -----------------------------------------------------
+// CTAs per row until they cover three quarters of the SMs.  16 warps per CTA, one CTA per SM, where that
+// takes all of a call's CTAs at once (clusters of 4: 33 fit, of 8: 15); else 8 warps and two CTAs per SM.
+void draft_setup(adasd_ctx* c) {
     int P = 1;
-    if (c->cfg.cluster_size == 1 || c->cfg.cluster_size == 2 || c->cfg.cluster_size == 4 ||
-        c->cfg.cluster_size == 8)
+    if (c->cfg.cluster_size == 1 || c->cfg.cluster_size == 2 || c->cfg.cluster_size == 4 || c->cfg.cluster_size == 8)
         P = c->cfg.cluster_size;
     else
         while (P < kDMaxP && (long long)c->cfg.B * P * 4 < 3LL * c->sm_count) P *= 2;
-    while (P < kDMaxP && (NU + P * kDW - 1) / (P * kDW) > kDMaxChunks * kDChunkUnits) P *= 2;
-    return P;
+    c->draft_p = P;
+    const long long grid = (long long)c->cfg.B * P;
+    c->draft_nw = P <= 4 && grid <= (P == 4 ? 132 : c->sm_count) ? kDWBig : kDW;
+    // dependents early: where the SMs hold two CTAs and a call needs at most half of them, or where they hold one
+    c->draft_early = c->draft_nw == kDWBig || grid * 2 <= c->sm_count;
+    const int N = c->cfg.dtype == ADASD_BF16 ? 8 : 4, NI = ((c->cfg.V + N - 1) / N + 31) / 32;
+    c->draft_it = NI >= 16 * P * c->draft_nw ? 8 : 4;
+}
+// Large batches of aligned bf16 rows: the kernel whose warps split a row to 16 bytes.
+bool draft_rows(const adasd_ctx* c) {
+    return c->cfg.dtype == ADASD_BF16 && (c->cfg.V & 7) == 0 && c->cfg.V >= 8192 && c->draft_p <= 2 &&
+           c->cfg.V <= kDMaxChunks * kDChunkUnits * 8 * c->draft_p * c->draft_nw;
+}
+template <int NW>
+cudaError_t draft_rows_prepare() {
+    cudaError_t e = cudaFuncSetAttribute(draft_stream_kernel<NW, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, NW * 2 * kDChunkBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(draft_stream_kernel<NW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, NW * 2 * kDChunkBytes);
+    return e;
+}
+template <int NW>
+int launch_draft_rows(adasd_ctx* c, const DraftParams& p, cudaStream_t stream) {
+    const int grid = p.B * c->draft_p, smem = NW * 2 * kDChunkBytes;
+    return c->warp_on() ? launch_pdl(draft_stream_kernel<NW, true>, grid, NW * 32, smem, c->draft_p, stream, p)
+                        : launch_pdl(draft_stream_kernel<NW, false>, grid, NW * 32, smem, c->draft_p, stream, p);
+}
+
+template <typename T, bool ALIGNED, int NW, int IT>
+cudaError_t draft_prepare_it() {
+    cudaError_t e = cudaFuncSetAttribute(draft_step_kernel<T, ALIGNED, NW, IT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, NW * kDRingB);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(draft_step_kernel<T, ALIGNED, NW, IT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, NW * kDRingB);
+    return e;
+}
+template <typename T, bool ALIGNED>
+cudaError_t draft_prepare(const adasd_ctx* c) {
+    if (c->draft_nw == kDW) return c->draft_it == 8 ? draft_prepare_it<T, ALIGNED, kDW, 8>() : draft_prepare_it<T, ALIGNED, kDW, 4>();
+    return c->draft_it == 8 ? draft_prepare_it<T, ALIGNED, kDWBig, 8>() : draft_prepare_it<T, ALIGNED, kDWBig, 4>();
+}
+template <typename T, bool ALIGNED, int NW, int IT>
+int launch_draft_it(adasd_ctx* c, const DraftParams& p, cudaStream_t stream) {
+    const int grid = p.B * c->draft_p;
+    return c->warp_on() ? launch_pdl(draft_step_kernel<T, ALIGNED, NW, IT, true>, grid, NW * 32, NW * kDRingB, c->draft_p, stream, p)
+                        : launch_pdl(draft_step_kernel<T, ALIGNED, NW, IT, false>, grid, NW * 32, NW * kDRingB, c->draft_p, stream, p);
+}
+template <typename T, bool ALIGNED>
+int launch_draft(adasd_ctx* c, const DraftParams& p, cudaStream_t stream) {
+    if (c->draft_nw == kDW)
+        return c->draft_it == 8 ? launch_draft_it<T, ALIGNED, kDW, 8>(c, p, stream) : launch_draft_it<T, ALIGNED, kDW, 4>(c, p, stream);
+    return c->draft_it == 8 ? launch_draft_it<T, ALIGNED, kDWBig, 8>(c, p, stream) : launch_draft_it<T, ALIGNED, kDWBig, 4>(c, p, stream);
+}
+template <typename T>
+int launch_draft(adasd_ctx* c, const DraftParams& p, bool aligned, cudaStream_t stream) {
+    return aligned ? launch_draft<T, true>(c, p, stream) : launch_draft<T, false>(c, p, stream);
 }
 
 template <int ITER, int MODE, bool WARPED>
@@ -489,22 +525,6 @@ int launch_verify(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
                : launch_cluster(verify_kernel<float, false, MODE>, p, positions, cs, stream);
 }
 
-// The most probable token of every active draft row (greedy drafting).
-int launch_argmax(adasd_ctx* ctx, const ArgmaxParams& a, cudaStream_t stream) {
-    const long long rows = (long long)a.B * a.R;
-    const unsigned grid = (unsigned)std::min<long long>(rows, 4LL * ctx->sm_count);
-    const bool vec = vec_ok(a.z, ctx->cfg.dtype, {a.seq_stride, a.row_stride});
-    if (ctx->cfg.dtype == ADASD_BF16) {
-        if (vec) row_argmax_kernel<__nv_bfloat16, true><<<grid, kAThreads, 0, stream>>>(a);
-        else row_argmax_kernel<__nv_bfloat16, false><<<grid, kAThreads, 0, stream>>>(a);
-    } else {
-        if (vec) row_argmax_kernel<float, true><<<grid, kAThreads, 0, stream>>>(a);
-        else row_argmax_kernel<float, false><<<grid, kAThreads, 0, stream>>>(a);
-    }
-    CUDA_TRY(cudaGetLastError());
-    return ADASD_OK;
-}
-
 struct DeviceGuard {
     int prev = -1;
     bool ok = false;
@@ -644,7 +664,11 @@ int adasd_create(adasd_ctx** out, const adasd_config* cfg) {
     if (rc == ADASD_OK) {
         const cudaError_t e1 = cfg->dtype == ADASD_BF16 ? stream_prepare<__nv_bfloat16, true>(c->stream_it) : stream_prepare<float, true>(c->stream_it);
         const cudaError_t e2 = cfg->dtype == ADASD_BF16 ? stream_prepare<__nv_bfloat16, false>(c->stream_it) : stream_prepare<float, false>(c->stream_it);
-        if (e1 != cudaSuccess || e2 != cudaSuccess) rc = ADASD_ERR_CUDA;
+        draft_setup(c);
+        const cudaError_t e3 = cfg->dtype == ADASD_BF16 ? draft_prepare<__nv_bfloat16, true>(c) : draft_prepare<float, true>(c);
+        const cudaError_t e4 = cfg->dtype == ADASD_BF16 ? draft_prepare<__nv_bfloat16, false>(c) : draft_prepare<float, false>(c);
+        const cudaError_t e5 = c->draft_nw == kDW ? draft_rows_prepare<kDW>() : draft_rows_prepare<kDWBig>();
+        if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess || e5 != cudaSuccess) rc = ADASD_ERR_CUDA;
     }
     if (rc == ADASD_OK && cudaDeviceSynchronize() != cudaSuccess) rc = ADASD_ERR_CUDA;
     if (rc != ADASD_OK) {
@@ -700,78 +724,29 @@ static int draft_entropy_impl(adasd_ctx* ctx, const void* logits_dev, int64_t ro
     p.active = active_inout_dev;
     p.H_out = H_out_dev;
     p.lse_out = lse_out_dev;
-    p.token_out = u_dev ? token_out_dev : nullptr;
+    p.token_out = token_out_dev;
+    p.argmax = (!u_dev && token_out_dev) ? 1 : 0;
+    p.early = ctx->draft_early ? 1 : 0;
     p.stop_out = stop_out_dev;
     p.draft_len = draft_len_inout_dev;
     p.st = ctx->st;
     p.B = ctx->cfg.B;
     p.V = ctx->cfg.V;
     p.expire_row = expire_row;
-    p.inv_temp = 1.f / ctx->temperature;
     p.c1 = kLog2e / ctx->temperature;
     if (ctx->cuts_on()) p.cut = ctx->cut_row;
-    const int cs = pick_cluster(ctx, p.B);
-    const bool vec = vec_ok(logits_dev, ctx->cfg.dtype, {row_stride});
-    if (expire_row >= 0 && !(vec && ctx->draft_stream && expire_row < ctx->cfg.B))
-        return ADASD_ERR_SHAPE;                  // the self-test needs the streaming kernel
+    const bool aligned = vec_ok(logits_dev, ctx->cfg.dtype, {row_stride});
+    // (the self-test is kept to the rows its header names)
+    if (expire_row >= 0 && !(aligned && ctx->cfg.dtype == ADASD_BF16 && (p.V & 7) == 0 && p.V >= 8192 && expire_row < p.B))
+        return ADASD_ERR_SHAPE;
     cudaStream_t st = (cudaStream_t)stream;
-    if (!u_dev && token_out_dev) {
-        // greedy drafting: the most probable token of every active row, before the step below can
-        // clear a row's entry in the active mask (the token that trips the stop check stays)
-        ArgmaxParams a;
-        memset(&a, 0, sizeof(a));
-        a.z = logits_dev;
-        a.seq_stride = row_stride;
-        a.row_stride = 0;
-        a.active = active_inout_dev;
-        a.out = token_out_dev;
-        a.status = ctx->st.status;
-        a.B = ctx->cfg.B;
-        a.R = 1;
-        a.V = ctx->cfg.V;
-        if (int rc = launch_argmax(ctx, a, st)) return rc;
-    }
     if (ctx->cuts_on()) {
         if (int rc = launch_cutoffs(ctx, logits_dev, row_stride, 0, 1, 1, nullptr, active_inout_dev, ctx->cut_row, st))
             return rc;
     }
-    if (vec && ctx->draft_stream) {
-        const int P = draft_stream_p(ctx);
-        // a grid of at most one CTA per SM runs 16 warps per CTA, a larger one 8 (two CTAs per SM)
-        const bool big = (long long)p.B * P <= ctx->sm_count && P * kDWBig <= kDMaxEntries;
-        const int W = big ? kDWBig : kDW;
-        cudaLaunchConfig_t lc;
-        memset(&lc, 0, sizeof(lc));
-        lc.gridDim = dim3((unsigned)(p.B * P), 1, 1);
-        lc.blockDim = dim3((unsigned)(W * 32), 1, 1);
-        lc.dynamicSmemBytes = (size_t)(W * 2 * kDChunkBytes);
-        lc.stream = st;
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)P;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        // the launch may overlap the tail of the kernel ahead of it (the kernel waits before it
-        // reads anything): draft steps come in runs of short calls
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        lc.attrs = attr;
-        lc.numAttrs = 2;
-        const bool warped = ctx->warp_on();
-        if (big) {
-            if (warped) CUDA_TRY(cudaLaunchKernelEx(&lc, draft_stream_kernel<kDWBig, true>, p));
-            else CUDA_TRY(cudaLaunchKernelEx(&lc, draft_stream_kernel<kDWBig, false>, p));
-        } else {
-            if (warped) CUDA_TRY(cudaLaunchKernelEx(&lc, draft_stream_kernel<kDW, true>, p));
-            else CUDA_TRY(cudaLaunchKernelEx(&lc, draft_stream_kernel<kDW, false>, p));
-        }
-        return ADASD_OK;
-    }
-    if (ctx->cfg.dtype == ADASD_BF16)
-        return vec ? launch_cluster(draft_kernel<__nv_bfloat16, true>, p, p.B, cs, st)
-                   : launch_cluster(draft_kernel<__nv_bfloat16, false>, p, p.B, cs, st);
-    return vec ? launch_cluster(draft_kernel<float, true>, p, p.B, cs, st)
-               : launch_cluster(draft_kernel<float, false>, p, p.B, cs, st);
+    if (aligned && !p.argmax && draft_rows(ctx))
+        return ctx->draft_nw == kDW ? launch_draft_rows<kDW>(ctx, p, st) : launch_draft_rows<kDWBig>(ctx, p, st);
+    return ctx->cfg.dtype == ADASD_BF16 ? launch_draft<__nv_bfloat16>(ctx, p, aligned, st) : launch_draft<float>(ctx, p, aligned, st);
 }
 
 int adasd_draft_entropy(adasd_ctx* ctx, const void* logits_dev, int64_t row_stride,
@@ -933,7 +908,7 @@ int adasd_greedy_verify(adasd_ctx* ctx, const void* target_logits_dev, int64_t t
     g.next = ctx->stream_next;
     g.Kmax = K;
     g.seg_bits = ctx->seg_bits;
-    return launch_pdl(greedy_finish_kernel, B, kGThreads, 0, 1, st, g);
+    return launch_pdl(greedy_finish_kernel, B, kGThreads, 0, 0, st, g);
 }
 
 int adasd_gen_only_update(adasd_ctx* ctx, const float* H_draft_dev, const int32_t* draft_len_dev,

@@ -85,6 +85,14 @@ __device__ __forceinline__ void tmem_wait_ld(float (&a)[4], float (&b)[4]) {
                  : "memory");
 }
 
+// {x, x} as an operand of packed arithmetic, kept in its register pair: a pair the compiler can see through
+// is made again at its uses, up to two moves for each packed instruction.
+__device__ __forceinline__ float2 pair2(float x) {
+    float2 r = make_float2(x, x);
+    asm volatile("" : "+f"(r.x), "+f"(r.y));
+    return r;
+}
+
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

@@ -1,44 +1,57 @@
-// Streaming draft-step kernel for sm_100a (adasd_draft_entropy on bf16 rows of a multiple of 8
-// logits): every row is read from HBM once.
+// Draft-step kernel for sm_100a (adasd_draft_entropy): bf16 or fp32 rows of any length, alignment and
+// stride, every row read from HBM once.
 //
-//  * One cluster of P CTAs per row (P = 1, 2, 4 or 8, chosen so that the launch fills the SMs);
-//    the 8 warps of a CTA split the CTA's part of the row into contiguous shares and stream
-//    them through two 4 KB buffers each (1-D bulk copies, bounded mbarrier waits).
-//  * Per chunk: packed bf16 maximum, then 2^(z log2 e - M) with the warp's running shift M
-//    (raised, with the sums rescaled, only when a chunk exceeds it), accumulating S = sum 2^t
-//    and T = sum 2^t t.  The chunk's own sum is kept in a small table for sampling.
-//  * The CTAs send their totals and tables to rank 0 over DSMEM; after ONE cluster barrier
-//    rank 0 forms H(q) = ln 2 (log2 S - T / S), the log-sum-exp and the stop flag H > T_G,
-//    finds the chunk that holds the inverse-CDF crossing of u and rescans just that chunk
-//    (4 KB, from L2) for the token x ~ q.
+//  * One cluster of P CTAs per row (P = 1, 2, 4 or 8, chosen so that the launch fills the SMs); the
+//    warps of the cluster split the row into contiguous shares and stream them through a ring of
+//    three 2 KB bulk copies each (bounded mbarrier waits).
+//  * Per chunk: packed maximum, then 2^((z - max) log2 e) with the warp's running maximum (the sums
+//    are rescaled when a chunk raises it), accumulating S = sum 2^t and T = sum 2^t t.  Sums over
+//    short runs of chunks are kept in a table for sampling.  Greedy drafting: the index of the
+//    maximum is looked up when a chunk raises it.
+//  * The warps send their totals and tables to rank 0 over DSMEM; after one cluster barrier rank 0
+//    forms H(q) = ln 2 (log2 S - T / S), the log-sum-exp and the stop flag H > T_G, finds the run of
+//    chunks that holds the inverse-CDF crossing of u and scans just that again (from L2).
+//
+// What bounds it: a call is a few microseconds, of which the stream itself is about half; the rest is
+// start-up, the first copy's latency and the serial end on one warp.  So the copies are asked for before
+// the cluster's CTAs have met, what the end needs from global memory is asked for at the start, and a call
+// signals its dependents at once: the next call's CTAs are set up while this one runs, and wait before
+// they read anything.  Where the grid does not leave half of the SMs free, a second CTA per SM would put
+// two rows of the same call on one SM and none on another (31 instead of 13 us a call for 128 rows of
+// 151936 bf16 logits): draft_setup allows it only where it cannot.
 #pragma once
 
-#include "adasd_cluster.cuh"
+#include "adasd_async.cuh"
 
 namespace adasd {
 
-constexpr int kDW = 8;                         // warps per CTA when two CTAs share an SM
-constexpr int kDWBig = 16;                     // warps per CTA when the grid has one CTA per SM at most
-constexpr int kDChunkUnits = 256;              // 16-byte units per chunk: 8 iterations of a warp
-constexpr int kDChunkBytes = kDChunkUnits * 16;
-constexpr int kDMaxChunks = 12;                // chunks per warp, at most (V <= 8 * 8 * 12 * 2048)
+constexpr int kDW = 8;                         // warps per CTA
+constexpr int kDWBig = 16;                     // ... when the grid has one CTA per SM at most
+constexpr int kDRingB = 6 * (4 * 512 + 16);     // bytes of a warp's ring: six chunks of 4 iterations (32 lanes x 16 bytes;
+                                               // + one unit: rows off a 16-byte boundary) or three of 8
+constexpr int kDMaxRing = 6;
+constexpr int kDRuns = 8;                      // runs of chunks a warp's table holds
 constexpr int kDMaxP = 8;
+constexpr int kDMaxEntries = 64;               // warps per cluster, at most: two table entries per lane
 
-constexpr int kDMaxEntries = 64;               // warps per cluster (P * NW), at most: two table entries per lane
 template <int NW>
 struct __align__(16) DraftShared {
-    float cm[kDMaxEntries][kDMaxChunks];       // rank 0: shift in force when a chunk was summed, by (rank, warp)
-    float cs[kDMaxEntries][kDMaxChunks];       // rank 0: the chunk's sum of 2^t under that shift
-    float4 wpart[kDMaxEntries];                // rank 0: every warp's (M, S, T, flags)
-    unsigned long long bar[NW][2];
+    float2 run[kDMaxEntries][kDRuns];          // rank 0: (shift, sum of 2^t under it) of every run, by warp of the cluster
+    float4 wpart[kDMaxEntries];                // rank 0: every warp's (largest logit, S, T, flags)
+    int32_t widx[kDMaxEntries];                // rank 0: index of every warp's largest logit (greedy drafting)
+    unsigned long long bar[NW][kDMaxRing];
 };
 
-// NW warps per CTA: 8 (two CTAs per SM) or 16 (one CTA per SM, for grids that do not fill the
-// SMs twice); P * NW <= kDMaxEntries.
-// WARPED: an adjusted distribution is set (Sec. 2.1.1); the ordinary instantiation carries none of its code.
-template <int NW, bool WARPED = false>
-__global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_stream_kernel(DraftParams p) {
-    constexpr int kDW = NW;                    // (shadows the namespace constant: warps of THIS kernel)
+// NW warps per CTA: 8, or 16 (grids that do not fill the SMs twice); P * NW <= kDMaxEntries.
+// IT: iterations of a chunk, 4 or (long shares: half the reductions) 8.
+// ALIGNED: every row starts on a 16-byte boundary.  WARPED: an adjusted distribution is set
+// (Sec. 2.1.1); the ordinary instantiation carries none of its code.
+template <typename T, bool ALIGNED, int NW, int IT, bool WARPED>
+__global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(DraftParams p) {
+    using U = Unit<T>;
+    constexpr int N = U::N, NP = N / 2;
+    constexpr int kDRing = IT == 8 ? 3 : 6, kDStage = IT * 512 + 16;
+    const float floor_v = N == 8 ? ADASD_FLOOR_BF : kFloor;
     extern __shared__ __align__(128) unsigned char dyn_smem[];
     __shared__ DraftShared<NW> sh;
     cg::cluster_group cluster = cg::this_cluster();
@@ -46,293 +59,301 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_stream_kerne
     const int rank = (int)cluster.block_rank();
     const int b = blockIdx.x / P;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // Launched with programmatic stream serialisation: the CTAs may be resident before the
-    // kernel ahead in the stream has finished; nothing it wrote (the logits, the active mask, the
-    // window lengths) is touched before this wait, which returns once that kernel is complete.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const bool active = !(p.active && p.active[b] == 0);      // same in every CTA of the cluster
-    // what the last step of the row needs from global memory is asked for now, by the warp that
-    // will need it, so that it is there after the stream: the uniform and the threshold
+    if (lane == 0) {
+        for (int s = 0; s < kDRing; ++s) mbar_init(reinterpret_cast<uint64_t*>(&sh.bar[warp][s]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncwarp();
+    if (p.early) pdl_trigger();
+    // nothing the kernel ahead in the stream wrote (logits, active mask, window lengths) is touched before this
+    pdl_wait();
+    if (p.active && p.active[b] == 0) return;  // the same in every CTA of the cluster
+
+    // the row in chunks of IT iterations (32 units of N elements each); this warp's share: whole chunks
+    // [ch0, ch1), so that only the row's last chunk is ragged
+    const int NU = (p.V + N - 1) / N, NC = (NU + 32 * IT - 1) / (32 * IT);
+    const int G = P * NW, g = rank * NW + warp;
+    auto share_begin = [&](int w) -> int { return (int)((long long)w * NC / G); };
+    const int ch0 = share_begin(g), nch = share_begin(g + 1) - ch0;
+    const int cpr = ((NC + G - 1) / G + kDRuns - 1) / kDRuns;                    // chunks per run
+    const unsigned long long ra = reinterpret_cast<unsigned long long>(reinterpret_cast<const T*>(p.z) + (long long)b * p.row_stride);
+    const unsigned char* const base = reinterpret_cast<const unsigned char*>(ALIGNED ? ra : ra & ~15ull);
+    const int shift = ALIGNED ? 0 : (int)((ra & 15ull) / sizeof(T));
+    const int g1 = (shift + p.V + N - 1) / N;                                    // granules that hold elements: [0, g1)
+    unsigned char* const ring = dyn_smem + (size_t)warp * kDRingB;
+
+    // self-test of the give-up path: the warp with the row's first chunk never asks for its first chunk and waits for it only
+    // briefly, so the wait runs out with nothing in flight
+    const bool expiring = (b == p.expire_row && ch0 == 0 && nch > 0);
+    auto issue = [&](int c, int slot) {
+        if (lane == 0 && c < nch && !(expiring && c == 0)) {
+            const int u0 = 32 * IT * (ch0 + c), u1 = u0 + 32 * IT;
+            const uint32_t bytes = (uint32_t)(min(ALIGNED ? u1 : u1 + 1, g1) - u0) * 16u;
+            uint64_t* bar = reinterpret_cast<uint64_t*>(&sh.bar[warp][slot]);
+            mbar_expect_tx(bar, bytes);
+            bulk_g2s(ring + slot * kDStage, base + (size_t)u0 * 16, bytes, bar);
+        }
+    };
+    for (int c = 0; c < kDRing; ++c) issue(c, c);
+    // every CTA of the cluster runs before anyone writes into rank 0
+    if (P > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    // what the last step of the row needs from global memory, asked for by the warp that will need it
     float u_row = 0.f, tg_row = 0.f;
     int32_t len_row = 0;
-    if (active && rank == 0 && warp == 0) {
+    if (g == 0) {
         if (p.u != nullptr) u_row = __ldg(p.u + b);
         tg_row = p.st.T_G[b];
         if (p.draft_len) len_row = p.draft_len[b];          // (only this row's CTA ever writes it)
     }
+    const float c1 = WARPED ? p.c1 : kLog2e;                // log2 e / temperature
+    const typename U::Cut cut = U::make_cut((WARPED && p.cut) ? __ldg(p.cut + b) : -INFINITY);
+    const bool greedy = p.argmax != 0;
+    if (P > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    DraftShared<NW>* const r0 = P > 1 ? cluster.map_shared_rank(&sh, 0) : &sh;
 
-    // this warp's share of the row, in 16-byte units
-    const int NU = p.V >> 3;
-    const int cu0 = (int)((long long)rank * NU / P), cu1 = (int)((long long)(rank + 1) * NU / P);
-    const int wu0 = cu0 + (int)((long long)warp * (cu1 - cu0) / kDW);
-    const int wu1 = cu0 + (int)((long long)(warp + 1) * (cu1 - cu0) / kDW);
-    const int nwu = wu1 - wu0;
-    const int nch = min(kDMaxChunks, (nwu + kDChunkUnits - 1) / kDChunkUnits);
-    const unsigned char* const src =
-        reinterpret_cast<const unsigned char*>(reinterpret_cast<const __nv_bfloat16*>(p.z) + (long long)b * p.row_stride) +
-        (size_t)wu0 * 16;
-    unsigned char* const bufs = dyn_smem + (size_t)warp * (2 * kDChunkBytes);
-
-    if (lane == 0) {
-        mbar_init(reinterpret_cast<uint64_t*>(&sh.bar[warp][0]), 1);
-        mbar_init(reinterpret_cast<uint64_t*>(&sh.bar[warp][1]), 1);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncwarp();
-    // every CTA of the cluster is running before anyone writes into rank 0 (a CTA on its own
-    // writes to itself, and every warp waits on barriers it set up itself)
-    if (P > 1) cluster.sync();
-    bool alive = true;
-    // self-test of the give-up path: this warp never asks for its first chunk and waits for it only
-    // briefly, so the wait runs out with nothing in flight
-    const bool expiring = (b == p.expire_row && rank == 0 && warp == 0);
-    auto issue = [&](int c) {
-        if (lane == 0 && c < nch && !(expiring && c == 0)) {
-            const uint32_t bytes = (uint32_t)min(kDChunkUnits, nwu - c * kDChunkUnits) * 16u;
-            uint64_t* bar = reinterpret_cast<uint64_t*>(&sh.bar[warp][c & 1]);
-            mbar_expect_tx(bar, bytes);
-            bulk_g2s(bufs + (size_t)(c & 1) * kDChunkBytes, src + (size_t)c * kDChunkBytes, bytes, bar);
-        }
-    };
-    // adjusted distribution: t = (z - max) log2 e / T, logits below the row's cutoff count as -inf
-    const float c1 = WARPED ? p.c1 : kLog2e;
-    const uint32_t cut2 = (WARPED && p.cut) ? cut_pair(__ldg(p.cut + b)) : kNoCut2;
-    float M = kFloorL;                                   // running shift (log2 domain)
-    // the largest logit so far (0 while there is none): t = (z - vM) log2 e is exactly 0 for it,
-    // so that a one-hot row gets S = 1, T = 0 and H = 0 exactly
-    float vM = 0.f;
-    float2 S2 = make_float2(0.f, 0.f), T2 = S2;          // lane partials under M
+    // v: the largest logit so far (kFloorL while there is none): t = (z - v) log2 e is exactly 0 for it, so
+    // that a one-hot row gets S = 1, T = 0 and H = 0 exactly
+    float v = kFloorL;
+    int vi = -1;
+    float2 S2 = make_float2(0.f, 0.f), T2 = S2, R2 = S2;    // lane partials under v; R2: S of the current run, not yet in S2
     uint32_t bad = 0u;
-    if (active) {
-        issue(0);
-        issue(1);
-        // table entries of chunks this warp does not have: no weight
-        if (lane >= nch && lane < kDMaxChunks) {
-            DraftShared<NW>* r0 = cluster.map_shared_rank(&sh, 0);
-            r0->cm[rank * kDW + warp][lane] = kFloorL;
-            r0->cs[rank * kDW + warp][lane] = 0.f;
+    const float2 L2 = pair2(c1);
+    int run = 0, in_run = 0, cfail = -1;                    // cfail: chunk whose copy never landed
+    int slot = 0;                                           // ring slot and phase of chunk c
+    uint32_t ph = 0;
+    for (int c = 0; c < nch; ++c) {
+        bool ok = mbar_wait_bounded(reinterpret_cast<uint64_t*>(&sh.bar[warp][slot]), ph,
+                                    expiring && c == 0 ? 64u : kCWaitSpins);
+        ok = __all_sync(0xFFFFFFFFu, ok);
+        if (!ok) {
+            if (lane == 0) atomicOr(p.st.status, ADASD_STATUS_TIMEOUT);
+            bad = 1u;
+            cfail = c;
+            break;
         }
-        int cfail = -1;                                      // chunk whose copy never landed
-        for (int c = 0; c < nch; ++c) {
-            bool ok = alive && mbar_wait_bounded(reinterpret_cast<uint64_t*>(&sh.bar[warp][c & 1]), (uint32_t)(c >> 1) & 1u,
-                                                 expiring && c == 0 ? 64u : kCWaitSpins);
-            ok = __all_sync(0xFFFFFFFFu, ok);
-            if (!ok) {
-                if (alive && lane == 0) atomicOr(p.st.status, ADASD_STATUS_TIMEOUT);
-                alive = false;
-                bad = 1u;
-                cfail = c;
-                break;
-            }
-            const unsigned char* sb = bufs + (size_t)(c & 1) * kDChunkBytes + (size_t)lane * 16;
-            const int ubase = c * kDChunkUnits + lane;
-            uint4 W[8];
-            uint32_t mx = 0xFF80FF80u;
+        const unsigned char* sb = ring + slot * kDStage + lane * 16;
+        const int ci = (ch0 + c) * IT;
+        auto load = [&](int k) -> uint4 {
+            uint4 w = *reinterpret_cast<const uint4*>(sb + k * 512);
+            if (!ALIGNED) w = U::realign(w, *reinterpret_cast<const uint4*>(sb + k * 512 + 16), shift);
+            return w;
+        };
+        auto mask = [&](uint4& w, int k) {                  // the row's end
+            const int e0 = (32 * (ci + k) + lane) * N;
+            if (e0 >= p.V) w = U::floor4();
+            else if (e0 + N > p.V) U::mask(w, 0, p.V - e0);
+        };
+        const bool edge = ch0 + c == NC - 1;
+        uint4 W[IT];
+        typename U::Max mx = U::max0();
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                W[i] = *reinterpret_cast<const uint4*>(sb + i * 512);
-                if (!(ubase + 32 * i < nwu)) W[i] = make_uint4(0xF149F149u, 0xF149F149u, 0xF149F149u, 0xF149F149u);
-                mx = bmax2(bmax2(mx, W[i].x), bmax2(W[i].y, bmax2(W[i].z, W[i].w)));
-            }
-            if (WARPED && cut2 != kNoCut2) {
+        for (int k = 0; k < IT; ++k) W[k] = load(k);
+        if (edge) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) bcut8(W[i], cut2);
-            }
-            // both buffers are in registers or free: fetch the chunk after the next
-            __syncwarp();
-            issue(c + 2);
-            const float2 mm = unpack2(mx);
-            if (mm.x != mm.x || mm.y != mm.y) bad = 1u;
-            const float vmax = warp_max_f32(fmaxf(mm.x, mm.y));
-            if (vmax == INFINITY) bad = 1u;
-            const float Mc = vmax > ADASD_FLOOR_BF ? vmax * c1 : kFloorL;
-            if (Mc > M) {                                 // raise the shift, rescale what is summed
-                const float d = M > kFloorL ? (vM - vmax) * c1 : kFloorL, f = ex2(d);
-                T2.x = f * fmaf(d, S2.x, T2.x);
-                T2.y = f * fmaf(d, S2.y, T2.y);
-                S2.x *= f;
-                S2.y *= f;
-                M = Mc;
-                vM = vmax;
-            }
-            const float2 nv2 = make_float2(-vM, -vM), L2 = make_float2(c1, c1);
-            float2 Sc = make_float2(0.f, 0.f);
+            for (int k = 0; k < IT; ++k) mask(W[k], k);
+        }
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const uint32_t w[4] = {W[i].x, W[i].y, W[i].z, W[i].w};
+        for (int k = 0; k < IT; ++k) U::max_add(mx, W[k]);
+        const float lm = U::max_val(mx, bad);
+        const float x = warp_max_f32(lm);
+        if (x == INFINITY) bad = 1u;
+        if (greedy && x > v && x > floor_v) {               // the lowest index of the chunk that has it
+            int first = 0x7FFFFFFF;
+            if (lm == x) {
+#pragma unroll 1
+                for (int k = IT - 1; k >= 0; --k) {
+                    uint4 w = load(k);
+                    mask(w, k);
+                    float2 z[NP];
+                    U::unpack(w, z);
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 z = unpack2(bclamp2(w[j]));
-                    const float2 t = __fmul2_rn(__fadd2_rn(z, nv2), L2);
-                    const float2 e = make_float2(ex2(t.x), ex2(t.y));
-                    Sc = __fadd2_rn(Sc, e);
-                    T2 = __ffma2_rn(e, t, T2);
+                    for (int j = NP - 1; j >= 0; --j) {
+                        const int e = (32 * (ci + k) + lane) * N + 2 * j;
+                        if (z[j].y == x) first = e + 1;
+                        if (z[j].x == x) first = e;
+                    }
                 }
             }
-            S2 = __fadd2_rn(S2, Sc);
-            const float cs = warp_sum(Sc.x + Sc.y);
-            if (lane == 0) {
-                DraftShared<NW>* r0 = cluster.map_shared_rank(&sh, 0);
-                r0->cm[rank * kDW + warp][c] = M;
-                r0->cs[rank * kDW + warp][c] = cs;
+            vi = __reduce_min_sync(0xFFFFFFFFu, first);
+        }
+        __syncwarp();
+        issue(c + kDRing, slot);                              // the chunk has been read, its slot is free
+        if (++slot == kDRing) {
+            slot = 0;
+            ph ^= 1u;
+        }
+        if (x > v && x > floor_v) {                         // a larger maximum: rescale what is summed
+            const float d = v > kFloorL ? (v - x) * c1 : kFloorL, f = ex2(d);
+            T2.x = f * fmaf(d, S2.x + R2.x, T2.x);
+            T2.y = f * fmaf(d, S2.y + R2.y, T2.y);
+            S2.x *= f;
+            S2.y *= f;
+            R2.x *= f;
+            R2.y *= f;
+            v = x;
+        }
+        const float nv = v > kFloorL ? -v : 0.f;
+        const float2 nv2 = pair2(nv);
+#pragma unroll
+        for (int k = 0; k < IT; ++k) {
+            if (WARPED) U::cut(W[k], cut);
+            float2 z[NP];
+            U::unpack(W[k], z);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                const float2 t = __fmul2_rn(__fadd2_rn(z[j], nv2), L2);
+                const float2 e = make_float2(ex2(t.x), ex2(t.y));
+                R2 = __fadd2_rn(R2, e);
+                T2 = __ffma2_rn(e, t, T2);
             }
         }
-        // a warp that gave up still waits (bounded) for what it had asked for and not taken: the
-        // chunk it gave up on and the one after it; nothing may land in this CTA after it has gone
-        if (cfail >= 0) {
-            for (int c = cfail; c < min(cfail + 2, nch); ++c)
-                if (!(expiring && c == 0))
-                    mbar_wait_bounded(reinterpret_cast<uint64_t*>(&sh.bar[warp][c & 1]), (uint32_t)(c >> 1) & 1u);
+        if (++in_run == cpr || c + 1 == nch) {
+            S2 = __fadd2_rn(S2, R2);
+            const float rs = warp_sum(R2.x + R2.y);
+            if (lane == 0) r0->run[g][run] = make_float2(v, rs);
+            R2 = make_float2(0.f, 0.f);
+            in_run = 0;
+            ++run;
         }
-        const float Sw = warp_sum(S2.x + S2.y), Tw = warp_sum(T2.x + T2.y);
-        bad = __reduce_or_sync(0xFFFFFFFFu, bad);
-        if (lane == 0)
-            cluster.map_shared_rank(&sh, 0)->wpart[rank * kDW + warp] = make_float4(M, Sw, Tw, __uint_as_float(bad));
+    }
+    // a warp that gave up still waits (bounded) for what it had asked for and not taken; nothing may
+    // land in this CTA after it has gone
+    if (cfail >= 0)
+        for (int c = cfail; c < min(cfail + kDRing, nch); ++c)
+            if (!(expiring && c == 0))
+                mbar_wait_bounded(reinterpret_cast<uint64_t*>(&sh.bar[warp][c % kDRing]), (uint32_t)(c / kDRing) & 1u);
+    const float Sw = warp_sum(S2.x + S2.y), Tw = warp_sum(T2.x + T2.y);
+    bad = __reduce_or_sync(0xFFFFFFFFu, bad);
+    if (lane >= run && lane < kDRuns) r0->run[g][lane] = make_float2(kFloorL, 0.f);      // runs this warp does not have
+    if (lane == 0) {
+        r0->wpart[g] = make_float4(v, Sw, Tw, __uint_as_float(bad));
+        r0->widx[g] = vi;
     }
     // totals and tables of every CTA are in rank 0's shared memory
     if (P > 1) cluster.sync();
     else __syncthreads();
-    if (!active || rank != 0) return;
+    if (g != 0) return;
     // (rank 0 only reads its own shared memory from here on; nobody writes to it any more)
 
-    if (warp == 0) {
-        // row totals: lane l holds warp-entry l (and l + 32 when P * 8 > 32)
-        const int NE = P * kDW;
-        const float4* wp = &sh.wpart[0];
-        float4 e0 = lane < NE ? wp[lane] : make_float4(kFloorL, 0.f, 0.f, 0.f);
-        float4 e1 = lane + 32 < NE ? wp[lane + 32] : make_float4(kFloorL, 0.f, 0.f, 0.f);
-        const float Mr = warp_max_f32(fmaxf(e0.x, e1.x));
-        const float d0 = e0.x - Mr, d1 = e1.x - Mr;
-        const float f0 = ex2(d0), f1 = ex2(d1);
-        const float S = warp_sum(f0 * e0.y + f1 * e1.y);
-        const float T = warp_sum(f0 * fmaf(d0, e0.y, e0.z) + f1 * fmaf(d1, e1.y, e1.z));
-        const uint32_t fl = __reduce_or_sync(0xFFFFFFFFu, __float_as_uint(e0.w) | __float_as_uint(e1.w));
-        const bool rowbad = (fl & 1u) || !(Mr > kFloorL);
-        const float lS = lg2(S);
-        float H = kLn2 * (lS - T / S), lse = kLn2 * (Mr + lS);
-        if (rowbad) H = lse = NAN;
+    // row totals: lane l holds warp l of the cluster, and l + 32
+    const float4 none = make_float4(kFloorL, 0.f, 0.f, 0.f);
+    const float4 e0 = lane < G ? sh.wpart[lane] : none, e1 = lane + 32 < G ? sh.wpart[lane + 32] : none;
+    const float Mr = warp_max_f32(fmaxf(e0.x, e1.x));
+    const float d0 = (e0.x - Mr) * c1, d1 = (e1.x - Mr) * c1;
+    const float w0 = ex2(d0) * e0.y, w1 = ex2(d1) * e1.y;
+    const float S = warp_sum(w0 + w1);
+    const float Tt = warp_sum(ex2(d0) * fmaf(d0, e0.y, e0.z) + ex2(d1) * fmaf(d1, e1.y, e1.z));
+    const uint32_t fl = __reduce_or_sync(0xFFFFFFFFu, __float_as_uint(e0.w) | __float_as_uint(e1.w));
+    const bool rowbad = (fl & 1u) || !(Mr > kFloorL);
+    const float lS = lg2(S);
+    float H = kLn2 * (lS - Tt / S), lse = kLn2 * fmaf(Mr, c1, lS);
+    if (rowbad) H = lse = NAN;
 
-        // x ~ q: the crossing of u * S in index order (rank, warp, chunk): first the warp share
-        // that holds it (entry l of the totals, and l + 32), then the chunk within that share
-        int tok = -1;
-        const bool sampling = (p.u != nullptr && p.token_out != nullptr);
-        if (sampling && !rowbad) {
-            float target = u_row * S;
-            const float w0 = f0 * e0.y, w1 = f1 * e1.y;
-            float i0 = w0, i1 = w1;
+    int tok = -1;
+    const bool sampling = !greedy && p.u != nullptr && p.token_out != nullptr;
+    if (greedy && !rowbad) {
+        // shares are in index order: the lowest index of those that have the maximum
+        const int i0 = lane < G && e0.x == Mr ? sh.widx[lane] : 0x7FFFFFFF, i1 = lane + 32 < G && e1.x == Mr ? sh.widx[lane + 32] : 0x7FFFFFFF;
+        tok = __reduce_min_sync(0xFFFFFFFFu, min(i0, i1));
+    } else if (sampling && !rowbad) {
+        // x ~ q: the crossing of u S in index order: first the share that holds it, then the run in it
+        float target = u_row * S;
+        float i0 = w0, i1 = w1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float t0 = __shfl_up_sync(0xFFFFFFFFu, i0, o), t1 = __shfl_up_sync(0xFFFFFFFFu, i1, o);
+            if (lane >= o) {
+                i0 += t0;
+                i1 += t1;
+            }
+        }
+        i1 += __shfl_sync(0xFFFFFFFFu, i0, 31);
+        const unsigned h0 = __ballot_sync(0xFFFFFFFFu, w0 > 0.f && i0 > target);
+        const unsigned h1 = __ballot_sync(0xFFFFFFFFu, w1 > 0.f && i1 > target);
+        const unsigned m0 = __ballot_sync(0xFFFFFFFFu, w0 > 0.f), m1 = __ballot_sync(0xFFFFFFFFu, w1 > 0.f);
+        int ent;
+        if (h0) ent = __ffs(h0) - 1;
+        else if (h1) ent = 32 + __ffs(h1) - 1;
+        else {                   // rounding left no crossing: last share with mass, last token with mass
+            ent = m1 ? 32 + 31 - __clz(m1) : 31 - __clz(m0);
+            target = INFINITY;
+        }
+        const float ebase = ent < 32 ? __shfl_sync(0xFFFFFFFFu, i0 - w0, ent) : __shfl_sync(0xFFFFFFFFu, i1 - w1, ent - 32);
+        const float2 rr = lane < kDRuns ? sh.run[ent][lane] : make_float2(kFloorL, 0.f);
+        const float rw = ex2((rr.x - Mr) * c1) * rr.y;
+        float incl = rw;
+#pragma unroll
+        for (int o = 1; o < kDRuns; o <<= 1) {
+            const float t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const unsigned ch = __ballot_sync(0xFFFFFFFFu, rw > 0.f && ebase + incl > target);
+        const unsigned cl = __ballot_sync(0xFFFFFFFFu, rw > 0.f);
+        const int r = ch ? __ffs(ch) - 1 : 31 - __clz(cl | 1u);
+        if (!ch) target = INFINITY;
+        float cc0 = ebase + __shfl_sync(0xFFFFFFFFu, incl - rw, r);
+        const int a0 = share_begin(ent) + r * cpr, a1 = min(share_begin(ent + 1), a0 + cpr);      // its chunks
+        int last = -1;
+        // the run again: a chunk at a time, lane l takes the units IT l .. IT l + IT - 1 of it, so that index order is
+        // lane order: one prefix over the lanes' sums places the crossing in a lane, which walks its tokens
+        const uint4* row = reinterpret_cast<const uint4*>(base);
+        for (int ci = a0; ci < a1 && tok < 0; ++ci) {
+            const int ub = 32 * IT * ci + lane * IT;
+            uint4 W[IT + 1];
+#pragma unroll
+            for (int k = 0; k < IT + (ALIGNED ? 0 : 1); ++k)
+                W[k] = ub + k < g1 ? __ldg(row + ub + k) : U::floor4();
+            float e[IT][N], ls = 0.f;
+#pragma unroll
+            for (int k = 0; k < IT; ++k) {
+                uint4 w = ALIGNED ? W[k] : U::realign(W[k], W[k + 1], shift);
+                const int el = (ub + k) * N;
+                if (el >= p.V) w = U::floor4();
+                else if (el + N > p.V) U::mask(w, 0, p.V - el);
+                if (WARPED) U::cut(w, cut);
+                float2 z[NP];
+                U::unpack(w, z);
+#pragma unroll
+                for (int j = 0; j < NP; ++j) {
+                    e[k][2 * j] = ex2((z[j].x - Mr) * c1);
+                    e[k][2 * j + 1] = ex2((z[j].y - Mr) * c1);
+                    ls += e[k][2 * j] + e[k][2 * j + 1];
+                }
+            }
+            float li = ls;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
-                const float t0 = __shfl_up_sync(0xFFFFFFFFu, i0, o), t1 = __shfl_up_sync(0xFFFFFFFFu, i1, o);
-                if (lane >= o) {
-                    i0 += t0;
-                    i1 += t1;
-                }
+                const float t = __shfl_up_sync(0xFFFFFFFFu, li, o);
+                if (lane >= o) li += t;
             }
-            const float tot0 = __shfl_sync(0xFFFFFFFFu, i0, 31);
-            i1 += tot0;
-            const unsigned h0 = __ballot_sync(0xFFFFFFFFu, w0 > 0.f && i0 > target);
-            const unsigned h1 = __ballot_sync(0xFFFFFFFFu, w1 > 0.f && i1 > target);
-            const unsigned m0 = __ballot_sync(0xFFFFFFFFu, w0 > 0.f), m1 = __ballot_sync(0xFFFFFFFFu, w1 > 0.f);
-            int ent = -1;
-            if (h0) ent = __ffs(h0) - 1;
-            else if (h1) ent = 32 + __ffs(h1) - 1;
-            else {                   // rounding left no crossing: last share with mass, last token with mass
-                if (m1) ent = 32 + 31 - __clz(m1);
-                else if (m0) ent = 31 - __clz(m0);
-                target = INFINITY;
-            }
-            if (ent >= 0) {
-                const float ebase = ent < 32 ? __shfl_sync(0xFFFFFFFFu, i0 - w0, ent)
-                                             : __shfl_sync(0xFFFFFFFFu, i1 - w1, ent - 32);
-                const float* cmf = &sh.cm[0][0] + ent * kDMaxChunks;
-                const float* csf = &sh.cs[0][0] + ent * kDMaxChunks;
-                const float v = lane < kDMaxChunks ? ex2(cmf[lane] - Mr) * csf[lane] : 0.f;
-                float incl = v;
+            float cc = cc0 + (li - ls);
+            int hit = -1;
 #pragma unroll
-                for (int o = 1; o < 16; o <<= 1) {
-                    const float t = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                    if (lane >= o) incl += t;
-                }
-                const unsigned ch = __ballot_sync(0xFFFFFFFFu, v > 0.f && ebase + incl > target);
-                const unsigned cl = __ballot_sync(0xFFFFFFFFu, v > 0.f);
-                int c = -1;
-                if (ch) c = __ffs(ch) - 1;
-                else if (cl) {
-                    c = 31 - __clz(cl);
-                    target = INFINITY;
-                }
-                if (c >= 0) {
-                    const float base = ebase + __shfl_sync(0xFFFFFFFFu, incl - v, c);
-                    const int r = ent / kDW, w = ent % kDW;
-                    const int cu0r = (int)((long long)r * NU / P), cu1r = (int)((long long)(r + 1) * NU / P);
-                    const int a0 = cu0r + (int)((long long)w * (cu1r - cu0r) / kDW);
-                    const int a1 = cu0r + (int)((long long)(w + 1) * (cu1r - cu0r) / kDW);
-                    const int u0 = a0 + c * kDChunkUnits, u1 = min(a1, u0 + kDChunkUnits);
-                    // the chunk again (4 KB, from L2), all of it in flight at once
-                    const uint4* row = reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(p.z) +
-                                                                      (long long)b * p.row_stride);
-                    // Lane l takes the units u0 + 8 l .. u0 + 8 l + 7, so that index order is lane order: one
-                    // prefix over the lanes' sums places the crossing in a lane, which walks its 64 tokens.
-                    uint4 Wq[8];
+            for (int k = 0; k < IT; ++k) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int u = u0 + lane * 8 + i;
-                        Wq[i] = u < u1 ? __ldg(row + u) : make_uint4(0xF149F149u, 0xF149F149u, 0xF149F149u, 0xF149F149u);
-                        if (WARPED) bcut8(Wq[i], cut2);
-                    }
-                    float wt[8][8];
-                    float ls = 0.f;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const uint32_t qw[4] = {Wq[i].x, Wq[i].y, Wq[i].z, Wq[i].w};
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const float2 z = unpack2(bclamp2(qw[j]));
-                            wt[i][2 * j] = ex2(fmaf(z.x, c1, -Mr));
-                            wt[i][2 * j + 1] = ex2(fmaf(z.y, c1, -Mr));
-                            ls += wt[i][2 * j] + wt[i][2 * j + 1];
-                        }
-                    }
-                    float li = ls;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const float t = __shfl_up_sync(0xFFFFFFFFu, li, o);
-                        if (lane >= o) li += t;
-                    }
-                    float cc = base + (li - ls);
-                    int hit = -1, last_pos = -1;
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            cc += wt[i][j];
-                            if (wt[i][j] > 0.f) {
-                                const int idx = (u0 + lane * 8 + i) * 8 + j;
-                                last_pos = idx;
-                                if (hit < 0 && cc > target) hit = idx;
-                            }
-                        }
-                    }
-                    const unsigned mh = __ballot_sync(0xFFFFFFFFu, hit >= 0);
-                    if (mh) tok = __shfl_sync(0xFFFFFFFFu, hit, __ffs(mh) - 1);
-                    if (tok < 0) {
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) last_pos = max(last_pos, __shfl_xor_sync(0xFFFFFFFFu, last_pos, o));
-                        tok = last_pos;
+                for (int j = 0; j < N; ++j) {
+                    cc += e[k][j];
+                    if (e[k][j] > 0.f) {
+                        last = (ub + k) * N + j;
+                        if (hit < 0 && cc > target) hit = last;
                     }
                 }
             }
+            const unsigned mh = __ballot_sync(0xFFFFFFFFu, hit >= 0);
+            if (mh) tok = __shfl_sync(0xFFFFFFFFu, hit, __ffs(mh) - 1);
+            cc0 += __shfl_sync(0xFFFFFFFFu, li, 31);
         }
-        if (lane == 0) {
-            if (rowbad) atomicOr(p.st.status, ADASD_STATUS_NAN);
-            p.H_out[b] = H;
-            if (p.lse_out) p.lse_out[b] = lse;
-            if (sampling) p.token_out[b] = tok;
-            const bool stop = H > tg_row;   // strict; NaN never stops
-            if (p.stop_out) p.stop_out[b] = stop ? 1 : 0;
-            if (p.draft_len) p.draft_len[b] = len_row + 1;
-            if (p.active && stop) p.active[b] = 0;
-        }
+        if (tok < 0) tok = __reduce_max_sync(0xFFFFFFFFu, last);
+    }
+    if (lane == 0) {
+        if (rowbad) atomicOr(p.st.status, ADASD_STATUS_NAN);
+        p.H_out[b] = H;
+        if (p.lse_out) p.lse_out[b] = lse;
+        if (sampling || greedy) p.token_out[b] = tok;
+        const bool stop = H > tg_row;   // strict; NaN never stops
+        if (p.stop_out) p.stop_out[b] = stop ? 1 : 0;
+        if (p.draft_len) p.draft_len[b] = len_row + 1;
+        if (p.active && stop) p.active[b] = 0;
     }
 }
 

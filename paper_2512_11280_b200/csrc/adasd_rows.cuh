@@ -66,7 +66,9 @@ struct DraftParams {
     State st;
     int32_t B, V;
     int32_t expire_row;     // self-test of the bounded waits: the row whose first copy is never asked for (-1: none)
-    float inv_temp, c1;     // adjusted distribution: 1 / temperature, log2 e / temperature
+    int32_t argmax;         // 1: the token is argmax q (greedy drafting)
+    int32_t early;          // 1: the next call's CTAs may be set up while this one runs
+    float c1;               // adjusted distribution: log2 e / temperature
     const float* cut;       // [B] logit below which a row's tokens are cut (null: no cut)
 };
 
@@ -80,97 +82,6 @@ struct RowShared {
     int32_t token;           // sampled token, written by the chosen warp
     int32_t is_last;
 };
-
-// ------------------------------------------------------------------------------------
-// Draft step: H(q), lse, x ~ q, stop = H > T_G   (Algorithm 1, generation loop body)
-// ------------------------------------------------------------------------------------
-template <typename T, bool VEC>
-__global__ void __launch_bounds__(kThreads) draft_kernel(DraftParams p) {
-    constexpr int N = Elt<T>::N;
-    cg::cluster_group cluster = cg::this_cluster();
-    const int CS = (int)cluster.num_blocks();
-    const int rank = (int)cluster.block_rank();
-    const int b = blockIdx.x / CS;
-    if (p.active && p.active[b] == 0) return;   // same decision in every CTA of the cluster
-
-    __shared__ RowShared sh;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int GW = CS * kWarps, gw = rank * kWarps + warp;
-    const int NU = (p.V + N - 1) / N;
-    const int u0 = (int)((long long)gw * NU / GW), u1 = (int)((long long)(gw + 1) * NU / GW);
-    const T* row = reinterpret_cast<const T*>(p.z) + (long long)b * p.row_stride;
-    const RowWarp wr = {p.inv_temp, p.cut ? p.cut[b] : -INFINITY};
-
-    // pass A: max, NaN flag
-    float vA[2] = {-INFINITY, 0.f};
-    for (int u = u0 + lane; u < u1; u += 32) {
-        float x[N];
-        load_unit_w<T, VEC>(row, u, p.V, x, wr);
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            vA[1] = (x[j] != x[j]) ? 1.f : vA[1];
-            vA[0] = fmaxf(vA[0], x[j]);
-        }
-    }
-    cluster_allreduce<2, true>(vA, sh.warp, sh.xA, CS, rank, cluster);
-    const bool bad = (vA[1] > 0.f) || !(vA[0] > kFloor) || (vA[0] == INFINITY);
-    const float m = vA[0];
-
-    // pass B: S = sum 2^t, T = sum 2^t t with t = (z - m) log2e (exactly 0 at the maximum, so
-    // S >= 1 and a one-hot row has H == 0 exactly); per-warp S for sampling
-    float vB[2] = {0.f, 0.f};
-    for (int u = u0 + lane; u < u1; u += 32) {
-        float x[N];
-        load_unit_w<T, VEC>(row, u, p.V, x, wr);
-#pragma unroll
-        for (int j = 0; j < N; ++j) {
-            float t = (fmaxf(x[j], kFloor) - m) * kLog2e;
-            float e = ex2(t);
-            vB[0] += e;
-            vB[1] = fmaf(e, t, vB[1]);
-        }
-    }
-    {
-        float ws = warp_sum(vB[0]);
-        if (lane == 0)
-            for (int r = 0; r < CS; ++r) cluster.map_shared_rank(sh.wtab, r)[gw] = ws;
-    }
-    cluster_allreduce<2, false>(vB, sh.warp, sh.xB, CS, rank, cluster);
-
-    const float S = vB[0];
-    const float log2S = lg2(S);
-    float H = kLn2 * (log2S - vB[1] / S);
-    float lse = fmaf(kLn2, log2S, m);
-    if (bad) H = lse = NAN;
-
-    // x ~ q by inverse CDF in index order
-    const bool sampling = (p.u != nullptr && p.token_out != nullptr);
-    if (sampling && !bad) {
-        float base = 0.f, target = 0.f;
-        int chosen = select_warp(sh.wtab, GW, p.u[b], base, target);
-        if (chosen == gw) {
-            int tok = warp_scan_select<N>(u0, u1, p.V, base, target, [&](int u, float(&w)[N]) {
-                float x[N];
-                load_unit_w<T, VEC>(row, u, p.V, x, wr);
-#pragma unroll
-                for (int j = 0; j < N; ++j) w[j] = ex2((fmaxf(x[j], kFloor) - m) * kLog2e);
-            });
-            if (lane == 0) p.token_out[b] = tok;
-        }
-    } else if (sampling && rank == 0 && threadIdx.x == 0) {
-        p.token_out[b] = -1;
-    }
-    if (rank == 0 && threadIdx.x == 0) {
-        if (bad) atomicOr(p.st.status, ADASD_STATUS_NAN);
-        p.H_out[b] = H;
-        if (p.lse_out) p.lse_out[b] = lse;
-        const bool stop = H > p.st.T_G[b];   // strict; NaN never stops
-        if (p.stop_out) p.stop_out[b] = stop ? 1 : 0;
-        if (p.draft_len) p.draft_len[b] += 1;
-        if (p.active && stop) p.active[b] = 0;
-    }
-    cluster.sync();   // no CTA leaves while a peer may still address its shared memory
-}
 
 // ------------------------------------------------------------------------------------
 // Verification position (b,i): softmax statistics of q_i and p_i, H, D_JS, d_i, y_i ~ p_i

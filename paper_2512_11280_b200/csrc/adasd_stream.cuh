@@ -163,6 +163,7 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
         ++n_items;
         __syncwarp();
     };
+    const float2 L2 = pair2(c1);
     bool alive = true;
     int is = 0, n_issued = 0, n_taken = 0;
     auto issue = [&]() {                         // the next chunk
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
                     v = m;
                 }
                 const float nv = v > kFloorL ? -v : 0.f;
-                const float2 nv2 = make_float2(nv, nv), L2 = make_float2(c1, c1);
+                const float2 nv2 = pair2(nv);
 #pragma unroll 4
                 for (int k = 0; k < IT; ++k) {
                     uint4 w = load(k);
