@@ -212,6 +212,13 @@ class Context:
             self.handle = None
             raise AdasdError(rc, "adasd_create")
         self.B, self.V, self.Kmax = B, V, Kmax
+        # What every hot call needs, looked up once: an engine issues these calls between two kernels of
+        # a few microseconds each, so the marshalling is kept to the address of each tensor.
+        L = lib()
+        self._draft_entropy, self._verify = L.adasd_draft_entropy, L.adasd_verify
+        self._vanilla_verify, self._greedy_verify = L.adasd_vanilla_verify, L.adasd_greedy_verify
+        self._raw_stream = torch._C._cuda_getCurrentRawStream
+        self._rec_key, self._rec = None, None      # the last record's addresses and their struct
 
     def close(self) -> None:
         if getattr(self, "handle", None):
@@ -225,7 +232,7 @@ class Context:
             pass
 
     def _stream(self) -> int:
-        return self.torch.cuda.current_stream(self.device).cuda_stream
+        return self._raw_stream(self.device.index)
 
     @staticmethod
     def _check(rc: int, where: str) -> None:
@@ -255,23 +262,40 @@ class Context:
 
     def draft_entropy(self, logits, H_out, u=None, token_out=None, active=None, lse_out=None,
                       stop_out=None, draft_len=None, row_stride: Optional[int] = None) -> None:
-        rs = logits.stride(0) if row_stride is None else row_stride
-        self._check(adasd_draft_entropy(self.handle, logits.data_ptr(), rs, _ptr(u), _ptr(active),
-                                        H_out.data_ptr(), _ptr(lse_out), _ptr(token_out),
-                                        _ptr(stop_out), _ptr(draft_len), self._stream()),
-                    "adasd_draft_entropy")
+        rc = self._draft_entropy(self.handle, logits.data_ptr(),
+                                 logits.stride(0) if row_stride is None else row_stride,
+                                 None if u is None else u.data_ptr(),
+                                 None if active is None else active.data_ptr(), H_out.data_ptr(),
+                                 None if lse_out is None else lse_out.data_ptr(),
+                                 None if token_out is None else token_out.data_ptr(),
+                                 None if stop_out is None else stop_out.data_ptr(),
+                                 None if draft_len is None else draft_len.data_ptr(),
+                                 self._raw_stream(self.device.index))
+        if rc:
+            raise AdasdError(rc, "adasd_draft_entropy")
+
+    def _record_ref(self, rec: Optional[dict]):
+        """The C struct of a record of device tensors; the struct of the last record is kept and
+        used again as long as the addresses are the same."""
+        if rec is None:
+            return None
+        key = [(k, v.data_ptr()) if v is not None else (k, None) for k, v in rec.items()]
+        if key != self._rec_key:
+            self._rec, self._rec_key = C.byref(RoundRecord(**dict(key))), key
+        return self._rec
 
     def verify(self, draft_logits, target_logits, draft_tokens, u_target, u_accept, accept_len,
                next_token, draft_len=None, record: Optional[dict] = None,
                fuse_update: bool = True) -> None:
-        rs = self.record_struct(record)
-        self._check(adasd_verify(self.handle, draft_logits.data_ptr(), target_logits.data_ptr(),
-                                 draft_logits.stride(0), draft_logits.stride(1),
-                                 target_logits.stride(0), target_logits.stride(1),
-                                 draft_tokens.data_ptr(), _ptr(draft_len), u_target.data_ptr(),
-                                 u_accept.data_ptr(), accept_len.data_ptr(), next_token.data_ptr(),
-                                 rs, ADASD_FUSE_UPDATE if fuse_update else 0, self._stream()),
-                    "adasd_verify")
+        ds, ts = draft_logits.stride(), target_logits.stride()
+        rc = self._verify(self.handle, draft_logits.data_ptr(), target_logits.data_ptr(), ds[0], ds[1],
+                          ts[0], ts[1], draft_tokens.data_ptr(),
+                          None if draft_len is None else draft_len.data_ptr(), u_target.data_ptr(),
+                          u_accept.data_ptr(), accept_len.data_ptr(), next_token.data_ptr(),
+                          self._record_ref(record), ADASD_FUSE_UPDATE if fuse_update else 0,
+                          self._raw_stream(self.device.index))
+        if rc:
+            raise AdasdError(rc, "adasd_verify")
 
     def update_thresholds(self, record: dict) -> None:
         self._check(adasd_update_thresholds(self.handle, self.record_struct(record), self._stream()),
@@ -279,20 +303,25 @@ class Context:
 
     def vanilla_verify(self, draft_logits, target_logits, draft_tokens, u_accept, u_resample,
                        accept_len, next_token, draft_len=None, alpha_out=None) -> None:
-        self._check(adasd_vanilla_verify(self.handle, draft_logits.data_ptr(),
-                                         target_logits.data_ptr(), draft_logits.stride(0),
-                                         draft_logits.stride(1), target_logits.stride(0),
-                                         target_logits.stride(1), draft_tokens.data_ptr(),
-                                         _ptr(draft_len), u_accept.data_ptr(), u_resample.data_ptr(),
-                                         accept_len.data_ptr(), next_token.data_ptr(),
-                                         _ptr(alpha_out), self._stream()), "adasd_vanilla_verify")
+        ds, ts = draft_logits.stride(), target_logits.stride()
+        rc = self._vanilla_verify(self.handle, draft_logits.data_ptr(), target_logits.data_ptr(), ds[0],
+                                  ds[1], ts[0], ts[1], draft_tokens.data_ptr(),
+                                  None if draft_len is None else draft_len.data_ptr(), u_accept.data_ptr(),
+                                  u_resample.data_ptr(), accept_len.data_ptr(), next_token.data_ptr(),
+                                  None if alpha_out is None else alpha_out.data_ptr(),
+                                  self._raw_stream(self.device.index))
+        if rc:
+            raise AdasdError(rc, "adasd_vanilla_verify")
 
     def greedy_verify(self, target_logits, draft_tokens, accept_len, next_token, draft_len=None,
                       argmax_out=None) -> None:
-        self._check(adasd_greedy_verify(self.handle, target_logits.data_ptr(), target_logits.stride(0),
-                                        target_logits.stride(1), draft_tokens.data_ptr(), _ptr(draft_len),
-                                        accept_len.data_ptr(), next_token.data_ptr(), _ptr(argmax_out),
-                                        self._stream()), "adasd_greedy_verify")
+        ts = target_logits.stride()
+        rc = self._greedy_verify(self.handle, target_logits.data_ptr(), ts[0], ts[1], draft_tokens.data_ptr(),
+                                 None if draft_len is None else draft_len.data_ptr(), accept_len.data_ptr(),
+                                 next_token.data_ptr(), None if argmax_out is None else argmax_out.data_ptr(),
+                                 self._raw_stream(self.device.index))
+        if rc:
+            raise AdasdError(rc, "adasd_greedy_verify")
 
     def gen_only_update(self, H_draft, accept_len, draft_len=None) -> None:
         self._check(adasd_gen_only_update(self.handle, H_draft.data_ptr(), _ptr(draft_len),
