@@ -14,6 +14,7 @@
 #include "adasd_rows.cuh"
 #include "adasd_cluster.cuh"
 #include "adasd_spec.cuh"
+#include "adasd_verify_tail.cuh"
 #include "adasd_draft_stream.cuh"
 #include "adasd_stream.cuh"
 #include "adasd_modes.cuh"
@@ -164,14 +165,13 @@ int kernel_static_smem(K kern) {
     return (int)fa.sharedSizeBytes;
 }
 
-// Both modes run the warp-specialised kernel.
-template <int ITER, int MODE>
+template <int ITER>
 int fast_occupancy(int cs, int smem) {
-    return kernel_occupancy(spec_verify_kernel<ITER, MODE>, kSThreads, cs, smem);
+    return kernel_occupancy(spec_verify_kernel<ITER>, kSThreads, cs, smem);
 }
-template <int ITER, int MODE>
+template <int ITER>
 int fast_static_smem() {
-    return kernel_static_smem(spec_verify_kernel<ITER, MODE>);
+    return kernel_static_smem(spec_verify_kernel<ITER>);
 }
 
 #define ADASD_ITER_SWITCH(iter, CALL, fail)  \
@@ -189,25 +189,22 @@ int fast_static_smem() {
         default: return fail;                \
     }
 
-template <int MODE>
 int fast_occupancy_iter(int iter, int cs, int smem) {
-#define CALL(I) fast_occupancy<I, MODE>(cs, smem)
+#define CALL(I) fast_occupancy<I>(cs, smem)
     ADASD_ITER_SWITCH(iter, CALL, 0)
 #undef CALL
 }
-template <int MODE>
 int fast_static_smem_iter(int iter) {
-#define CALL(I) fast_static_smem<I, MODE>()
+#define CALL(I) fast_static_smem<I>()
     ADASD_ITER_SWITCH(iter, CALL, -1)
 #undef CALL
 }
 
-// Chooses, for one mode, the cluster size that covers the most SMs among those whose per-CTA
+// Verification kernel of aligned bf16 rows: chooses the cluster size that covers the most SMs among those whose per-CTA
 // slice fits on chip: two position buffers per compute warp, iter * 512 bytes per row (the
 // 2^t values live in registers or are worked out again).  bf16 rows of a multiple of 8
 // elements only.
-template <int MODE>
-void fast_setup_mode(adasd_ctx* c, size_t smem_optin) {
+void fast_setup(adasd_ctx* c, size_t smem_optin) {
     adasd_ctx::Fast& f = c->fast;
     f.iter = 0;
     const int V = c->cfg.V;
@@ -219,11 +216,11 @@ void fast_setup_mode(adasd_ctx* c, size_t smem_optin) {
         const int ncu = (NU + cs - 1) / cs, nwi = (ncu + 31) / 32;
         const int I_lo = nwi / kSW, rem = nwi % kSW, iter = I_lo + (rem ? 1 : 0);
         if (iter < 1 || iter > kSMaxIter) continue;
-        const int st = fast_static_smem_iter<MODE>(iter);
+        const int st = fast_static_smem_iter(iter);
         if (st < 0) continue;
         const int smem = nwi * 2048;      // two position buffers: 512 bytes per row and warp-iteration
         if (smem > (int)smem_optin - st - 1024) continue;
-        const int ncl = fast_occupancy_iter<MODE>(iter, cs, smem);
+        const int ncl = fast_occupancy_iter(iter, cs, smem);
         const int score = ncl * cs;
         if (score > best_score) {
             best_score = score;
@@ -234,8 +231,7 @@ void fast_setup_mode(adasd_ctx* c, size_t smem_optin) {
         }
     }
 }
-void fast_setup(adasd_ctx* c, size_t smem_optin) {
-    fast_setup_mode<MODE_ADASD>(c, smem_optin);
+void cutoff_setup(adasd_ctx* c) {
     c->cut_hist = cudaFuncSetAttribute(row_cutoff_hist_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        kHistWords * 4) == cudaSuccess;
     if (!c->cut_hist) cudaGetLastError();
@@ -377,41 +373,26 @@ int launch_draft(adasd_ctx* c, const DraftParams& p, bool aligned, cudaStream_t 
     return aligned ? launch_draft<T, true>(c, p, stream) : launch_draft<T, false>(c, p, stream);
 }
 
-template <int ITER, int MODE, bool WARPED>
+template <int ITER, bool WARPED>
 int fast_launch(adasd_ctx* c, const VerifyParams& p, cudaStream_t stream) {
     const long long positions = (long long)p.B * (p.Kmax + 1);
     const adasd_ctx::Fast& f = c->fast;
     ClusterGeom gq = f.geom;
     if (positions < gq.ncl) gq.ncl = (int)positions;
-    cudaLaunchConfig_t lc;
-    memset(&lc, 0, sizeof(lc));
-    lc.gridDim = dim3((unsigned)(gq.ncl * f.cs), 1, 1);
-    lc.blockDim = dim3((unsigned)kSThreads, 1, 1);
-    lc.dynamicSmemBytes = (size_t)f.smem;
-    lc.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)f.cs;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    lc.attrs = attr;
-    lc.numAttrs = 1;
     if (WARPED) {
         // the instantiation for adjusted distributions: same footprint, its own attribute
-        CUDA_TRY(cudaFuncSetAttribute(spec_verify_kernel<ITER, MODE, WARPED>, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem));
+        CUDA_TRY(cudaFuncSetAttribute(spec_verify_kernel<ITER, WARPED>, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem));
     }
-    CUDA_TRY(cudaLaunchKernelEx(&lc, spec_verify_kernel<ITER, MODE, WARPED>, p, gq));
-    return ADASD_OK;
+    return launch_pdl(spec_verify_kernel<ITER, WARPED>, gq.ncl * f.cs, kSThreads, f.smem, f.cs, stream, p, gq);
 }
 
-template <int MODE>
 int fast_launch_iter(adasd_ctx* c, const VerifyParams& p, cudaStream_t stream) {
     if (c->warp_on()) {
-#define CALL(I) fast_launch<I, MODE, true>(c, p, stream)
+#define CALL(I) fast_launch<I, true>(c, p, stream)
         ADASD_ITER_SWITCH(c->fast.iter, CALL, ADASD_ERR_SHAPE)
 #undef CALL
     }
-#define CALL(I) fast_launch<I, MODE, false>(c, p, stream)
+#define CALL(I) fast_launch<I, false>(c, p, stream)
     ADASD_ITER_SWITCH(c->fast.iter, CALL, ADASD_ERR_SHAPE)
 #undef CALL
 }
@@ -445,11 +426,6 @@ int fill_verify_params(adasd_ctx* ctx, VerifyParams& p, const void* zd, const vo
     p.B = ctx->cfg.B;
     p.V = ctx->cfg.V;
     p.Kmax = ctx->cfg.Kmax;
-    p.tail.Kmax = ctx->cfg.Kmax;
-    p.tail.min_samples = ctx->cfg.min_kde_samples;
-    p.tail.bw_rule = ctx->cfg.kde_bandwidth;
-    p.tail.reject_rule = ctx->cfg.reject_rule;
-    p.tail.update = 0;
     p.inv_temp = 1.f / ctx->temperature;
     p.c1 = kLog2e / ctx->temperature;
     if (ctx->cuts_on()) {
@@ -507,22 +483,30 @@ int launch_round_cutoffs(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t str
     return launch_cutoffs(ctx, p.zd, p.d_seq, p.d_row, p.Kmax, 0, p.draft_len, nullptr, ctx->cut_d, stream);
 }
 
-template <int MODE>
 int launch_verify(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
     const long long positions = (long long)p.B * (p.Kmax + 1);
     const int cs = pick_cluster(ctx, positions);
     const bool vec = vec_ok(p.zd, ctx->cfg.dtype, {p.d_seq, p.d_row}) &&
                      vec_ok(p.zt, ctx->cfg.dtype, {p.t_seq, p.t_row});
     if (int rc = launch_round_cutoffs(ctx, p, stream)) return rc;
-    if (vec && ctx->fast.iter > 0) {
-        return fast_launch_iter<MODE>(ctx, p, stream);
-    }
+    if (vec && ctx->fast.iter > 0) return fast_launch_iter(ctx, p, stream);
     if (ctx->cfg.dtype == ADASD_BF16) {
-        return vec ? launch_cluster(verify_kernel<__nv_bfloat16, true, MODE>, p, positions, cs, stream)
-                   : launch_cluster(verify_kernel<__nv_bfloat16, false, MODE>, p, positions, cs, stream);
+        return vec ? launch_cluster(verify_kernel<__nv_bfloat16, true, MODE_ADASD>, p, positions, cs, stream)
+                   : launch_cluster(verify_kernel<__nv_bfloat16, false, MODE_ADASD>, p, positions, cs, stream);
     }
-    return vec ? launch_cluster(verify_kernel<float, true, MODE>, p, positions, cs, stream)
-               : launch_cluster(verify_kernel<float, false, MODE>, p, positions, cs, stream);
+    return vec ? launch_cluster(verify_kernel<float, true, MODE_ADASD>, p, positions, cs, stream)
+               : launch_cluster(verify_kernel<float, false, MODE_ADASD>, p, positions, cs, stream);
+}
+
+// CTAs per sequence of the tail kernel: a list entry costs every candidate one exponential, so a
+// sequence whose lists can hold more than a few entries per thread gets more threads, as long as the
+// sequences leave room for them.
+int tail_cluster(const adasd_ctx* c) {
+    int S = 1;
+    while (S < kTailMaxS && (long long)c->cfg.list_capacity > 4LL * kTailThreads * S &&
+           (long long)c->cfg.B * S * 2 <= 4LL * c->sm_count)
+        S *= 2;
+    return S;
 }
 
 struct DeviceGuard {
@@ -639,16 +623,8 @@ int adasd_create(adasd_ctx** out, const adasd_config* cfg) {
     ALLOC(s.LR, B * cap);
     ALLOC(s.status, 1);
     ALLOC(t.H_d, B * K);
-    ALLOC(t.H_t, B * (K + 1));
-    ALLOC(t.lse_d, B * K);
-    ALLOC(t.lse_t, B * (K + 1));
-    ALLOC(t.jsd, B * K);
     ALLOC(t.dist, B * K);
-    ALLOC(t.p_acc, B * K);
     ALLOC(t.y, B * (K + 1));
-    ALLOC(t.ticket, B);
-    ALLOC(t.q_items, B);
-    ALLOC(t.q_ctl, 4);
     ALLOC(c->cut_t, B * (K + 1));
     ALLOC(c->cut_d, B * K);
     ALLOC(c->cut_row, B);
@@ -659,8 +635,10 @@ int adasd_create(adasd_ctx** out, const adasd_config* cfg) {
     c->temperature = 1.f;
     c->top_k = 0;
     c->top_p = 1.f;
-    if (rc == ADASD_OK && cudaMemset(t.q_items, 0xFF, B * sizeof(int32_t)) != cudaSuccess) rc = ADASD_ERR_CUDA;
-    if (rc == ADASD_OK) fast_setup(c, prop.sharedMemPerBlockOptin);
+    if (rc == ADASD_OK) {
+        fast_setup(c, prop.sharedMemPerBlockOptin);
+        cutoff_setup(c);
+    }
     if (rc == ADASD_OK) {
         const cudaError_t e1 = cfg->dtype == ADASD_BF16 ? stream_prepare<__nv_bfloat16, true>(c->stream_it) : stream_prepare<float, true>(c->stream_it);
         const cudaError_t e2 = cfg->dtype == ADASD_BF16 ? stream_prepare<__nv_bfloat16, false>(c->stream_it) : stream_prepare<float, false>(c->stream_it);
@@ -788,8 +766,30 @@ int adasd_verify(adasd_ctx* ctx, const void* draft_logits_dev, const void* targe
     p.accept_len = accept_len_dev;
     p.next_token = next_token_dev;
     if (record) p.user = *record;
-    p.tail.update = (flags & ADASD_FUSE_UPDATE) ? 1u : 0u;
-    return launch_verify<MODE_ADASD>(ctx, p, (cudaStream_t)stream);
+    cudaStream_t st = (cudaStream_t)stream;
+    if ((rc = launch_verify(ctx, p, st)) != ADASD_OK) return rc;
+    TailParams t;
+    memset(&t, 0, sizeof(t));
+    t.cfg.Kmax = ctx->cfg.Kmax;
+    t.cfg.min_samples = ctx->cfg.min_kde_samples;
+    t.cfg.bw_rule = ctx->cfg.kde_bandwidth;
+    t.cfg.reject_rule = ctx->cfg.reject_rule;
+    t.cfg.update = (flags & ADASD_FUSE_UPDATE) ? 1u : 0u;
+    t.st = ctx->st;
+    t.H_d = ctx->sc.H_d;
+    t.dist = ctx->sc.dist;
+    t.y = ctx->sc.y;
+    t.x = p.x;
+    t.u_accept = p.u_accept;
+    t.draft_len = p.draft_len;
+    t.p_acc = p.user.p_acc;
+    t.accept_len_rec = p.user.accept_len;
+    t.rejected_rec = p.user.rejected;
+    t.draft_len_rec = p.user.draft_len;
+    t.accept_len = p.accept_len;
+    t.next_token = p.next_token;
+    const int S = tail_cluster(ctx);
+    return launch_pdl(verify_tail_kernel, ctx->cfg.B * S, kTailThreads, 0, S, st, t);
 }
 
 int adasd_update_thresholds(adasd_ctx* ctx, const adasd_round_record* record, void* stream) {
@@ -1098,7 +1098,6 @@ int adasd_vanilla_verify_static(int32_t B, int32_t V, int32_t Kmax, int32_t dtyp
     p.B = B;
     p.V = V;
     p.Kmax = Kmax;
-    p.tail.Kmax = Kmax;
 
     const long long positions = (long long)B * (Kmax + 1);
     int cs = kMaxCluster;

@@ -13,20 +13,13 @@ namespace adasd {
 constexpr int MODE_ADASD = 0;
 constexpr int MODE_VANILLA = 1;
 
-struct Scratch {            // context-owned per-round scratch, all [B,Kmax(+1)]
-    float* H_d;
-    float* H_t;
-    float* lse_d;
-    float* lse_t;
-    float* jsd;
+struct Scratch {            // per-round scratch: the context's, or the fixed array of the allocation-free call
+    float* H_d;             // [B,Kmax] entropies and distances of a round's candidates, for its tail
     float* dist;
-    float* p_acc;
-    int32_t* y;
-    int32_t* van_flag;      // [B,Kmax] vanilla: 1 accept / 0 reject
-    int32_t* van_tok;       // [B,Kmax+1] vanilla: resample (or bonus) candidate
-    uint32_t* ticket;       // [B] arrival counter of a sequence's positions
-    int32_t* q_items;       // [B] chip-wide queue of completed sequences awaiting their tail (-1: empty)
-    uint32_t* q_ctl;        // [4] queue counters: pushed, drawn, workers gone (all 0 between launches)
+    int32_t* y;             // [B,Kmax+1] target samples
+    int32_t* van_flag;      // allocation-free vanilla call: [B,Kmax] 1 accept / 0 reject
+    int32_t* van_tok;       // ... [B,Kmax+1] resample (or bonus) candidate
+    uint32_t* ticket;       // ... [B] arrival counter of a sequence's positions
 };
 
 struct VerifyParams {
@@ -44,7 +37,6 @@ struct VerifyParams {
     adasd_round_record user;   // caller's record (entries may be null)
     Scratch sc;
     State st;
-    TailConfig tail;
     int32_t B, V, Kmax;
     // adjusted distribution (Sec. 2.1.1): 1 / temperature and, per row, the logit below which
     // tokens are cut (null: no cut); the staged kernels fold the temperature into c1 = log2 e / T
@@ -79,14 +71,11 @@ struct RowShared {
     float xC[kMaxCluster * 4];
     float wtab[kMaxGW];      // per-warp weight totals of the row being sampled
     float wtab2[kMaxGW];     // vanilla: per-warp residual totals
-    int32_t token;           // sampled token, written by the chosen warp
-    int32_t is_last;
 };
 
 // ------------------------------------------------------------------------------------
 // Verification position (b,i): softmax statistics of q_i and p_i, H, D_JS, d_i, y_i ~ p_i
-// (AdaSD mode) or alpha_i and the residual sample (vanilla mode).  The cluster that
-// publishes the last position of a sequence runs that sequence's tail.
+// (AdaSD mode) or alpha_i and the residual sample (vanilla mode).
 // ------------------------------------------------------------------------------------
 template <typename T, bool VEC, int MODE>
 __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
@@ -103,7 +92,6 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
     const bool bonus = (i == K_t);
 
     __shared__ RowShared sh;
-    __shared__ TailShared tsh;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int GW = CS * kWarps, gw = rank * kWarps + warp;
     const int NU = (p.V + N - 1) / N;
@@ -282,8 +270,6 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
                 p.sc.y[it] = -1;
                 if (p.user.y) p.user.y[it] = -1;
             }
-            p.sc.H_t[it] = Ht;
-            p.sc.lse_t[it] = lse_t;
             if (p.user.H_t) p.user.H_t[it] = Ht;
             if (p.user.lse_t) p.user.lse_t[it] = lse_t;
             if (!bonus) {
@@ -295,8 +281,6 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
                 dist = fminf(dist, 1.f);
                 if (bad) Hd = lse_d = jsd = dist = NAN;
                 p.sc.H_d[id] = Hd;
-                p.sc.lse_d[id] = lse_d;
-                p.sc.jsd[id] = jsd;
                 p.sc.dist[id] = dist;
                 if (p.user.H_d) p.user.H_d[id] = Hd;
                 if (p.user.lse_d) p.user.lse_d[id] = lse_d;
@@ -314,47 +298,21 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
 
     // all writes of this cluster are done once every CTA has passed this barrier
     cluster.sync();
-    if (rank != 0) return;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        unsigned old = atomicAdd(p.sc.ticket + b, 1u);
-        int last = (old == (unsigned)K_t);
-        if (last) {
-            p.sc.ticket[b] = 0u;    // ready for the next round
-            __threadfence();
+    if (MODE == MODE_ADASD || rank != 0 || threadIdx.x != 0) return;
+    // vanilla: the cluster that publishes the last position of a sequence finds its longest accepted prefix
+    __threadfence();
+    if (atomicAdd(p.sc.ticket + b, 1u) != (unsigned)K_t) return;
+    p.sc.ticket[b] = 0u;    // ready for the next round
+    __threadfence();
+    int w = K_t;
+    for (int j = 0; j < K_t; ++j) {
+        if (__ldcg(p.sc.van_flag + (size_t)b * Kmax + j) == 0) {
+            w = j;
+            break;
         }
-        sh.is_last = last;
     }
-    __syncthreads();
-    if (!sh.is_last) return;
-
-    if (MODE == MODE_ADASD) {
-        TailIO io;
-        io.H_d = p.sc.H_d;
-        io.dist = p.sc.dist;
-        io.y = p.sc.y;
-        io.x = p.x;
-        io.u_accept = p.u_accept;
-        io.draft_len = p.draft_len;
-        io.p_acc = p.sc.p_acc;
-        io.p_acc_user = p.user.p_acc;
-        io.accept_len = p.accept_len;
-        io.next_token = p.next_token;
-        io.accept_len_rec = p.user.accept_len;
-        io.rejected_rec = p.user.rejected;
-        io.draft_len_rec = p.user.draft_len;
-        verify_tail(p.tail, io, p.st, b, tsh);
-    } else if (threadIdx.x == 0) {
-        int w = K_t;
-        for (int j = 0; j < K_t; ++j) {
-            if (__ldcg(p.sc.van_flag + (size_t)b * Kmax + j) == 0) {
-                w = j;
-                break;
-            }
-        }
-        p.accept_len[b] = w;
-        p.next_token[b] = __ldcg(p.sc.van_tok + (size_t)b * (Kmax + 1) + w);
-    }
+    p.accept_len[b] = w;
+    p.next_token[b] = __ldcg(p.sc.van_tok + (size_t)b * (Kmax + 1) + w);
 }
 
 // ------------------------------------------------------------------------------------

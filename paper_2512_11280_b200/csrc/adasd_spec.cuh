@@ -1,5 +1,4 @@
-// Warp-specialised verification kernel for sm_100a (AdaSD mode and vanilla speculative
-// sampling mode).
+// Warp-specialised verification kernel for sm_100a (adasd_verify on 16-byte aligned bf16 rows).
 //
 // Persistent thread-block clusters; a position (b,i) = target row p_i + draft row q_i (bf16).
 // The CTAs of a cluster split both rows into contiguous slices, the compute warps of a CTA
@@ -16,20 +15,17 @@
 //
 //  * 12 COMPUTE warps per CTA (three per scheduler) do nothing but the passes over their share of a position
 //    (A: maxima and flags; B: 2^t, S = sum 2^t, T = sum 2^t t and the largest |z_t - z_d|;
-//    C: (p+q) log2 (p+q) in AdaSD mode - or, when the two rows are nearly equal everywhere, the
-//    well-conditioned sum of (p+q) phi((q-p)/(q+p)) - and the residual mass max(0, p - q) of a
-//    rejected row in vanilla mode), the refill of their own buffers and, for the one warp that
+//    C: (p+q) log2 (p+q) - or, when the two rows are nearly equal everywhere, the
+//    well-conditioned sum of (p+q) phi((q-p)/(q+p))), the refill of their own buffers and, for the one warp that
 //    holds it, the inverse-CDF crossing.  Per position: A(n+1), head of B(n+1) | wait for the
 //    scale factors of n | C(n) | tail of B(n+1), publish its partials, refill.
 //  * 1 CONTROL warp per CTA finds the cluster's positions, folds the warp partials into the
 //    CTA's totals, exchanges them with the other CTAs of the cluster (st.async into their
 //    shared memory, counted on their mbarriers: no cluster-wide barrier in the loop) and
-//    turns the row totals into two small messages per compute warp: its scale factors (and,
-//    vanilla, whether the row was accepted), then whether it holds the inverse-CDF crossing.
-//  * 1 TAIL warp (leader CTA) finalises each position once the compute warps' sums are in,
-//    draws the sequence's ticket and runs the tails (KDE/Bayes, accept scan, list appends,
-//    T_G; vanilla: longest accepted prefix) of completed sequences, off everybody's critical
-//    path; AdaSD tails are handed to the idle tail warps of the cluster's other CTAs.
+//    turns the row totals into two small messages per compute warp: its scale factors,
+//    then whether it holds the inverse-CDF crossing.
+//  * 1 TAIL warp (leader CTA) finalises each position once the compute warps' sums are in.
+// The tail of a sequence (KDE/Bayes, accept scan, appends, T_G) is verify_tail_kernel.
 //
 // The CTA has 16 warps of 128 registers per thread: the whole register file (136 per compute
 // thread and 104 per service thread after setmaxnreg).
@@ -82,8 +78,7 @@ struct __align__(16) PosCtx {
 // holds the inverse-CDF crossing (sel), the weight before its share and the target.
 struct __align__(16) WarpMsg {
     float at, ad, ft;             // first part: ready when scal_bar completes
-    int32_t act;                  // vanilla: 0 nothing left to do, 1 sample from p, 2 residual pass;
-                                  // AdaSD: 1, plus 4 when the rows are nearly equal (pass C in its u form)
+    int32_t act;                  // 1, plus 4 when the rows are nearly equal (pass C in its u form)
     float target;                 // second part: ready when sel_bar completes
     int32_t sel;
     float base;
@@ -99,20 +94,15 @@ struct __align__(16) SpecShared {
     float fin[kSFinRing][12];         // leader: row totals (and alpha, accept flag) kept for finalisation
     RowPart finc[kSFinRing][kCMaxCluster];   // leader: every CTA's totals, kept for the float64 finalisation
     uint32_t tmem_base;               // tensor-memory address the allocation returned
-    float rw[kCW];                    // vanilla: residual mass of each compute warp's share
-    float4 rtab[kCMaxCluster];        // vanilla: every CTA's residual mass (written over DSMEM)
     unsigned long long entry_bar[2];  // one arrival per compute warp: wtab[par] complete
     unsigned long long ctab_bar[2];   // CS * 32 bytes from the control warps of the cluster: ctab[par] complete
     unsigned long long scal_bar[2];   // 1 arrival: first part of wmsg[par] ready
     unsigned long long sel_bar[2];    // 1 arrival: second part of wmsg[par] ready
     unsigned long long c_bar[kSFinRing];   // leader: 16 bytes from every compute warp of the cluster: tabC complete
-    unsigned long long resid_bar;     // vanilla: one arrival per compute warp: rw complete
-    unsigned long long r_bar;         // vanilla: CS * 16 bytes from the control warps of the cluster: rtab complete
     unsigned long long bar[kCW][2];   // per compute warp: "position buffer filled" barriers
     int32_t n_issued;                 // leader: positions whose messages have been sent
     int32_t n_final;                  // leader: number of positions of this cluster, -1 until known
     int32_t fin_done;                 // leader: positions finalised so far (written by the tail warp)
-    float td[3][ADASD_KMAX_LIMIT], tH[3][ADASD_KMAX_LIMIT];   // scratch of the three tail workers of a CTA
 };
 
 __device__ __forceinline__ void st_cluster_u32(uint32_t remote_addr, uint32_t v) {
@@ -222,150 +212,9 @@ __device__ __forceinline__ FinOut finalize_math(const RowPart* finc, int CS, flo
     return o;
 }
 
-// The per-sequence tail of a round, run by ONE warp: lane i owns candidate i.  Same
-// arithmetic as verify_tail (KDE sums over L_D^A and L_D^R, Bayes posterior with the
-// round's earlier distances counted as accepted, first-rejection scan, appends, T_G).
-// sd/sH: 32-entry shared-memory scratch of this warp.
-__device__ __forceinline__ void verify_tail_warp(const TailConfig& cfg, const TailIO& io, State& st, int b,
-                                                 float* sd, float* sH) {
-    const int lane = threadIdx.x & 31;
-    const int Kmax = cfg.Kmax;
-    int K_t = io.draft_len ? __ldcg(io.draft_len + b) : Kmax;
-    K_t = max(0, min(K_t, Kmax));
-    float d = 0.f, H = 0.f, u = 0.f;
-    int x = 0, y = 0;
-    if (lane < K_t) {
-        d = __ldcg(io.dist + (size_t)b * Kmax + lane);
-        H = __ldcg(io.H_d + (size_t)b * Kmax + lane);
-        y = __ldcg(io.y + (size_t)b * (Kmax + 1) + lane);
-        x = io.x[(size_t)b * Kmax + lane];
-        u = io.u_accept[(size_t)b * Kmax + lane];
-        sd[lane] = d;
-        sH[lane] = H;
-    }
-    __syncwarp();
-    const int nA0 = st.nA[b], nR0 = st.nR[b];
-    const bool inside = d > 0.f && d < 1.f;          // enters the KDE lists when accepted
-
-    // bandwidths: candidate i sees L_D^A plus the distances d_1..d_{i-1} of this round that
-    // lie strictly inside (0,1): the list "as it stands" when candidate i is reached at all
-    double n = (double)nA0, s = st.sumA[b], s2 = st.sumA2[b];
-    for (int j = 0; j < K_t; ++j) {
-        const float dj = __shfl_sync(0xFFFFFFFFu, d, j);
-        if (j < lane && dj > 0.f && dj < 1.f) {
-            n += 1.0;
-            s += (double)dj;
-            s2 += (double)dj * (double)dj;
-        }
-    }
-    const double hA = kde_bandwidth(n, s, s2, cfg.bw_rule);
-    const bool ok = lane < K_t && (n >= (double)cfg.min_samples) && (hA > 0.0);
-    const float cA = ok ? (float)(-0.5 * 1.4426950408889634 / (hA * hA)) : 0.f;
-    const float ihA = ok ? (float)(1.0 / hA) : 0.f;
-    const double hR = kde_bandwidth((double)nR0, st.sumR[b], st.sumR2[b], cfg.bw_rule);
-    const bool validR = (nR0 >= cfg.min_samples) && (hR > 0.0);
-    const float cR = validR ? (float)(-0.5 * 1.4426950408889634 / (hR * hR)) : 0.f;
-    const float ihR = validR ? (float)(1.0 / hR) : 0.f;
-    const bool any_valid = (__ballot_sync(0xFFFFFFFFu, ok) != 0u) && validR;
-
-    float SA = 0.f, SR = 0.f;
-    if (any_valid) {
-        const float* LA = st.LA + (size_t)b * st.cap;
-        const float* LR = st.LR + (size_t)b * st.cap;
-        for (int i0 = 0; i0 < K_t; i0 += 8) {
-            float accA[8], accR[8], di[8], ci[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int i = min(i0 + k, K_t - 1);
-                accA[k] = accR[k] = 0.f;
-                di[k] = __shfl_sync(0xFFFFFFFFu, d, i);
-                ci[k] = __shfl_sync(0xFFFFFFFFu, cA, i);
-            }
-            // four list entries per lane and trip, all four loads in flight together (the lists live
-            // in L2 / HBM: one load per trip would leave the warp waiting on memory, not on the
-            // special-function pipe); entries past the end sit far away, where the kernel is 0
-            for (int j0 = 0; j0 < nA0; j0 += 128) {
-                float xj[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int j = j0 + 32 * q + lane;
-                    xj[q] = j < nA0 ? __ldcg(LA + j) : 1.0e9f;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const float t = di[k] - xj[q];
-                        accA[k] += ex2(ci[k] * t * t);
-                    }
-                }
-            }
-            for (int j0 = 0; j0 < nR0; j0 += 128) {
-                float xj[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int j = j0 + 32 * q + lane;
-                    xj[q] = j < nR0 ? __ldcg(LR + j) : 1.0e9f;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const float t = di[k] - xj[q];
-                        accR[k] += ex2(cR * t * t);
-                    }
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const float a = warp_sum(accA[k]), r = warp_sum(accR[k]);
-                if (lane == i0 + k) {
-                    SA = a;
-                    SR = r;
-                }
-            }
-        }
-    }
-    // kernel terms of this round's earlier distances, then the posterior
-    float extra = 0.f;
-    for (int j = 0; j < K_t; ++j) {
-        const float dj = __shfl_sync(0xFFFFFFFFu, d, j);
-        if (j < lane && dj > 0.f && dj < 1.f) {
-            const float t = d - dj;
-            extra += ex2(cA * t * t);
-        }
-    }
-    float P = 0.f;
-    if (any_valid && ok) {
-        // n_A f_A = SA / (h_A sqrt(2 pi)),  n_R f_R = SR / (h_R sqrt(2 pi))
-        const float a = (SA + extra) * ihA;
-        const float r = SR * ihR;
-        const float den = a + r;
-        if (den > 0.f && den < INFINITY) P = a / den;
-    }
-    if (lane < K_t) {
-        io.p_acc[(size_t)b * Kmax + lane] = P;
-        if (io.p_acc_user) io.p_acc_user[(size_t)b * Kmax + lane] = P;
-    }
-    const bool rej = cfg.reject_rule == 0 ? (u >= P) : (P < 0.5f);
-    const unsigned m = __ballot_sync(0xFFFFFFFFu, lane < K_t && x != y && rej);
-    (void)inside;
-    if (lane == 0) {
-        const int w = m ? (__ffs(m) - 1) : K_t;
-        const bool rejected = (m != 0u);
-        io.accept_len[b] = w;
-        io.next_token[b] = __ldcg(io.y + (size_t)b * (Kmax + 1) + w);
-        if (io.accept_len_rec) io.accept_len_rec[b] = w;
-        if (io.rejected_rec) io.rejected_rec[b] = rejected ? 1 : 0;
-        if (io.draft_len_rec) io.draft_len_rec[b] = K_t;
-        if (cfg.update) apply_update(st, b, w, rejected, sd, sH);
-    }
-    __syncwarp();
-}
-
 // ------------------------------------------------------------------------------------
 // WARPED: an adjusted distribution is set (Sec. 2.1.1); the ordinary instantiation carries none of its code.
-template <int ITER, int MODE, bool WARPED = false>
+template <int ITER, bool WARPED = false>
 __global__ void __launch_bounds__(kSThreads, 1)
 spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
     const float c1 = WARPED ? p.c1 : kLog2e;                   // log2 e / temperature
@@ -406,12 +255,12 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
             mbar_init(reinterpret_cast<uint64_t*>(&sh.sel_bar[k]), 1);
         }
         for (int k = 0; k < kSFinRing; ++k) mbar_init(reinterpret_cast<uint64_t*>(&sh.c_bar[k]), 1);
-        mbar_init(reinterpret_cast<uint64_t*>(&sh.resid_bar), kSW);
-        mbar_init(reinterpret_cast<uint64_t*>(&sh.r_bar), 1);
     }
     if (warp < kSW && lane == 0)
         for (int s = 0; s < 2; ++s) mbar_init(reinterpret_cast<uint64_t*>(&sh.bar[warp][s]), 1);
     __syncthreads();
+    pdl_wait();
+    pdl_trigger();
 
     // first active position among start, start + ncl, ... (32 candidates per round)
     auto window = [&](int b) -> int {
@@ -902,51 +751,15 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
             float A = 0.f, PQ = 0.f;
             int tok = -1;
             const int act = __float_as_int(m0.w);
-            if (MODE == MODE_ADASD) {
-                if (!bonus) {
-                    if (act & 4) pass_c(std::true_type{}, n, m0.x, m0.y, A, PQ);
-                    else pass_c(std::false_type{}, n, m0.x, m0.y, A, PQ);
-                }
-                // y_i ~ p_i: the control warp says (a little later than the scale factors) whether
-                // this warp holds the crossing
-                wait_cta(&sh.sel_bar[par], ph);
-                const float4 m1 = *reinterpret_cast<const float4*>(&sh.wmsg[par][warp].target);   // target, sel, base
-                if (__float_as_int(m1.y) != 0) tok = select_kept(m1.z, m0.z, m1.x, vals_p);
-            } else {
-                // vanilla: an accepted row needs nothing more; the bonus row draws from p; a rejected
-                // row draws from the residual max(0, p - q) / R, whose mass this warp now adds up
-                const float at = m0.x, ad = m0.y;
-                auto vals_r = [&](int k, float(&v)[8]) {
-                    float a[8], d[8];
-                    load_kept(k, n, true, a, d);
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) v[j] = fmaxf(fmaf(a[j], at, -d[j] * ad), 0.f);
-                };
-                if (act == 2) {
-                    float r = 0.f;
-#pragma unroll
-                    for (int k = 0; k < ITER; ++k) {
-                        if (k_on(k)) {
-                            float v[8];
-                            vals_r(k, v);
-                            r += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
-                        }
-                    }
-                    r = warp_sum(r);
-                    if (lane == 0) {
-                        sh.rw[warp] = r;
-                        mbar_arrive_cta(reinterpret_cast<uint64_t*>(&sh.resid_bar));
-                    }
-                    __syncwarp();
-                }
-                if (act != 0) {
-                    wait_cta(&sh.sel_bar[par], ph);
-                    const float4 m1 = *reinterpret_cast<const float4*>(&sh.wmsg[par][warp].target);   // target, sel, base
-                    const int sel = __float_as_int(m1.y);
-                    if (sel == 1) tok = select_kept(m1.z, m0.z, m1.x, vals_p);
-                    else if (sel == 2) tok = select_kept(m1.z, 1.f, m1.x, vals_r);
-                }
+            if (!bonus) {
+                if (act & 4) pass_c(std::true_type{}, n, m0.x, m0.y, A, PQ);
+                else pass_c(std::false_type{}, n, m0.x, m0.y, A, PQ);
             }
+            // y_i ~ p_i: the control warp says (a little later than the scale factors) whether
+            // this warp holds the crossing
+            wait_cta(&sh.sel_bar[par], ph);
+            const float4 m1 = *reinterpret_cast<const float4*>(&sh.wmsg[par][warp].target);   // target, sel, base
+            if (__float_as_int(m1.y) != 0) tok = select_kept(m1.z, m0.z, m1.x, vals_p);
             // this warp's sums (and the token, if it drew it) go to the leader CTA in one message
             if (lane == 0) {
                 const int fr = n & (kSFinRing - 1);
@@ -980,7 +793,6 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
             return __shfl_sync(0xFFFFFFFFu, v, 0);
         };
         int n = 0;
-        uint32_t nres = 0;                        // residual exchanges so far (phase of their barriers)
         while (sh.pc[n & (kSPosRing - 1)].pos < total) {
             const int par = n & 1;
             const uint32_t ph = (uint32_t)(n >> 1) & 1u;
@@ -996,29 +808,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
             // per-position scalars, fetched before the wait so that they are there after it
             const PosCtx& pcn = sh.pc[n & (kSPosRing - 1)];
             const bool bonus = pcn.bonus != 0;
-            float u_samp, u_acc = 0.f, ztx = 0.f, zdx = 0.f;
-            bool x_ok = false;
-            if (MODE == MODE_ADASD) {
-                u_samp = __ldg(p.u_target + pcn.pos);
-            } else {
-                const int b = pcn.pos / K1, i = pcn.pos - b * K1;
-                u_samp = __ldg(p.u_resample + b);
-                if (!bonus) {
-                    const size_t idd = (size_t)b * Kmax + i;
-                    u_acc = __ldg(p.u_accept + idd);
-                    const int xi = __ldg(p.x + idd);
-                    x_ok = xi >= 0 && xi < p.V;
-                    if (x_ok) {
-                        ztx = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p.zt)[(long long)b * p.t_seq + (long long)i * p.t_row + xi]);
-                        zdx = __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p.zd)[(long long)b * p.d_seq + (long long)i * p.d_row + xi]);
-                        // a candidate below its row's cutoff has probability 0 there
-                        if (WARPED) {
-                            if (ztx < unpack2(pcn.cut_t).x) ztx = -INFINITY;
-                            if (zdx < unpack2(pcn.cut_d).x) zdx = -INFINITY;
-                        }
-                    }
-                }
-            }
+            const float u_samp = __ldg(p.u_target + pcn.pos);
 
             // the CTA's totals from its compute warps, sent to every CTA of the cluster
             wait_cta(&sh.entry_bar[par], ph);
@@ -1071,26 +861,11 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
             const float st_c = cft * e0.y;                    // CTA sums of the target row, scaled to Mt
             const float St = sum8(st_c), Sd = sum8(cfd * e1.x);
 
-            // vanilla: alpha = min(1, p(x) / q(x)) at the draft token, and what is left to do
             const uint32_t fl = __reduce_or_sync(0xFFFFFFFFu, __float_as_uint(e1.z));
             const bool bad = (fl & 1u) || !(Mt > kFloorL) || !(Md > kFloorL);
             // AdaSD: the two rows are nearly equal everywhere -> pass C in its well-conditioned form
-            const bool near = (MODE == MODE_ADASD) && !bonus && !bad && (fl & 2u) && warp_max_f32(e1.w) * inv_temp <= kSNearDz;
-            float alpha = 0.f;
-            bool van_accept = true;
-            int act = near ? 5 : 1;               // AdaSD: every row draws y_i ~ p_i
-            if (MODE == MODE_VANILLA) {
-                if (!bonus) {
-                    if (x_ok) {
-                        const float a = fmaf(fmaxf(ztx, ADASD_FLOOR_BF), c1, -Mt) - lg2(St);
-                        const float q = fmaf(fmaxf(zdx, ADASD_FLOOR_BF), c1, -Md) - lg2(Sd);
-                        alpha = fminf(1.f, ex2(a - q));
-                        if (!(ex2(q) > 0.f)) alpha = 1.f;   // q(x) = 0 cannot have been drafted
-                    }
-                    van_accept = u_acc < alpha;
-                }
-                act = bad ? 0 : (bonus ? 1 : (van_accept ? 0 : 2));
-            }
+            const bool near = !bonus && !bad && (fl & 2u) && warp_max_f32(e1.w) * inv_temp <= kSNearDz;
+            const int act = near ? 5 : 1;
 
             // first message per compute warp (lane w): its scale factors; pass C starts on it
             const float ftw = ex2(w0.x - Mt), fdw = ex2(w0.w - Md);
@@ -1150,26 +925,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
                     }
                 }
             };
-            bool from_p = ((act & 3) == 1);
-            if (MODE == MODE_VANILLA && act == 2) {
-                // residual mass: warp sums -> CTA sum -> every CTA of the cluster
-                const uint32_t rph = nres & 1u;
-                ++nres;
-                wait_cta(&sh.resid_bar, rph);
-                const float rwv = (lane < kSW) ? sh.rw[lane] : 0.f;
-                const float r_cta = warp_sum(rwv);
-                if (lane == 0) mbar_expect_tx(reinterpret_cast<uint64_t*>(&sh.r_bar), (uint32_t)(CS * 16));
-                __syncwarp();
-                if (lane < CS)
-                    st_async_v4(mapa_u32(&sh.rtab[rank], (uint32_t)lane), make_float4(r_cta, 0.f, 0.f, 0.f),
-                                mapa_u32(&sh.r_bar, (uint32_t)lane));
-                wait_cta(&sh.r_bar, rph);
-                const float rc = (lane < CS) ? sh.rtab[lane].x : 0.f;
-                const float R = sum8(rc);
-                if (R > 0.f && alive) locate(rc, rwv, u_samp * R, 2);
-                else from_p = true;               // no residual mass: draw from p
-            }
-            if (from_p && !bad) locate(st_c, ftw * w0.y, u_samp * St, 1);
+            if (!bad) locate(st_c, ftw * w0.y, u_samp * St, 1);
             if (lane < kSW)
                 *reinterpret_cast<float4*>(&sh.wmsg[par][lane].target) = make_float4(target, __int_as_float(sel), base, 0.f);
             if (leader && lane == 0) {
@@ -1181,8 +937,6 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
                 f[4] = Sd;
                 f[5] = Td;
                 f[6] = __uint_as_float(fl | (alive ? 0u : 1u));
-                f[7] = alpha;
-                f[8] = van_accept ? 1.f : 0.f;
                 f[9] = near ? 1.f : 0.f;
             }
             // every CTA's totals, for the finaliser's float64 combination
@@ -1210,23 +964,9 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
         // Leader CTA only: finalises every position of the cluster, in order, as soon as its sums
         // are in, and runs the tail of each sequence whose last position that was.
         if (leader) {
-            TailIO io;
-            io.H_d = p.sc.H_d;
-            io.dist = p.sc.dist;
-            io.y = p.sc.y;
-            io.x = p.x;
-            io.u_accept = p.u_accept;
-            io.draft_len = p.draft_len;
-            io.p_acc = p.sc.p_acc;
-            io.p_acc_user = p.user.p_acc;
-            io.accept_len = p.accept_len;
-            io.next_token = p.next_token;
-            io.accept_len_rec = p.user.accept_len;
-            io.rejected_rec = p.user.rejected;
-            io.draft_len_rec = p.user.draft_len;
             // leader: the published scalars of position number m, once every compute warp of the
             // cluster has sent its pass-C sums (they did before publishing their next partials)
-            auto finalize = [&](int m) -> int {
+            auto finalize = [&](int m) {
                 const int par = m & (kSFinRing - 1);
                 wait_cta(&sh.c_bar[par], (uint32_t)(m / kSFinRing) & 1u);
                 const float4 c0 = sh.tabC[par][4 * lane], c1 = sh.tabC[par][4 * lane + 1];
@@ -1239,11 +979,8 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
                 const int tok_all = __reduce_max_sync(0xFFFFFFFFu, max(max(__float_as_int(c0.z), __float_as_int(c1.z)),
                                                                        max(__float_as_int(c2.z), __float_as_int(c3.z))));
                 const float Mt = sh.fin[par][0], Md = sh.fin[par][3];
-                FinOut fo = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                if (MODE == MODE_ADASD)
-                    fo = finalize_math(&sh.finc[par][0], CS, Mt, Md, A, PQ, __float_as_uint(sh.fin[par][6]),
+                const FinOut fo = finalize_math(&sh.finc[par][0], CS, Mt, Md, A, PQ, __float_as_uint(sh.fin[par][6]),
                                        sh.fin[par][9] != 0.f);
-                int done_b = -1;
                 if (lane == 0) {
                     const PosCtx& c = sh.pc[m & (kSPosRing - 1)];
                     const int b = c.pos / K1, i = c.pos - b * K1;
@@ -1256,17 +993,8 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
                         atomicOr(p.st.status, ADASD_STATUS_NAN);
                         tok = -1;
                     }
-                    if (MODE == MODE_VANILLA) {
-                        if (!bonus) {
-                            p.sc.van_flag[idd] = (sh.fin[par][8] != 0.f && !bad) ? 1 : 0;
-                            if (p.alpha_out) p.alpha_out[idd] = bad ? NAN : sh.fin[par][7];
-                        }
-                        p.sc.van_tok[idt] = tok;
-                    } else {
                     float Ht = fo.Ht, lse_t = fo.lse_t;
                     if (bad) Ht = lse_t = NAN;
-                    p.sc.H_t[idt] = Ht;
-                    p.sc.lse_t[idt] = lse_t;
                     p.sc.y[idt] = tok;
                     if (p.user.H_t) p.user.H_t[idt] = Ht;
                     if (p.user.lse_t) p.user.lse_t[idt] = lse_t;
@@ -1275,34 +1003,12 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
                         float Hd = fo.Hd, lse_d = fo.lse_d, jsd = fo.jsd, dist = fo.dist;
                         if (bad) Hd = lse_d = jsd = dist = NAN;
                         p.sc.H_d[idd] = Hd;
-                        p.sc.lse_d[idd] = lse_d;
-                        p.sc.jsd[idd] = jsd;
                         p.sc.dist[idd] = dist;
                         if (p.user.H_d) p.user.H_d[idd] = Hd;
                         if (p.user.lse_d) p.user.lse_d[idd] = lse_d;
                         if (p.user.jsd) p.user.jsd[idd] = jsd;
                         if (p.user.dist) p.user.dist[idd] = dist;
                     }
-                    }
-                    __threadfence();
-                    const unsigned ticket = atomicAdd(p.sc.ticket + b, 1u);
-                    if (ticket == (unsigned)c.kt) {
-                        p.sc.ticket[b] = 0u;          // ready for the next round
-                        done_b = b;
-                    }
-                }
-                return __shfl_sync(0xFFFFFFFFu, done_b, 0);
-            };
-
-            // A completed sequence goes to the chip-wide queue of tails (device memory): whichever
-            // worker warp on the chip is free takes it.  (Handing the tails to this cluster's own
-            // workers would pile them up on the cluster that runs last, which draws most last tickets
-            // and would fall back further.)
-            auto push = [&](int b) {
-                if (lane == 0) {
-                    __threadfence();                      // this sequence's position scalars are out
-                    const uint32_t idx = atomicAdd(p.sc.q_ctl + 0, 1u);
-                    if (idx < (uint32_t)p.B) *reinterpret_cast<volatile int32_t*>(p.sc.q_items + idx) = b;
                 }
                 __syncwarp();
             };
@@ -1326,84 +1032,12 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
                 }
                 go = __shfl_sync(0xFFFFFFFFu, go, 0);
                 if (go <= 0) break;
-                const int done_b = finalize(m);
-                if (done_b >= 0) {
-                    if (MODE == MODE_VANILLA) {
-                        // longest accepted prefix, then the token drawn at the first rejection
-                        // (or the bonus token)
-                        __threadfence();
-                        const int kt = window(done_b);
-                        const bool rej = lane < kt && __ldcg(p.sc.van_flag + (size_t)done_b * Kmax + lane) == 0;
-                        const unsigned mr = __ballot_sync(0xFFFFFFFFu, rej);
-                        if (lane == 0) {
-                            const int w = mr ? (__ffs(mr) - 1) : kt;
-                            p.accept_len[done_b] = w;
-                            p.next_token[done_b] = __ldcg(p.sc.van_tok + (size_t)done_b * K1 + w);
-                        }
-                    } else {
-                        push(done_b);
-                    }
-                }
+                finalize(m);
                 if (lane == 0) {
                     __threadfence_block();
                     *reinterpret_cast<volatile int32_t*>(&sh.fin_done) = m + 1;
                 }
             }
-        }
-    }
-    // ============================== tail workers ==========================================
-    // AdaSD mode: the tail warps of the non-leader CTAs and the two spare warps of every CTA take
-    // completed sequences from the chip-wide queue and run their tails (KDE/Bayes, accept scan,
-    // appends, T_G).  Every sequence has a bonus row, so exactly B tails are queued per launch: a
-    // worker leaves when it draws a number >= B, and the last worker to leave puts the counters
-    // back to zero for the next launch.
-    if (MODE == MODE_ADASD && warp >= kSTail && !(leader && warp == kSTail)) {
-        TailIO io;
-        io.H_d = p.sc.H_d;
-        io.dist = p.sc.dist;
-        io.y = p.sc.y;
-        io.x = p.x;
-        io.u_accept = p.u_accept;
-        io.draft_len = p.draft_len;
-        io.p_acc = p.sc.p_acc;
-        io.p_acc_user = p.user.p_acc;
-        io.accept_len = p.accept_len;
-        io.next_token = p.next_token;
-        io.accept_len_rec = p.user.accept_len;
-        io.rejected_rec = p.user.rejected;
-        io.draft_len_rec = p.user.draft_len;
-        const int slot = warp - kSTail;           // this worker's scratch
-        const uint32_t nworkers = (uint32_t)(gridDim.x / CS) * (uint32_t)(3 * CS - 1);
-        for (;;) {
-            int b = -2;
-            if (lane == 0) {
-                const uint32_t idx = atomicAdd(p.sc.q_ctl + 1, 1u);
-                if (idx >= (uint32_t)p.B) {
-                    b = -1;                       // no more tails this launch
-                    if (atomicAdd(p.sc.q_ctl + 2, 1u) + 1u == nworkers) {
-                        p.sc.q_ctl[0] = 0u;       // every worker has left: ready for the next launch
-                        p.sc.q_ctl[1] = 0u;
-                        p.sc.q_ctl[2] = 0u;
-                    }
-                } else {
-                    volatile int32_t* item = p.sc.q_items + idx;
-                    for (uint32_t it = 0; it < kSPollSpins; ++it) {
-                        b = *item;
-                        if (b >= 0) break;
-                        __nanosleep(400);
-                    }
-                    if (b >= 0) *item = -1;       // the entry is free again
-                    else {
-                        b = -3;                   // nothing came: give this one up, go on
-                        atomicOr(p.st.status, ADASD_STATUS_TIMEOUT);
-                    }
-                }
-            }
-            b = __shfl_sync(0xFFFFFFFFu, b, 0);
-            if (b == -1) break;
-            if (b < 0) continue;
-            __threadfence();
-            verify_tail_warp(p.tail, io, p.st, b, sh.td[slot], sh.tH[slot]);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
