@@ -17,6 +17,7 @@
 #include "adasd_verify_tail.cuh"
 #include "adasd_draft_stream.cuh"
 #include "adasd_stream.cuh"
+#include "adasd_topk.cuh"
 #include "adasd_modes.cuh"
 
 using namespace adasd;
@@ -435,9 +436,9 @@ int fill_verify_params(adasd_ctx* ctx, VerifyParams& p, const void* zd, const vo
     return ADASD_OK;
 }
 
-// One cutoff logit per needed row (top-k / top-p of the adjusted distribution).
-int launch_cutoffs(adasd_ctx* ctx, const void* z, long long seq_stride, long long row_stride, int R, int extra,
-                   const int32_t* draft_len, const uint8_t* active, float* cut, cudaStream_t stream) {
+// One cutoff logit per needed row (top-k / top-p of the adjusted distribution) of one or two arrays of rows.
+CutParams cut_params(const adasd_ctx* ctx, const void* z, long long seq_stride, long long row_stride, int R, int extra,
+                     const int32_t* draft_len, const uint8_t* active, float* cut) {
     CutParams c;
     memset(&c, 0, sizeof(c));
     c.z = z;
@@ -454,33 +455,59 @@ int launch_cutoffs(adasd_ctx* ctx, const void* z, long long seq_stride, long lon
     c.c1 = 1.4426950408889634 / (double)ctx->temperature;
     c.top_k = ctx->top_k;
     c.top_p = ctx->top_p;
-    const long long rows = (long long)c.B * R;
-    const bool vec = vec_ok(z, ctx->cfg.dtype, {seq_stride, row_stride});
-    if (ctx->cfg.dtype == ADASD_BF16 && vec && ctx->cut_hist) {
-        // one pass per row over a histogram of the 65536 bf16 values; a row it cannot do (a value
-        // that occurs 65536 times or more) is left flagged for the radix kernel
-        const int g1 = (int)std::min<long long>(rows, (long long)ctx->sm_count);
-        row_cutoff_hist_kernel<<<g1, kHistThreads, kHistWords * 4, stream>>>(c);
-        CUDA_TRY(cudaGetLastError());
-        c.only_flagged = 1;
+    return c;
+}
+int launch_cutoffs(adasd_ctx* ctx, CutParams c, const CutParams* second, cudaStream_t stream) {
+    const bool bf = ctx->cfg.dtype == ADASD_BF16;
+    const bool vec1 = vec_ok(c.z, ctx->cfg.dtype, {c.seq_stride, c.row_stride});
+    const bool vec2 = !second || vec_ok(second->z, ctx->cfg.dtype, {second->seq_stride, second->row_stride});
+    CutParams c2 = second ? *second : c;
+    const long long rows = (long long)c.B * (c.R + (second ? second->R : 0));
+    const bool select = c.top_k > 0 && c.top_k < c.V && c.top_k <= kSelMaxK && c.V >= kSelMinV && rows <= 0x7FFFFFFF / kSelMaxP;
+    if (select) {
+        // top-k on: selection, a row over as many CTAs as are resident at once; it flags what it cannot do
+        int P = 1;
+        while (P < kSelMaxP && rows * P * 2 <= 3LL * ctx->sm_count) P *= 2;
+        const int g = (int)(rows * P);
+        const bool aligned = vec1 && vec2;
+        int rc;
+        if (bf)
+            rc = aligned ? launch_pdl(row_cutoff_select_kernel<__nv_bfloat16, true>, g, kSelThreads, 0, P, stream, c, c2)
+                         : launch_pdl(row_cutoff_select_kernel<__nv_bfloat16, false>, g, kSelThreads, 0, P, stream, c, c2);
+        else
+            rc = aligned ? launch_pdl(row_cutoff_select_kernel<float, true>, g, kSelThreads, 0, P, stream, c, c2)
+                         : launch_pdl(row_cutoff_select_kernel<float, false>, g, kSelThreads, 0, P, stream, c, c2);
+        if (rc != ADASD_OK) return rc;
     }
-    const int grid = (int)std::min<long long>(rows, 2LL * ctx->sm_count);
-    if (ctx->cfg.dtype == ADASD_BF16) {
-        if (vec) row_cutoff_kernel<__nv_bfloat16, true><<<grid, kCutThreads, 0, stream>>>(c);
-        else row_cutoff_kernel<__nv_bfloat16, false><<<grid, kCutThreads, 0, stream>>>(c);
-    } else {
-        if (vec) row_cutoff_kernel<float, true><<<grid, kCutThreads, 0, stream>>>(c);
-        else row_cutoff_kernel<float, false><<<grid, kCutThreads, 0, stream>>>(c);
+    for (int k = 0; k < (second ? 2 : 1); ++k) {
+        CutParams& q = k ? c2 : c;
+        const bool vec = k ? vec2 : vec1;
+        const long long n = (long long)q.B * q.R;
+        q.only_flagged = select ? 1 : 0;
+        if (!select && bf && vec && ctx->cut_hist) {
+            // one pass per row over a histogram of the 65536 bf16 values; a row it cannot do (a value
+            // that occurs 65536 times or more) is left flagged for the radix kernel
+            row_cutoff_hist_kernel<<<(unsigned)std::min<long long>(n, (long long)ctx->sm_count), kHistThreads, kHistWords * 4, stream>>>(q);
+            CUDA_TRY(cudaGetLastError());
+            q.only_flagged = 1;
+        }
+        const int grid = (int)std::min<long long>(n, 2LL * ctx->sm_count);
+        int rc;
+        if (bf)
+            rc = vec ? launch_pdl(row_cutoff_kernel<__nv_bfloat16, true>, grid, kCutThreads, 0, 0, stream, q)
+                     : launch_pdl(row_cutoff_kernel<__nv_bfloat16, false>, grid, kCutThreads, 0, 0, stream, q);
+        else
+            rc = vec ? launch_pdl(row_cutoff_kernel<float, true>, grid, kCutThreads, 0, 0, stream, q)
+                     : launch_pdl(row_cutoff_kernel<float, false>, grid, kCutThreads, 0, 0, stream, q);
+        if (rc != ADASD_OK) return rc;
     }
-    CUDA_TRY(cudaGetLastError());
     return ADASD_OK;
 }
-
 // ... of the rows of a verification round
 int launch_round_cutoffs(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
     if (!ctx->cuts_on()) return ADASD_OK;
-    if (int rc = launch_cutoffs(ctx, p.zt, p.t_seq, p.t_row, p.Kmax + 1, 1, p.draft_len, nullptr, ctx->cut_t, stream)) return rc;
-    return launch_cutoffs(ctx, p.zd, p.d_seq, p.d_row, p.Kmax, 0, p.draft_len, nullptr, ctx->cut_d, stream);
+    const CutParams d = cut_params(ctx, p.zd, p.d_seq, p.d_row, p.Kmax, 0, p.draft_len, nullptr, ctx->cut_d);
+    return launch_cutoffs(ctx, cut_params(ctx, p.zt, p.t_seq, p.t_row, p.Kmax + 1, 1, p.draft_len, nullptr, ctx->cut_t), &d, stream);
 }
 
 int launch_verify(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
@@ -719,7 +746,7 @@ static int draft_entropy_impl(adasd_ctx* ctx, const void* logits_dev, int64_t ro
         return ADASD_ERR_SHAPE;
     cudaStream_t st = (cudaStream_t)stream;
     if (ctx->cuts_on()) {
-        if (int rc = launch_cutoffs(ctx, logits_dev, row_stride, 0, 1, 1, nullptr, active_inout_dev, ctx->cut_row, st))
+        if (int rc = launch_cutoffs(ctx, cut_params(ctx, logits_dev, row_stride, 0, 1, 1, nullptr, active_inout_dev, ctx->cut_row), nullptr, st))
             return rc;
     }
     if (aligned && !p.argmax && draft_rows(ctx))

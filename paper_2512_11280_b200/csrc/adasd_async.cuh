@@ -1,17 +1,11 @@
 // Asynchronous building blocks for sm_100a shared by the streaming kernels: cluster-scope
-// mbarrier and st.async wrappers, tensor memory as a scratchpad, programmatic dependent launch.
+// mbarrier and st.async wrappers, tensor memory as a scratchpad, 16-byte units of a row.
 #pragma once
 
 #include "adasd_cluster.cuh"
+#include "adasd_pdl.cuh"
 
 namespace adasd {
-
-// ---- programmatic dependent launch -------------------------------------------------------
-// The launch ahead in the stream may still be running when a kernel launched with programmatic
-// stream serialisation starts: nothing that launch wrote may be read before pdl_wait().
-// pdl_trigger() lets the launch after this one become resident (it waits in its own pdl_wait()).
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---- mbarriers and DSMEM -----------------------------------------------------------------
 __device__ __forceinline__ void mbar_arrive_cta(uint64_t* bar) {

@@ -21,6 +21,7 @@
 #pragma once
 
 #include "adasd_device.cuh"
+#include "adasd_pdl.cuh"
 
 namespace adasd {
 
@@ -120,6 +121,8 @@ __global__ void __launch_bounds__(kCutThreads) row_cutoff_kernel(CutParams p) {
     const int total = p.B * p.R;
     const bool use_k = p.top_k > 0 && p.top_k < p.V;
     const bool use_p = p.top_p < 1.f;
+    pdl_wait();
+    if (p.only_flagged) pdl_trigger();                       // (usually nothing to do)
 
     for (int row = blockIdx.x; row < total; row += gridDim.x) {
         const int b = row / p.R, j = row - b * p.R;
