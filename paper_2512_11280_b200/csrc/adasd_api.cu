@@ -14,6 +14,7 @@
 #include "adasd_rows.cuh"
 #include "adasd_cluster.cuh"
 #include "adasd_spec.cuh"
+#include "adasd_sweep.cuh"
 #include "adasd_verify_tail.cuh"
 #include "adasd_draft_stream.cuh"
 #include "adasd_stream.cuh"
@@ -37,6 +38,7 @@ struct adasd_ctx {
     } fast;
     int draft_p, draft_nw, draft_it;      // draft step: CTAs per row, warps per CTA, iterations of a chunk
     bool draft_early;         // ... the next call's CTAs may be set up while one runs
+    SweepTables sweep;        // verification of other rows: tables, segments
     bool cut_hist;            // the one-pass cutoff kernel got its 128 KB of shared memory
     // adjusted distribution (adasd_set_warpers) and the per-row cutoffs a call works out
     float temperature;
@@ -510,19 +512,48 @@ int launch_round_cutoffs(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t str
     return launch_cutoffs(ctx, cut_params(ctx, p.zt, p.t_seq, p.t_row, p.Kmax + 1, 1, p.draft_len, nullptr, ctx->cut_t), &d, stream);
 }
 
+// ---- verification of rows the warp-specialised kernel does not take ---------------------------
+// Segments of a position: six items of either sweep for every warp of a grid that fills the chip while they
+// keep three 2 KB chunks a row, fewer chunks only where warps would have nothing to do.
+void sweep_setup(adasd_ctx* c) {
+    const int N = c->cfg.dtype == ADASD_BF16 ? 8 : 4;
+    const int NC = ((c->cfg.V + N - 1) / N + 32 * kSweepIt - 1) / (32 * kSweepIt);
+    const long long P = (long long)c->cfg.B * (c->cfg.Kmax + 1), warps = 2LL * c->sm_count * kSweepW;
+    int bits = 0;
+    while (bits < kSweepMaxBits && (P << (bits + 1)) < 0x40000000LL) {
+        const int next = NC >> (bits + 1);           // chunks of the next shorter segment (at least one)
+        if (!((next >= 3 && (P << bits) < 6 * warps) || (next >= 1 && (P << bits) < warps))) break;
+        ++bits;
+    }
+    c->sweep.bits = bits;
+}
+template <typename T, bool ALIGNED>
+cudaError_t sweep_prepare() {
+    cudaError_t e = cudaFuncSetAttribute(sweep_kernel<T, ALIGNED, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep_kernel<T, ALIGNED, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep_kernel<T, ALIGNED, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(sweep_kernel<T, ALIGNED, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSweepSmem);
+    return e;
+}
+template <typename T, bool ALIGNED, bool WARPED>
+int launch_sweep(adasd_ctx* c, const VerifyParams& p, cudaStream_t stream) {
+    const long long items = ((long long)p.B * (p.Kmax + 1)) << c->sweep.bits;
+    const int grid = (int)std::min<long long>((items + kSweepW - 1) / kSweepW, 2LL * c->sm_count);
+    if (int rc = launch_pdl(sweep_kernel<T, ALIGNED, WARPED, false>, grid, kSweepThreads, kSweepSmem, 0, stream, p, c->sweep)) return rc;
+    return launch_pdl(sweep_kernel<T, ALIGNED, WARPED, true>, grid, kSweepThreads, kSweepSmem, 0, stream, p, c->sweep);
+}
+template <typename T>
+int launch_sweep(adasd_ctx* c, const VerifyParams& p, bool aligned, cudaStream_t stream) {
+    if (aligned) return c->warp_on() ? launch_sweep<T, true, true>(c, p, stream) : launch_sweep<T, true, false>(c, p, stream);
+    return c->warp_on() ? launch_sweep<T, false, true>(c, p, stream) : launch_sweep<T, false, false>(c, p, stream);
+}
+
 int launch_verify(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
-    const long long positions = (long long)p.B * (p.Kmax + 1);
-    const int cs = pick_cluster(ctx, positions);
     const bool vec = vec_ok(p.zd, ctx->cfg.dtype, {p.d_seq, p.d_row}) &&
                      vec_ok(p.zt, ctx->cfg.dtype, {p.t_seq, p.t_row});
     if (int rc = launch_round_cutoffs(ctx, p, stream)) return rc;
     if (vec && ctx->fast.iter > 0) return fast_launch_iter(ctx, p, stream);
-    if (ctx->cfg.dtype == ADASD_BF16) {
-        return vec ? launch_cluster(verify_kernel<__nv_bfloat16, true, MODE_ADASD>, p, positions, cs, stream)
-                   : launch_cluster(verify_kernel<__nv_bfloat16, false, MODE_ADASD>, p, positions, cs, stream);
-    }
-    return vec ? launch_cluster(verify_kernel<float, true, MODE_ADASD>, p, positions, cs, stream)
-               : launch_cluster(verify_kernel<float, false, MODE_ADASD>, p, positions, cs, stream);
+    return ctx->cfg.dtype == ADASD_BF16 ? launch_sweep<__nv_bfloat16>(ctx, p, vec, stream) : launch_sweep<float>(ctx, p, vec, stream);
 }
 
 // CTAs per sequence of the tail kernel: a list entry costs every candidate one exponential, so a
@@ -656,6 +687,11 @@ int adasd_create(adasd_ctx** out, const adasd_config* cfg) {
     ALLOC(c->cut_d, B * K);
     ALLOC(c->cut_row, B);
     ALLOC(c->stream_next, 1);
+    sweep_setup(c);
+    ALLOC(c->sweep.seg1, (B * (K + 1)) << c->sweep.bits);
+    ALLOC(c->sweep.seg2, (B * (K + 1)) << c->sweep.bits);
+    ALLOC(c->sweep.done, B * (K + 1));
+    ALLOC(c->sweep.next, 2);
     stream_setup(c);
     ALLOC(c->seg, (B * (2 * K + 1)) << c->seg_bits);
 #undef ALLOC
@@ -673,6 +709,9 @@ int adasd_create(adasd_ctx** out, const adasd_config* cfg) {
         const cudaError_t e3 = cfg->dtype == ADASD_BF16 ? draft_prepare<__nv_bfloat16, true>(c) : draft_prepare<float, true>(c);
         const cudaError_t e4 = cfg->dtype == ADASD_BF16 ? draft_prepare<__nv_bfloat16, false>(c) : draft_prepare<float, false>(c);
         const cudaError_t e5 = c->draft_nw == kDW ? draft_rows_prepare<kDW>() : draft_rows_prepare<kDWBig>();
+        const cudaError_t e6 = cfg->dtype == ADASD_BF16 ? sweep_prepare<__nv_bfloat16, true>() : sweep_prepare<float, true>();
+        const cudaError_t e7 = cfg->dtype == ADASD_BF16 ? sweep_prepare<__nv_bfloat16, false>() : sweep_prepare<float, false>();
+        if (e6 != cudaSuccess || e7 != cudaSuccess) rc = ADASD_ERR_CUDA;
         if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess || e4 != cudaSuccess || e5 != cudaSuccess) rc = ADASD_ERR_CUDA;
     }
     if (rc == ADASD_OK && cudaDeviceSynchronize() != cudaSuccess) rc = ADASD_ERR_CUDA;

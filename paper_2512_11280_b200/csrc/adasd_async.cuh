@@ -101,10 +101,10 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
 // ---- 16-byte units of a logit row ----------------------------------------------------------
 // A row is cut into units of 16 bytes that are ALIGNED IN MEMORY, whatever the row's own address:
 // a row that starts m elements past a 16-byte boundary has unit u = its elements u N - m ..
-// u N - m + N - 1, and the elements before its start and past its end are masked.  Per type: N
-// elements a unit, packed maximum with NaN kept, the cut of an adjusted distribution, the largest
-// difference of two rows, unpacking to fp32 with -inf (and NaN) clamped to a finite floor (unpack_raw:
-// not clamped, for sums in which no product with a -inf occurs).
+// u N - m + N - 1, and the elements before its start and past its end read as -inf.  Per type: N
+// elements a unit, packed maximum with NaN kept, the cut of an adjusted distribution (to -inf), the range
+// of the difference of two rows, unpacking to fp32 with -inf (and NaN) clamped to a finite floor
+// (unpack_raw: not clamped, for sums in which no product with a -inf occurs).
 template <typename T>
 struct Unit;
 
@@ -124,32 +124,45 @@ struct Unit<__nv_bfloat16> {
     using Cut = uint32_t;
     static __device__ __forceinline__ Cut no_cut() { return kNoCut2; }
     static __device__ __forceinline__ Cut make_cut(float c) { return cut_pair(c); }
-    static __device__ __forceinline__ void cut(uint4& w, Cut c) { bcut8(w, c); }
-    static __device__ __forceinline__ uint4 floor4() { return make_uint4(0xF149F149u, 0xF149F149u, 0xF149F149u, 0xF149F149u); }
-    // elements outside [lo, hi) of the unit become the floor
+    static __device__ __forceinline__ uint32_t cut2(uint32_t a, uint32_t c) {
+        uint32_t m;
+        asm("set.lt.u32.bf16x2 %0, %1, %2;" : "=r"(m) : "r"(a), "r"(c));   // 0xFFFF per half that is below; a NaN is not
+        return (a & ~m) | (0xFF80FF80u & m);
+    }
+    static __device__ __forceinline__ void cut(uint4& w, Cut c) {
+        w = make_uint4(cut2(w.x, c), cut2(w.y, c), cut2(w.z, c), cut2(w.w, c));
+    }
+    static __device__ __forceinline__ uint4 none4() { return make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u); }
+    // elements outside [lo, hi) of the unit become -inf
     static __device__ __forceinline__ void mask(uint4& w, int lo, int hi) {
         uint32_t* p = &w.x;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (2 * j < lo || 2 * j >= hi) p[j] = (p[j] & 0xFFFF0000u) | 0xF149u;
-            if (2 * j + 1 < lo || 2 * j + 1 >= hi) p[j] = (p[j] & 0xFFFFu) | 0xF1490000u;
+            if (2 * j < lo || 2 * j >= hi) p[j] = (p[j] & 0xFFFF0000u) | 0xFF80u;
+            if (2 * j + 1 < lo || 2 * j + 1 >= hi) p[j] = (p[j] & 0xFFFFu) | 0xFF800000u;
         }
     }
-    using Diff = uint32_t;                    // packed pair of |differences|, rounded to bf16 (0 only for equal values)
-    static __device__ __forceinline__ Diff diff0() { return 0u; }
-    static __device__ __forceinline__ uint32_t dmax(uint32_t m, uint32_t a, uint32_t b) {
-        uint32_t d, r;
+    // largest and smallest z_t - z_d, packed pairs rounded to bf16 (0 only for equal values); tokens that
+    // both rows exclude (-inf - -inf) do not count
+    struct Diff {
+        uint32_t hi, lo;
+    };
+    static __device__ __forceinline__ Diff diff0() { return {0xFF80FF80u, 0x7F807F80u}; }
+    static __device__ __forceinline__ void diff2(Diff& m, uint32_t a, uint32_t b) {
+        uint32_t d;
         asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-        d &= 0x7FFF7FFFu;
-        asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(m), "r"(d));       // (-inf) - (-inf) is dropped
-        return r;
+        asm("max.bf16x2 %0, %1, %2;" : "=r"(m.hi) : "r"(m.hi), "r"(d));
+        asm("min.bf16x2 %0, %1, %2;" : "=r"(m.lo) : "r"(m.lo), "r"(d));
     }
     static __device__ __forceinline__ void diff_add(Diff& m, const uint4& a, const uint4& b) {
-        m = dmax(dmax(dmax(dmax(m, a.x, b.x), a.y, b.y), a.z, b.z), a.w, b.w);
+        diff2(m, a.x, b.x);
+        diff2(m, a.y, b.y);
+        diff2(m, a.z, b.z);
+        diff2(m, a.w, b.w);
     }
-    static __device__ __forceinline__ float diff_val(Diff m) {
-        const float2 v = unpack2(m);
-        return fmaxf(v.x, v.y);
+    static __device__ __forceinline__ float2 diff_val(const Diff& m) {      // (largest, smallest)
+        const float2 h = unpack2(m.hi), l = unpack2(m.lo);
+        return make_float2(fmaxf(h.x, h.y), fminf(l.x, l.y));
     }
     static __device__ __forceinline__ void unpack(const uint4& w, float2 (&z)[4]) {
         z[0] = unpack2(bclamp2(w.x));
@@ -196,30 +209,34 @@ struct Unit<float> {
     static __device__ __forceinline__ Cut no_cut() { return -INFINITY; }
     static __device__ __forceinline__ Cut make_cut(float c) { return c; }
     static __device__ __forceinline__ uint32_t cut1(uint32_t w, float c) {
-        return __uint_as_float(w) < c ? __float_as_uint(kFloor) : w;
+        return __uint_as_float(w) < c ? 0xFF800000u : w;
     }
     static __device__ __forceinline__ void cut(uint4& w, Cut c) {
         w = make_uint4(cut1(w.x, c), cut1(w.y, c), cut1(w.z, c), cut1(w.w, c));
     }
-    static __device__ __forceinline__ uint4 floor4() {
-        const uint32_t f = __float_as_uint(kFloor);
-        return make_uint4(f, f, f, f);
-    }
+    static __device__ __forceinline__ uint4 none4() { return make_uint4(0xFF800000u, 0xFF800000u, 0xFF800000u, 0xFF800000u); }
     static __device__ __forceinline__ void mask(uint4& w, int lo, int hi) {
         uint32_t* p = &w.x;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            if (j < lo || j >= hi) p[j] = __float_as_uint(kFloor);
+            if (j < lo || j >= hi) p[j] = 0xFF800000u;
     }
-    using Diff = float;
-    static __device__ __forceinline__ Diff diff0() { return 0.f; }
+    struct Diff {
+        float hi, lo;
+    };
+    static __device__ __forceinline__ Diff diff0() { return {-INFINITY, INFINITY}; }
+    static __device__ __forceinline__ void diff1(Diff& m, uint32_t a, uint32_t b) {
+        const float d = __uint_as_float(a) - __uint_as_float(b);
+        m.hi = fmaxf(m.hi, d);
+        m.lo = fminf(m.lo, d);
+    }
     static __device__ __forceinline__ void diff_add(Diff& m, const uint4& a, const uint4& b) {
-        m = fmaxf(m, fabsf(__uint_as_float(a.x) - __uint_as_float(b.x)));
-        m = fmaxf(m, fabsf(__uint_as_float(a.y) - __uint_as_float(b.y)));
-        m = fmaxf(m, fabsf(__uint_as_float(a.z) - __uint_as_float(b.z)));
-        m = fmaxf(m, fabsf(__uint_as_float(a.w) - __uint_as_float(b.w)));
+        diff1(m, a.x, b.x);
+        diff1(m, a.y, b.y);
+        diff1(m, a.z, b.z);
+        diff1(m, a.w, b.w);
     }
-    static __device__ __forceinline__ float diff_val(Diff m) { return m; }
+    static __device__ __forceinline__ float2 diff_val(const Diff& m) { return make_float2(m.hi, m.lo); }
     static __device__ __forceinline__ void unpack(const uint4& w, float2 (&z)[2]) {
         z[0] = make_float2(fmaxf(__uint_as_float(w.x), kFloor), fmaxf(__uint_as_float(w.y), kFloor));
         z[1] = make_float2(fmaxf(__uint_as_float(w.z), kFloor), fmaxf(__uint_as_float(w.w), kFloor));

@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
         };
         auto mask = [&](uint4& w, int k) {                  // the row's end
             const int e0 = (32 * (ci + k) + lane) * N;
-            if (e0 >= p.V) w = U::floor4();
+            if (e0 >= p.V) w = U::none4();
             else if (e0 + N > p.V) U::mask(w, 0, p.V - e0);
         };
         const bool edge = ch0 + c == NC - 1;
@@ -302,13 +302,13 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
             uint4 W[IT + 1];
 #pragma unroll
             for (int k = 0; k < IT + (ALIGNED ? 0 : 1); ++k)
-                W[k] = ub + k < g1 ? __ldg(row + ub + k) : U::floor4();
+                W[k] = ub + k < g1 ? __ldg(row + ub + k) : U::none4();
             float e[IT][N], ls = 0.f;
 #pragma unroll
             for (int k = 0; k < IT; ++k) {
                 uint4 w = ALIGNED ? W[k] : U::realign(W[k], W[k + 1], shift);
                 const int el = (ub + k) * N;
-                if (el >= p.V) w = U::floor4();
+                if (el >= p.V) w = U::none4();
                 else if (el + N > p.V) U::mask(w, 0, p.V - el);
                 if (WARPED) U::cut(w, cut);
                 float2 z[NP];

@@ -450,8 +450,8 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
     };
     const Row row_t = row_of(rt + (long long)i * p.t_row), row_d = row_of(rd + (long long)min(i, K - 1) * p.d_row);
     auto load = [&](const Row& r, int u) -> uint4 {
-        uint4 w = u < r.g1 ? __ldg(r.base + u) : U::floor4();
-        if (!ALIGNED) w = U::realign(w, u + 1 < r.g1 ? __ldg(r.base + u + 1) : U::floor4(), r.shift);
+        uint4 w = u < r.g1 ? __ldg(r.base + u) : U::none4();
+        if (!ALIGNED) w = U::realign(w, u + 1 < r.g1 ? __ldg(r.base + u + 1) : U::none4(), r.shift);
         return w;
     };
     auto weights = [&](uint4 a, uint4 d, int u, float (&pv)[N], float (&rv)[N]) {
@@ -490,8 +490,8 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int u = 32 * (it + k) + lane;
-                a[k] = it + k < it1 ? load(row_t, u) : U::floor4();
-                d[k] = (it + k < it1 && !bonus) ? load(row_d, u) : U::floor4();
+                a[k] = it + k < it1 ? load(row_t, u) : U::none4();
+                d[k] = (it + k < it1 && !bonus) ? load(row_d, u) : U::none4();
             }
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -577,8 +577,8 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const int u = 32 * (it + k) + lane;
-                    a[k] = it + k < a1 ? load(row_t, u) : U::floor4();
-                    d[k] = (it + k < a1 && !bonus) ? load(row_d, u) : U::floor4();
+                    a[k] = it + k < a1 ? load(row_t, u) : U::none4();
+                    d[k] = (it + k < a1 && !bonus) ? load(row_d, u) : U::none4();
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
