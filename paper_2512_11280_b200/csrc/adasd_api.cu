@@ -513,19 +513,20 @@ int launch_round_cutoffs(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t str
 }
 
 // ---- verification of rows the warp-specialised kernel does not take ---------------------------
-// Segments of a position: six items of either sweep for every warp of a grid that fills the chip while they
-// keep three 2 KB chunks a row, fewer chunks only where warps would have nothing to do.
+// Segments of a position: as many as make the most loaded warp of a grid that fills the chip take the fewest
+// chunks, an item (its description, the folding of statistics, a drained ring) counting as two chunks more.
 void sweep_setup(adasd_ctx* c) {
     const int N = c->cfg.dtype == ADASD_BF16 ? 8 : 4;
     const int NC = ((c->cfg.V + N - 1) / N + 32 * kSweepIt - 1) / (32 * kSweepIt);
     const long long P = (long long)c->cfg.B * (c->cfg.Kmax + 1), warps = 2LL * c->sm_count * kSweepW;
-    int bits = 0;
-    while (bits < kSweepMaxBits && (P << (bits + 1)) < 0x40000000LL) {
-        const int next = NC >> (bits + 1);           // chunks of the next shorter segment (at least one)
-        if (!((next >= 3 && (P << bits) < 6 * warps) || (next >= 1 && (P << bits) < warps))) break;
-        ++bits;
+    long long best = 0;
+    for (int segs = 1; segs <= std::min(NC, kSweepMaxSegs) && P * segs < 0x40000000LL; ++segs) {
+        const long long load = ((P * segs + warps - 1) / warps) * ((NC + segs - 1) / segs + 2);
+        if (segs == 1 || load < best) {
+            best = load;
+            c->sweep.segs = segs;
+        }
     }
-    c->sweep.bits = bits;
 }
 template <typename T, bool ALIGNED>
 cudaError_t sweep_prepare() {
@@ -537,8 +538,8 @@ cudaError_t sweep_prepare() {
 }
 template <typename T, bool ALIGNED, bool WARPED>
 int launch_sweep(adasd_ctx* c, const VerifyParams& p, cudaStream_t stream) {
-    const long long items = ((long long)p.B * (p.Kmax + 1)) << c->sweep.bits;
-    const int grid = (int)std::min<long long>((items + kSweepW - 1) / kSweepW, 2LL * c->sm_count);
+    const long long items = (long long)p.B * (p.Kmax + 1) * c->sweep.segs;
+    const int grid = (int)std::min<long long>(items, 2LL * c->sm_count);
     if (int rc = launch_pdl(sweep_kernel<T, ALIGNED, WARPED, false>, grid, kSweepThreads, kSweepSmem, 0, stream, p, c->sweep)) return rc;
     return launch_pdl(sweep_kernel<T, ALIGNED, WARPED, true>, grid, kSweepThreads, kSweepSmem, 0, stream, p, c->sweep);
 }
@@ -688,8 +689,8 @@ int adasd_create(adasd_ctx** out, const adasd_config* cfg) {
     ALLOC(c->cut_row, B);
     ALLOC(c->stream_next, 1);
     sweep_setup(c);
-    ALLOC(c->sweep.seg1, (B * (K + 1)) << c->sweep.bits);
-    ALLOC(c->sweep.seg2, (B * (K + 1)) << c->sweep.bits);
+    ALLOC(c->sweep.seg1, B * (K + 1) * c->sweep.segs);
+    ALLOC(c->sweep.seg2, B * (K + 1) * c->sweep.segs);
     ALLOC(c->sweep.done, B * (K + 1));
     ALLOC(c->sweep.next, 2);
     stream_setup(c);

@@ -144,26 +144,6 @@ struct Unit<__nv_bfloat16> {
     }
     // largest and smallest z_t - z_d, packed pairs rounded to bf16 (0 only for equal values); tokens that
     // both rows exclude (-inf - -inf) do not count
-    struct Diff {
-        uint32_t hi, lo;
-    };
-    static __device__ __forceinline__ Diff diff0() { return {0xFF80FF80u, 0x7F807F80u}; }
-    static __device__ __forceinline__ void diff2(Diff& m, uint32_t a, uint32_t b) {
-        uint32_t d;
-        asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
-        asm("max.bf16x2 %0, %1, %2;" : "=r"(m.hi) : "r"(m.hi), "r"(d));
-        asm("min.bf16x2 %0, %1, %2;" : "=r"(m.lo) : "r"(m.lo), "r"(d));
-    }
-    static __device__ __forceinline__ void diff_add(Diff& m, const uint4& a, const uint4& b) {
-        diff2(m, a.x, b.x);
-        diff2(m, a.y, b.y);
-        diff2(m, a.z, b.z);
-        diff2(m, a.w, b.w);
-    }
-    static __device__ __forceinline__ float2 diff_val(const Diff& m) {      // (largest, smallest)
-        const float2 h = unpack2(m.hi), l = unpack2(m.lo);
-        return make_float2(fmaxf(h.x, h.y), fminf(l.x, l.y));
-    }
     static __device__ __forceinline__ void unpack(const uint4& w, float2 (&z)[4]) {
         z[0] = unpack2(bclamp2(w.x));
         z[1] = unpack2(bclamp2(w.y));
@@ -221,22 +201,6 @@ struct Unit<float> {
         for (int j = 0; j < 4; ++j)
             if (j < lo || j >= hi) p[j] = 0xFF800000u;
     }
-    struct Diff {
-        float hi, lo;
-    };
-    static __device__ __forceinline__ Diff diff0() { return {-INFINITY, INFINITY}; }
-    static __device__ __forceinline__ void diff1(Diff& m, uint32_t a, uint32_t b) {
-        const float d = __uint_as_float(a) - __uint_as_float(b);
-        m.hi = fmaxf(m.hi, d);
-        m.lo = fminf(m.lo, d);
-    }
-    static __device__ __forceinline__ void diff_add(Diff& m, const uint4& a, const uint4& b) {
-        diff1(m, a.x, b.x);
-        diff1(m, a.y, b.y);
-        diff1(m, a.z, b.z);
-        diff1(m, a.w, b.w);
-    }
-    static __device__ __forceinline__ float2 diff_val(const Diff& m) { return make_float2(m.hi, m.lo); }
     static __device__ __forceinline__ void unpack(const uint4& w, float2 (&z)[2]) {
         z[0] = make_float2(fmaxf(__uint_as_float(w.x), kFloor), fmaxf(__uint_as_float(w.y), kFloor));
         z[1] = make_float2(fmaxf(__uint_as_float(w.z), kFloor), fmaxf(__uint_as_float(w.w), kFloor));

@@ -4,13 +4,12 @@
 //
 // A position is swept twice, by two launches of sweep_kernel.  Sweep 1 forms 2^t, t = (z - max) log2 e, with a
 // running maximum and adds up S = sum 2^t and T = sum 2^t t of both rows; sweep 2, with the row totals known,
-// forms (p+q) log2 (p+q) - or, where the two rows are nearly equal everywhere, the well-conditioned
-// (p+q) phi((q-p)/(q+p)) - with p = 2^t_p / S_p, and scans for the token y_i ~ p_i.
+// forms the divergence from non-negative terms of p = 2^t_p / S_p and q, and scans for the token y_i ~ p_i.
 //
 // Either sweep of a position is cut into segments; a WARP takes a segment at a time (an "item"), its rows
 // coming through a ring of bulk copies that runs on across items.  The warps never meet: sweep 1 leaves every
 // segment's statistics in a table, a warp of sweep 2 folds those of its position when it takes the item on,
-// and the last warp of a position (a counter in device memory) publishes the position's scalars.  Nothing in
+// and the last warp of a position (a counter in device memory) publishes its distance.  Nothing in
 // a launch waits for anything but its own copies.
 //
 // What bounds them: sweep 1 HBM, sweep 2 L2 or HBM (fp32) and the special-function pipe (bf16), for few rows
@@ -31,25 +30,23 @@ constexpr int kSweepRing = 3;
 constexpr int kSweepRowB = kSweepIt * 512 + 16;  // one row's chunk (+ one unit: unaligned draft rows)
 constexpr int kSweepStage = 2 * kSweepRowB;
 constexpr int kSweepSmem = kSweepW * kSweepRing * kSweepStage;
-constexpr int kSweepMaxBits = 6;                 // 64 segments, two to a lane of the folding warp
+constexpr int kSweepMaxSegs = 64;                // segments of a position, two to a lane of the folding warp
 constexpr int kSweepItems = 8;                   // descriptions of items a warp keeps (it holds at most five)
-constexpr float kNearSpread = 1.f;               // rows count as nearly equal when no |ln(p / q)| can exceed it
 
 // Statistics of both rows over a segment: largest logits (kFloorL: none), S and T under them.
 struct __align__(16) SegStats {
     float vt, St, Tt, vd;
     float Sd, Td;
-    uint32_t flags;               // 1: NaN / +inf / expired wait, 2: the rows differ
-    uint32_t dz;                  // range of z_t - z_d over the tokens that either row has: bf16 (largest, smallest), rounded outwards
+    uint32_t bad;                 // 1: NaN / +inf / expired wait
+    uint32_t pad;
 };
-constexpr uint32_t kNoRange = 0xFF807F80u;       // an empty range of differences: (-inf, +inf)
 
 struct SweepTables {
     SegStats* seg1;               // [positions][segments]
-    float2* seg2;                 // [positions][segments] sweep-2 sums
+    float2* seg2;                 // [positions][segments] sweep-2 sums: of s phi(u), of 2^t_p 2^t_q
     uint32_t* done;               // [positions] items done of sweep 2 (0 between rounds)
     uint32_t* next;               // [2] items drawn so far by either sweep (0 before its launch)
-    int32_t bits;                 // 2^bits segments a position, at most one per chunk
+    int32_t segs;                 // segments of a position, each of one chunk or more
 };
 
 // An item as its warp describes it to itself when it asks for the first copy.
@@ -60,12 +57,8 @@ struct __align__(16) SweepItem {
     int32_t seg, ch0, ch1;        // segment, and its chunks
     int32_t bonus;                // the sequence's bonus row (target row only)
     float cut_t, cut_d;           // adjusted distribution: the rows' cutoff logits
-    // sweep 2: the position's totals
-    float vt, rt, vd, rd;         // row maxima, 1 / S
-    float base, target;           // this segment holds the crossing of u S: weight (under vt) before it, and where that lies
-    int32_t scan;                 // ... 1: it does
-    uint32_t flags;               // 2: the rows differ, 4: nearly equal
-    int32_t pad[3];
+    // sweep 2, bonus row: largest logit; this segment holds the crossing of u S: weight (under vt) before it, and where that lies
+    float vt, base, target;
 };
 // A warp's place among the items.
 struct __align__(16) SweepWarp {
@@ -84,16 +77,15 @@ struct ItemRows {
 
 // A position's totals from its segments, by a whole warp.
 struct PosTotals {
-    float vt, rt, vd, rd, base, target;
-    int32_t sel;                  // the segment with the crossing of u S, -1: none
-    uint32_t flags;               // 1: unusable, 2: the rows differ, 4: nearly equal
+    float vt, St, vd, Sd, base, target;
+    int32_t sel;                  // the segment with the crossing of u S, -1: the position is unusable
 };
 template <bool WARPED>
 __device__ __forceinline__ PosTotals fold_position(const VerifyParams& p, const SweepTables& q, int pos, float u) {
-    const int lane = threadIdx.x & 31, segs = 1 << q.bits;
+    const int lane = threadIdx.x & 31, segs = q.segs;
     const float c1 = WARPED ? p.c1 : kLog2e;
-    const float4* sp = reinterpret_cast<const float4*>(q.seg1 + ((size_t)pos << q.bits));
-    const float4 none0 = make_float4(kFloorL, 0.f, 0.f, kFloorL), none1 = make_float4(0.f, 0.f, 0.f, __uint_as_float(kNoRange));
+    const float4* sp = reinterpret_cast<const float4*>(q.seg1 + (size_t)pos * segs);
+    const float4 none0 = make_float4(kFloorL, 0.f, 0.f, kFloorL), none1 = make_float4(0.f, 0.f, 0.f, 0.f);
     const bool in0 = lane < segs, in1 = lane + 32 < segs;
     const float4 a0 = in0 ? __ldcg(sp + 2 * lane) : none0, a1 = in0 ? __ldcg(sp + 2 * lane + 1) : none1;
     const float4 b0 = in1 ? __ldcg(sp + 2 * (lane + 32)) : none0, b1 = in1 ? __ldcg(sp + 2 * (lane + 32) + 1) : none1;
@@ -101,38 +93,32 @@ __device__ __forceinline__ PosTotals fold_position(const VerifyParams& p, const 
     t.vt = warp_max_f32(fmaxf(a0.x, b0.x));
     t.vd = warp_max_f32(fmaxf(a0.w, b0.w));
     const float w0 = ex2((a0.x - t.vt) * c1) * a0.y, w1 = ex2((b0.x - t.vt) * c1) * b0.y;
-    const float St = warp_sum(w0 + w1);
-    const float Sd = warp_sum(ex2((a0.w - t.vd) * c1) * a1.x + ex2((b0.w - t.vd) * c1) * b1.x);
-    t.rt = __fdiv_rn(1.f, St);
-    t.rd = __fdiv_rn(1.f, Sd);
-    uint32_t fl = __reduce_or_sync(0xFFFFFFFFu, __float_as_uint(a1.z) | __float_as_uint(b1.z)) & 3u;
-    if (!(t.vt > kFloorL) || !(t.vd > kFloorL)) fl |= 1u;
-    // ln(p / q) = (z_t - z_d) / T - (lse_t - lse_d), and the difference of the log-sum-exps lies in the range of
-    // the logits' differences: the width of that range bounds every |ln(p / q)|
-    const float2 r0 = unpack2(__float_as_uint(a1.w)), r1 = unpack2(__float_as_uint(b1.w));       // (smallest, largest)
-    const float dhi = warp_max_f32(fmaxf(r0.y, r1.y)), dlo = -warp_max_f32(-fminf(r0.x, r1.x));
-    if (fl == 2u && (dhi - dlo) * (WARPED ? p.inv_temp : 1.f) <= kNearSpread) fl |= 4u;
-    t.flags = fl;
-    // the segment with the crossing of u S in index order; if rounding leaves none, the last with mass
+    const float wd = ex2((a0.w - t.vd) * c1) * a1.x + ex2((b0.w - t.vd) * c1) * b1.x;
+    const bool bad = __any_sync(0xFFFFFFFFu, (__float_as_uint(a1.z) | __float_as_uint(b1.z)) & 1u) || !(t.vt > kFloorL) || !(t.vd > kFloorL);
+    // running weights: lane by lane over the first 32 segments, then over the others
+    float i0 = w0, i1 = w1, Sd = wd;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const float t0 = __shfl_up_sync(0xFFFFFFFFu, i0, o), t1 = __shfl_up_sync(0xFFFFFFFFu, i1, o);
+        Sd += __shfl_xor_sync(0xFFFFFFFFu, Sd, o);
+        if (lane >= o) {
+            i0 += t0;
+            i1 += t1;
+        }
+    }
+    i1 += __shfl_sync(0xFFFFFFFFu, i0, 31);
+    t.St = __shfl_sync(0xFFFFFFFFu, i1, 31);
+    t.Sd = Sd;
     t.sel = -1;
     t.base = 0.f;
-    t.target = u * St;
-    if (!(fl & 1u)) {
-        float i0 = w0, i1 = w1;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float t0 = __shfl_up_sync(0xFFFFFFFFu, i0, o), t1 = __shfl_up_sync(0xFFFFFFFFu, i1, o);
-            if (lane >= o) {
-                i0 += t0;
-                i1 += t1;
-            }
-        }
-        i1 += __shfl_sync(0xFFFFFFFFu, i0, 31);
+    t.target = u * t.St;
+    if (!bad) {
+        // the segment with the crossing of u S in index order; if rounding leaves none, the last with mass
         const unsigned h0 = __ballot_sync(0xFFFFFFFFu, w0 > 0.f && i0 > t.target), h1 = __ballot_sync(0xFFFFFFFFu, w1 > 0.f && i1 > t.target);
-        const unsigned m0 = __ballot_sync(0xFFFFFFFFu, w0 > 0.f), m1 = __ballot_sync(0xFFFFFFFFu, w1 > 0.f);
         if (h0) t.sel = __ffs(h0) - 1;
         else if (h1) t.sel = 32 + __ffs(h1) - 1;
         else {
+            const unsigned m0 = __ballot_sync(0xFFFFFFFFu, w0 > 0.f), m1 = __ballot_sync(0xFFFFFFFFu, w1 > 0.f);
             t.sel = m1 ? 32 + 31 - __clz(m1) : 31 - __clz(m0);
             t.target = INFINITY;
         }
@@ -141,15 +127,13 @@ __device__ __forceinline__ PosTotals fold_position(const VerifyParams& p, const 
     return t;
 }
 
-// The scalars of one position, worked out in float64 by a whole warp: in fp32 the totals (entropies of up to
-// 17 bits, log2 of sums of up to 2^17) carry errors of about 1e-6 each, which the difference
-// H(m) - (H(p) + H(q)) / 2 keeps.  none: the position is unusable.
+// Entropies and log-sum-exps of one position, worked out in float64 by a whole warp (its first segment's).
+// none: the position is unusable.
 template <bool WARPED>
-__device__ __noinline__ void publish_position(const VerifyParams& p, const SweepTables& q, int pos, bool bonus, bool none, float vt, float vd,
-                                              uint32_t flags, double A, float PQ) {
-    const int lane = threadIdx.x & 31, segs = 1 << q.bits;
+__device__ __noinline__ void publish_entropies(const VerifyParams& p, const SweepTables& q, int pos, bool bonus, bool none, float vt, float vd) {
+    const int lane = threadIdx.x & 31, segs = q.segs;
     const double c1 = (double)(WARPED ? p.c1 : kLog2e);
-    const SegStats* const seg = q.seg1 + ((size_t)pos << q.bits);
+    const SegStats* const seg = q.seg1 + (size_t)pos * segs;
     // S = sum f_c S_c, T = sum f_c (T_c + d_c S_c) with d_c = (v_c - v) log2 e / T, f_c = 2^d_c
     double St = 0.0, Tt = 0.0, Sd = 0.0, Td = 0.0;
     for (int s = lane; s < segs; s += 32) {
@@ -169,29 +153,32 @@ __device__ __noinline__ void publish_position(const VerifyParams& p, const Sweep
     Tt = warp_sum_f64(Tt);
     Sd = warp_sum_f64(Sd);
     Td = warp_sum_f64(Td);
-    if (lane != 0) return;
-    const double kLn2d = 0.69314718055994530942;
-    const double lSt = log2(St), lSd = log2(Sd);
-    const double Hbt = lSt - Tt / St, Hbd = lSd - Td / Sd;      // entropies in bits
-    if (p.user.H_t) p.user.H_t[pos] = none ? NAN : (float)(kLn2d * Hbt);
-    if (p.user.lse_t) p.user.lse_t[pos] = none ? NAN : (float)(kLn2d * ((double)vt * c1 + lSt));
-    if (bonus) return;
-    // nearly equal rows: A is sum s phi(u), D_JS = A / 4 (nats), nothing cancels; else
-    // D_JS = H(m) - (H(p) + H(q)) / 2 with H(m) = (ln 2 / 2) (2 - sum s log2 s), s = p + q
-    const double jd = (flags & 4u) ? 0.25 * A : 0.5 * kLn2d * ((2.0 - A) - (Hbt + Hbd));
-    float jsd = (float)fmin(fmax(jd, 0.0), kLn2d);
-    if (!(flags & 2u)) jsd = 0.f;                               // identical rows: exactly 0
+    // lane 0: the target row, lane 1: the draft row
+    if (lane >= (bonus ? 1 : 2)) return;
+    const double kLn2d = 0.69314718055994530942, S = lane ? Sd : St, lS = log2(S);
+    const float H = none ? NAN : (float)(kLn2d * (lS - (lane ? Td : Tt) / S));
+    const float lse = none ? NAN : (float)(kLn2d * ((double)(lane ? vd : vt) * c1 + lS));
+    const size_t id = (size_t)(pos / (p.Kmax + 1)) * p.Kmax + pos % (p.Kmax + 1);
+    if (lane == 0) {
+        if (p.user.H_t) p.user.H_t[pos] = H;
+        if (p.user.lse_t) p.user.lse_t[pos] = lse;
+    } else {
+        p.sc.H_d[id] = H;
+        if (p.user.H_d) p.user.H_d[id] = H;
+        if (p.user.lse_d) p.user.lse_d[id] = lse;
+    }
+}
+
+// D_JS and the distance of one position, by one lane.  A: sum s phi(u), PQ: 0 where the supports are disjoint.
+__device__ __forceinline__ void publish_distance(const VerifyParams& p, int pos, bool none, double A, float PQ) {
+    float jsd = fminf((float)(0.25 * A), kLn2);
     if (!(PQ > 0.f)) jsd = kLn2;                                // disjoint supports: ln 2
-    float dist = jsd >= kLn2 ? 1.f : fminf((float)sqrt((double)jsd / kLn2d), 1.f);
-    float Hd = (float)(kLn2d * Hbd), lse_d = (float)(kLn2d * ((double)vd * c1 + lSd));
-    if (none) Hd = lse_d = jsd = dist = NAN;
-    const size_t idd = (size_t)(pos / (p.Kmax + 1)) * p.Kmax + pos % (p.Kmax + 1);
-    p.sc.H_d[idd] = Hd;
-    p.sc.dist[idd] = dist;
-    if (p.user.H_d) p.user.H_d[idd] = Hd;
-    if (p.user.lse_d) p.user.lse_d[idd] = lse_d;
-    if (p.user.jsd) p.user.jsd[idd] = jsd;
-    if (p.user.dist) p.user.dist[idd] = dist;
+    float dist = jsd >= kLn2 ? 1.f : fminf(sqrtf(jsd / kLn2), 1.f);
+    if (none) jsd = dist = NAN;
+    const size_t id = (size_t)(pos / (p.Kmax + 1)) * p.Kmax + pos % (p.Kmax + 1);
+    p.sc.dist[id] = dist;
+    if (p.user.jsd) p.user.jsd[id] = jsd;
+    if (p.user.dist) p.user.dist[id] = dist;
 }
 
 // Row sums of sweep 1 under the running maximum v (warp-wide; kFloorL: nothing finite so far).
@@ -223,52 +210,52 @@ struct RowSums {
     }
 };
 
-// Sweep-2 terms of one unit of both rows.
-// NEAR == false: A += (p+q) log2 (p+q), and the overlap indicator PQ += 2^t_p 2^t_q.
-// NEAR == true (|ln(p / q)| <= kNearSpread throughout): the divergence itself from non-negative terms,
-// D_JS = 1/4 sum s phi(u) with s = p + q, u = (q - p) / s and phi(u) = (1-u) ln(1-u) + (1+u) ln(1+u)
-// = u^2 + u^4/6 + u^6/15 + u^8/28 + u^10/45 + ...; |u| <= tanh(1/2) there, so five terms are good to 1e-5
-// of phi, and nothing cancels however close the rows are.
+// Sweep-2 terms of one unit of both rows: the overlap indicator PQ += 2^t_p 2^t_q, and the divergence from
+// non-negative terms, D_JS = 1/4 sum s phi(u) with s = p + q, u = |q - p| / s and
+// phi(u) = (1-u) ln(1-u) + (1+u) ln(1+u), which do not cancel however close the rows are:
+//   u < 1/2: u^2 + u^4/6 + u^6/15 + u^8/28 + u^10/45 (good to 1e-5 of phi there);
+//   else   : 2 ln(1+u) - (1-u) |ln(p / q)|, the logarithm of p / q from the logits and 1 - u = 2 min(p,q) / s.
+// Four special-function results a pair.
 struct PairConsts {
-    float2 nt2, nd2, at2, ad2, L2, tiny2;
+    float2 nt2, nd2, at2, ad2, L2;
+    float dl;                     // log2 (rd / rt): log2 (q / p) = t_q - t_p + dl
 };
-template <typename U, bool NEAR>
+template <typename U>
 __device__ __forceinline__ void pair_add(const uint4& Tw, const uint4& Dw, const PairConsts& c, float2& A2, float2& PQ2) {
     float2 z[U::N / 2], y[U::N / 2];
-    U::unpack(Tw, z);
-    U::unpack(Dw, y);
+    U::unpack_raw(Tw, z);
+    U::unpack_raw(Dw, y);
 #pragma unroll
     for (int j = 0; j < U::N / 2; ++j) {
         const float2 t = __fmul2_rn(__fadd2_rn(z[j], c.nt2), c.L2), r = __fmul2_rn(__fadd2_rn(y[j], c.nd2), c.L2);
         const float2 a = make_float2(ex2(t.x), ex2(t.y)), d = make_float2(ex2(r.x), ex2(r.y));
-        if (NEAR) {
-            const float2 pp = __fmul2_rn(a, c.at2), qq = __fmul2_rn(d, c.ad2);
-            const float2 ss = __fadd2_rn(__fadd2_rn(pp, c.tiny2), qq);
-            const float2 df = __ffma2_rn(pp, make_float2(-1.f, -1.f), qq);                // q - p
-            const float2 u = __fmul2_rn(df, make_float2(rcp_approx(ss.x), rcp_approx(ss.y)));
-            const float2 w = __fmul2_rn(u, u);
-            float2 f = __ffma2_rn(w, make_float2(1.f / 45.f, 1.f / 45.f), make_float2(1.f / 28.f, 1.f / 28.f));
-            f = __ffma2_rn(f, w, make_float2(1.f / 15.f, 1.f / 15.f));
-            f = __ffma2_rn(f, w, make_float2(1.f / 6.f, 1.f / 6.f));
-            f = __ffma2_rn(f, w, make_float2(1.f, 1.f));
-            A2 = __ffma2_rn(__fmul2_rn(ss, w), f, A2);
-        } else {
-            const float2 pp = __ffma2_rn(a, c.at2, c.tiny2);
-            const float2 ss = __ffma2_rn(d, c.ad2, pp);
-            A2 = __ffma2_rn(ss, make_float2(lg2(ss.x), lg2(ss.y)), A2);
-            PQ2 = __ffma2_rn(a, d, PQ2);
-        }
+        const float2 pp = __fmul2_rn(a, c.at2), qq = __fmul2_rn(d, c.ad2);
+        const float2 ss = __fadd2_rn(__fadd2_rn(pp, pair2(kTiny)), qq);
+        const float2 df = __ffma2_rn(pp, pair2(-1.f), qq);                                // q - p
+        const float2 rs = make_float2(rcp_approx(ss.x), rcp_approx(ss.y));
+        const float2 u = __fmul2_rn(df, rs), w = __fmul2_rn(u, u);
+        float2 f = __ffma2_rn(w, pair2(1.f / 45.f), pair2(1.f / 28.f));
+        f = __ffma2_rn(f, w, pair2(1.f / 15.f));
+        f = __ffma2_rn(f, w, pair2(1.f / 6.f));
+        f = __ffma2_rn(f, w, pair2(1.f));
+        f = __fmul2_rn(f, w);
+        // (fminf: the difference of two logits of -inf is NaN, and 0 times it has to be 0)
+        const float hx = fminf(pp.x, qq.x) * rs.x * fminf(fabsf(r.x - t.x + c.dl), 1e30f);
+        const float hy = fminf(pp.y, qq.y) * rs.y * fminf(fabsf(r.y - t.y + c.dl), 1e30f);
+        const float gx = 2.f * kLn2 * (lg2(1.f + fabsf(u.x)) - hx), gy = 2.f * kLn2 * (lg2(1.f + fabsf(u.y)) - hy);
+        A2 = __ffma2_rn(ss, make_float2(w.x < 0.25f ? f.x : gx, w.y < 0.25f ? f.y : gy), A2);
+        PQ2 = __ffma2_rn(a, d, PQ2);
     }
 }
 
 // Describes item number j (of P segs; position by position, sequence by sequence) to the warp, in sweep 2 the
-// next one that has something to do: the bonus row only needs the scan of one segment, an unusable position
-// only its outputs.  (A function of its own, like publish_position: the loops keep the registers.)
+// next one that has something to do: a bonus row only needs the scan of one segment.  (A function of its
+// own, like publish_entropies: the loops keep the registers.)
 template <typename T, bool ALIGNED, bool WARPED, bool SECOND>
 __device__ __noinline__ ItemRows sweep_item(const VerifyParams& p, const SweepTables& q, SweepWarp* w, uint32_t P, int NC, uint32_t j) {
     constexpr int N = Unit<T>::N;
     const int lane = threadIdx.x & 31, K = p.Kmax, K1 = K + 1;
-    const uint32_t segs = 1u << q.bits;
+    const uint32_t segs = (uint32_t)q.segs;
     SweepItem d;
     ItemRows r;
     d.pos = -1;
@@ -276,8 +263,8 @@ __device__ __noinline__ ItemRows sweep_item(const VerifyParams& p, const SweepTa
     r.glo = r.ghi = r.ch1 = 0;
     r.ch = -1;
     for (; j < P * segs;) {
-        const uint32_t rank = j >> q.bits;
-        const int seg = (int)(j & (segs - 1u));
+        const uint32_t rank = j / segs;
+        const int seg = (int)(j - rank * segs);
         int b, i;
         bool bonus;
         if (!p.draft_len) {
@@ -314,36 +301,32 @@ __device__ __noinline__ ItemRows sweep_item(const VerifyParams& p, const SweepTa
             bonus = i == n - 1;
         }
         const int pos = b * K1 + i;
-        if (SECOND) {
+        if (SECOND && bonus) {
+            pdl_wait();                              // (the warp's first item is described before the wait)
             const PosTotals t = fold_position<WARPED>(p, q, pos, __ldg(p.u_target + pos));
-            const bool none = (t.flags & 1u) != 0u;
-            if (seg == 0 && (none || bonus)) {
-                publish_position<WARPED>(p, q, pos, bonus, none, t.vt, t.vd, t.flags, 0.0, 1.f);
+            const bool none = t.sel < 0;
+            if (seg == 0) {
+                publish_entropies<WARPED>(p, q, pos, true, none, t.vt, t.vd);
                 if (none && lane == 0) {
                     atomicOr(p.st.status, ADASD_STATUS_NAN);
                     p.sc.y[pos] = -1;
                     if (p.user.y) p.user.y[pos] = -1;
                 }
             }
-            if (none || (bonus && t.sel != seg)) {
+            if (t.sel != seg) {
                 if (lane == 0) j = gridDim.x * kSweepW + atomicAdd(q.next + 1, 1u);
                 j = __shfl_sync(0xFFFFFFFFu, j, 0);
                 continue;
             }
             d.vt = t.vt;
-            d.rt = t.rt;
-            d.vd = t.vd;
-            d.rd = t.rd;
             d.base = t.base;
             d.target = t.target;
-            d.scan = t.sel == seg ? 1 : 0;
-            d.flags = t.flags;
         }
         d.pos = pos;
         d.seg = seg;
         d.bonus = bonus ? 1 : 0;
-        d.ch0 = (int)(((unsigned long long)seg * NC) >> q.bits);
-        d.ch1 = (int)(((unsigned long long)(seg + 1) * NC) >> q.bits);
+        d.ch0 = (int)((uint32_t)(seg * NC) / segs);
+        d.ch1 = (int)((uint32_t)((seg + 1) * NC) / segs);
         const unsigned long long at = reinterpret_cast<unsigned long long>(
             reinterpret_cast<const T*>(p.zt) + (long long)b * p.t_seq + (long long)i * p.t_row);
         const unsigned long long ad = reinterpret_cast<unsigned long long>(
@@ -385,10 +368,10 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int K = p.Kmax;
     const float c1 = WARPED ? p.c1 : kLog2e;         // log2 e / temperature
-    const uint32_t segs = 1u << q.bits;
     // chunks of a position (unaligned rows: one unit more, wherever the row starts)
     const int NC = ((ALIGNED ? (p.V + N - 1) / N : (p.V + 2 * N - 2) / N) + 32 * IT - 1) / (32 * IT);
-    const uint32_t GW = gridDim.x * kSweepW, gw = blockIdx.x * kSweepW + (uint32_t)warp;
+    // (few items: spread over the SMs)
+    const uint32_t GW = gridDim.x * kSweepW, gw = (uint32_t)warp * gridDim.x + blockIdx.x;
     unsigned char* const ring = dyn_smem + (size_t)warp * (kSweepRing * kSweepStage);
     SweepWarp* const sw = warps_s + warp;
     if (lane == 0) {
@@ -399,9 +382,10 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
-    pdl_wait();
-    pdl_trigger();
-    if (gw == 0 && lane == 0) q.next[SECOND ? 0 : 1] = 0u;       // the other sweep's counter, for its next launch
+    if (!SECOND) {
+        pdl_wait();
+        pdl_trigger();
+    }
     // active positions of the round (i <= K_b)
     uint32_t P = 0;
     if (p.draft_len) {
@@ -421,11 +405,10 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
     };
     ItemRows rows = sweep_item<T, ALIGNED, WARPED, SECOND>(p, q, sw, P, NC, gw);
     int is = 0, n_issued = 0, n_taken = 0;
-    auto issue = [&]() {                             // the next chunk
-        if (rows.ch < 0) return;
+    auto ask = [&](int ch) {                         // ring slot `is` gets a chunk of both rows
         if (lane < 2) {
             // (unaligned draft rows: one granule more)
-            const int u0 = 32 * IT * rows.ch, a = ALIGNED ? u0 : max(u0, rows.glo), e = min(u0 + 32 * IT + (ALIGNED ? 0 : lane), rows.ghi);
+            const int u0 = 32 * IT * ch, a = ALIGNED ? u0 : max(u0, rows.glo), e = min(u0 + 32 * IT + (ALIGNED ? 0 : lane), rows.ghi);
             const uint32_t bytes = (uint32_t)max(e - a, 0) * 16u;
             uint64_t* bar = reinterpret_cast<uint64_t*>(&sw->bar[is]);
             mbar_expect_tx(bar, bytes);
@@ -436,6 +419,10 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
         __syncwarp();
         ++n_issued;
         is = is + 1 == kSweepRing ? 0 : is + 1;
+    };
+    auto issue = [&](bool asked) {                   // the next chunk
+        if (rows.ch < 0) return;
+        if (!asked) ask(rows.ch);
         if (++rows.ch == rows.ch1) {
             if (!pending) draw();
             pending = false;
@@ -444,8 +431,18 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
             draw();
         }
     };
+    // Sweep 2 asks for its first copies before it waits for sweep 1: logits and window lengths were there
+    // before that one began.
+    int early = 0;
+    if (SECOND) {
 #pragma unroll 1
-    for (int k = 0; k < kSweepRing; ++k) issue();
+        for (; early < kSweepRing && rows.ch >= 0 && rows.ch + early < rows.ch1; ++early) ask(rows.ch + early);
+        pdl_wait();
+        pdl_trigger();
+    }
+    if (gw == 0 && lane == 0) q.next[SECOND ? 0 : 1] = 0u;       // the other sweep's counter, for its next launch
+#pragma unroll 1
+    for (int k = 0; k < kSweepRing; ++k) issue(k < early);
 
     int rs = 0;                                      // ring slot and phase of the next chunk to take
     uint32_t rph = 0;
@@ -495,7 +492,6 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
 
         if (!SECOND) {
             RowSums rt = {kFloorL, make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, rd = rt;
-            typename U::Diff dz = U::diff0();
             uint32_t bad = 0u;
             auto chunk = [&](auto bonus_c, auto edge_c, int ch, const unsigned char* sb) {
                 constexpr bool BONUS = decltype(bonus_c)::value, edge = decltype(edge_c)::value;
@@ -527,7 +523,6 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
                         uint4 Dw = unit_d(sb, k);
                         if (edge) mask(Dw, ch, k);
                         if (WARPED) U::cut(Dw, cut_d);
-                        U::diff_add(dz, Tw, Dw);
                         rd.add<U>(Dw, nd2, L2);
                     }
                 }
@@ -543,56 +538,92 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
                     else chunk(std::false_type{}, std::false_type{}, ch, sb);
                 }
                 __syncwarp();
-                issue();                             // the chunk has been read, its slot is free
+                issue(false);                        // the chunk has been read, its slot is free
             }
             if (!alive) bad = 1u;
             const float St = warp_sum(rt.S.x + rt.S.y), Tt = warp_sum(rt.T.x + rt.T.y);
             const float Sd = bonus ? St : warp_sum(rd.S.x + rd.S.y), Td = bonus ? Tt : warp_sum(rd.T.x + rd.T.y);
-            const float2 dv = U::diff_val(dz);
-            const float hi = warp_max_f32(dv.x), lo = -warp_max_f32(-dv.y);
-            if (hi > 0.f || lo < 0.f) bad |= 2u;
             bad = __reduce_or_sync(0xFFFFFFFFu, bad);
             if (lane == 0) {
-                const uint32_t z = ((uint32_t)__bfloat16_as_ushort(__float2bfloat16_ru(hi)) << 16) |
-                                   (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rd(lo));
-                float4* w = reinterpret_cast<float4*>(q.seg1 + ((size_t)pos << q.bits) + seg);
+                float4* w = reinterpret_cast<float4*>(q.seg1 + (size_t)pos * q.segs + seg);
                 __stcg(w, make_float4(rt.v, St, Tt, bonus ? rt.v : rd.v));
-                __stcg(w + 1, make_float4(Sd, Td, __uint_as_float(bad), __uint_as_float(z)));
+                __stcg(w + 1, make_float4(Sd, Td, __uint_as_float(bad), 0.f));
             }
             continue;
         }
 
         // ================================== sweep 2 =========================================
-        const float vt = c.vt, vd = c.vd, target = c.target;
-        const uint32_t flags = c.flags;
-        const bool scan = c.scan != 0, near = (flags & 4u) != 0u;
+        float vt, run, target;                       // scan: weight before the chunk, where the sample's crossing lies
+        bool scan = true, none = false;
         PairConsts pc;
-        pc.nt2 = pair2(-vt);
-        pc.nd2 = pair2(-vd);
-        pc.at2 = pair2(c.rt);
-        pc.ad2 = pair2(c.rd);
-        pc.L2 = L2;
-        pc.tiny2 = pair2(kTiny);
+        if (bonus) {
+            vt = c.vt;
+            run = c.base;
+            target = c.target;
+        } else {
+            const PosTotals t = fold_position<WARPED>(p, q, pos, __ldg(p.u_target + pos));
+            none = t.sel < 0;
+            vt = t.vt;
+            run = t.base;
+            target = t.target;
+            scan = t.sel == seg;
+            const float rt = __fdiv_rn(1.f, t.St), rd = __fdiv_rn(1.f, t.Sd);
+            pc.nt2 = pair2(-vt);
+            pc.nd2 = pair2(-t.vd);
+            pc.at2 = pair2(rt);
+            pc.ad2 = pair2(rd);
+            pc.L2 = L2;
+            pc.dl = lg2(t.St) - lg2(t.Sd);
+            if (seg == 0) {
+                publish_entropies<WARPED>(p, q, pos, false, none, vt, t.vd);
+                if (none && lane == 0) {
+                    publish_distance(p, pos, true, 0.0, 1.f);
+                    atomicOr(p.st.status, ADASD_STATUS_NAN);
+                    p.sc.y[pos] = -1;
+                    if (p.user.y) p.user.y[pos] = -1;
+                }
+            }
+        }
         float2 A2 = make_float2(0.f, 0.f), PQ2 = A2;
-        float run = c.base;                          // weight before the chunk, for the scan
         int tok = -1, last = -1;
         // y_i: the first element (index order) where the running weight exceeds the target, else the last
-        // one of the segment with weight
+        // one of the segment with weight.  A chunk's weight first, element by element only in the chunk that
+        // holds the crossing.
+        auto scan_unit = [&](const unsigned char* sb, int ch, int k, float (&e)[N]) {
+            uint4 w = unit_t(sb, k);
+            mask(w, ch, k);
+            if (WARPED) U::cut(w, cut_t);
+            float2 z[NP];
+            U::unpack_raw(w, z);
+#pragma unroll
+            for (int j = 0; j < NP; ++j) {
+                e[2 * j] = ex2((z[j].x - vt) * c1);
+                e[2 * j + 1] = ex2((z[j].y - vt) * c1);
+            }
+        };
         auto scan_chunk = [&](const unsigned char* sb, int ch) {
+            float tot = 0.f, e[N];
+#pragma unroll 1
+            for (int k = 0; k < IT; ++k) {
+                scan_unit(sb, ch, k, e);
+                const int e0 = (32 * (ch * IT + k) + lane) * N - mt;
+#pragma unroll
+                for (int j = 0; j < N; ++j) {
+                    tot += e[j];
+                    if (e[j] > 0.f) last = e0 + j;
+                }
+            }
+            tot = warp_sum(tot);
+            if (!(run + tot > target)) {
+                run += tot;
+                return;
+            }
 #pragma unroll 1
             for (int k = 0; k < IT && tok < 0; ++k) {
-                uint4 w = unit_t(sb, k);
-                mask(w, ch, k);
-                if (WARPED) U::cut(w, cut_t);
-                float2 z[NP];
-                U::unpack(w, z);
-                float e[N], s = 0.f;
+                scan_unit(sb, ch, k, e);
+                float s = 0.f;
 #pragma unroll
-                for (int j = 0; j < NP; ++j) {
-                    e[2 * j] = ex2((z[j].x - vt) * c1);
-                    e[2 * j + 1] = ex2((z[j].y - vt) * c1);
-                    s += e[2 * j] + e[2 * j + 1];
-                }
+                for (int j = 0; j < N; ++j) s += e[j];
                 float incl = s;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -605,18 +636,15 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
 #pragma unroll
                 for (int j = 0; j < N; ++j) {
                     cc += e[j];
-                    if (e[j] > 0.f) {
-                        last = e0 + j;
-                        if (hit < 0 && cc > target) hit = last;
-                    }
+                    if (e[j] > 0.f && hit < 0 && cc > target) hit = e0 + j;
                 }
                 const unsigned mh = __ballot_sync(0xFFFFFFFFu, hit >= 0);
                 if (mh) tok = __shfl_sync(0xFFFFFFFFu, hit, __ffs(mh) - 1);
                 run += __shfl_sync(0xFFFFFFFFu, incl, 31);
             }
         };
-        auto chunk = [&](auto near_c, auto edge_c, int ch, const unsigned char* sb) {
-            constexpr bool NEAR = decltype(near_c)::value, edge = decltype(edge_c)::value;
+        auto chunk = [&](auto edge_c, int ch, const unsigned char* sb) {
+            constexpr bool edge = decltype(edge_c)::value;
 #pragma unroll 2
             for (int k = 0; k < IT; ++k) {
                 uint4 Tw = unit_t(sb, k), Dw = unit_d(sb, k);
@@ -628,24 +656,19 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
                     U::cut(Tw, cut_t);
                     U::cut(Dw, cut_d);
                 }
-                pair_add<U, NEAR>(Tw, Dw, pc, A2, PQ2);
+                pair_add<U>(Tw, Dw, pc, A2, PQ2);
             }
         };
         for (int ch = ch0; ch < ch1 && alive; ++ch) {
             const unsigned char* sb = take();
             if (!alive) break;
             if (scan && tok < 0) scan_chunk(sb, ch);
-            if (!bonus) {
-                if (is_edge(ch)) {
-                    if (near) chunk(std::true_type{}, std::true_type{}, ch, sb);
-                    else chunk(std::false_type{}, std::true_type{}, ch, sb);
-                } else {
-                    if (near) chunk(std::true_type{}, std::false_type{}, ch, sb);
-                    else chunk(std::false_type{}, std::false_type{}, ch, sb);
-                }
+            if (!bonus && !none) {
+                if (is_edge(ch)) chunk(std::true_type{}, ch, sb);
+                else chunk(std::false_type{}, ch, sb);
             }
             __syncwarp();
-            issue();                                 // the chunk has been read, its slot is free
+            issue(false);                            // the chunk has been read, its slot is free
         }
         if (scan) {
             if (tok < 0) tok = __reduce_max_sync(0xFFFFFFFFu, last);
@@ -655,23 +678,24 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
                 if (p.user.y) p.user.y[pos] = tok;
             }
         }
-        if (bonus) continue;
-        const float A = warp_sum(A2.x + A2.y), PQ = near ? 1.f : warp_sum(PQ2.x + PQ2.y);
-        float2* const seg2 = q.seg2 + ((size_t)pos << q.bits);
+        if (bonus || none) continue;
+        const float A = warp_sum(A2.x + A2.y), PQ = warp_sum(PQ2.x + PQ2.y);
+        float2* const seg2 = q.seg2 + (size_t)pos * q.segs;
         uint32_t old = 0u;
         if (lane == 0) {
             __stcg(seg2 + seg, alive ? make_float2(A, PQ) : make_float2(NAN, 0.f));
             __threadfence();
             old = atomicAdd(q.done + pos, 1u);
         }
-        if (__shfl_sync(0xFFFFFFFFu, old, 0) + 1u != segs) continue;
+        if (__shfl_sync(0xFFFFFFFFu, old, 0) + 1u != (uint32_t)q.segs) continue;
         // the position's last segment
         __threadfence();
         if (lane == 0) q.done[pos] = 0u;             // ready for the next round
-        const float2 s0 = lane < (int)segs ? __ldcg(seg2 + lane) : make_float2(0.f, 0.f);
-        const float2 s1 = lane + 32 < (int)segs ? __ldcg(seg2 + lane + 32) : make_float2(0.f, 0.f);
+        const float2 s0 = lane < q.segs ? __ldcg(seg2 + lane) : make_float2(0.f, 0.f);
+        const float2 s1 = lane + 32 < q.segs ? __ldcg(seg2 + lane + 32) : make_float2(0.f, 0.f);
         const double At = warp_sum_f64((double)s0.x + (double)s1.x);
-        publish_position<WARPED>(p, q, pos, false, At != At, vt, vd, flags, At, warp_sum(s0.y + s1.y));
+        const float PQt = warp_sum(s0.y + s1.y);
+        if (lane == 0) publish_distance(p, pos, At != At, At, PQt);
         __syncwarp();
     }
     // a warp that gave up still waits (bounded) for whatever it had in flight
