@@ -240,7 +240,7 @@ int adasd_gen_only_update(adasd_ctx* ctx, const float* H_draft_dev, const int32_
  * token always stays.  adasd_vanilla_verify_static takes no context and applies none.
  *
  * Cost: temperature is a constant in the row passes.  With top-k or top-p on, each call first
- * finds one cutoff logit per row (row_cutoff_kernel: one more read of the rows), and the row
+ * finds one cutoff logit per row (one more read of the rows), and the row
  * passes read logits below it as -inf.  Rows without a usable maximum are not cut and are
  * reported by the row pass (ADASD_STATUS_NAN).
  * The values are read when a call is issued (or captured in a graph), not when it runs.

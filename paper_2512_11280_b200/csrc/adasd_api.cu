@@ -93,14 +93,6 @@ inline bool vec_ok(const void* base, int dtype, std::initializer_list<long long>
     return true;
 }
 
-int pick_cluster(const adasd_ctx* c, long long rows) {
-    if (c->cfg.cluster_size > 0) return c->cfg.cluster_size;
-    const long long want = 2LL * c->sm_count;
-    for (int cs = 1; cs <= kMaxCluster; cs *= 2)
-        if (rows * cs >= want) return cs;
-    return kMaxCluster;
-}
-
 template <typename P>
 int launch_cluster(void (*kernel)(P), const P& params, long long clusters, int cs,
                    cudaStream_t stream) {
@@ -1180,10 +1172,10 @@ int adasd_vanilla_verify_static(int32_t B, int32_t V, int32_t Kmax, int32_t dtyp
     const bool vec = vec_ok(draft_logits_dev, dtype, {d_seq_stride, d_row_stride}) &&
                      vec_ok(target_logits_dev, dtype, {t_seq_stride, t_row_stride});
     if (dtype == ADASD_BF16)
-        return vec ? launch_cluster(verify_kernel<__nv_bfloat16, true, MODE_VANILLA>, p, positions, cs, st)
-                   : launch_cluster(verify_kernel<__nv_bfloat16, false, MODE_VANILLA>, p, positions, cs, st);
-    return vec ? launch_cluster(verify_kernel<float, true, MODE_VANILLA>, p, positions, cs, st)
-               : launch_cluster(verify_kernel<float, false, MODE_VANILLA>, p, positions, cs, st);
+        return vec ? launch_cluster(static_vanilla_kernel<__nv_bfloat16, true>, p, positions, cs, st)
+                   : launch_cluster(static_vanilla_kernel<__nv_bfloat16, false>, p, positions, cs, st);
+    return vec ? launch_cluster(static_vanilla_kernel<float, true>, p, positions, cs, st)
+               : launch_cluster(static_vanilla_kernel<float, false>, p, positions, cs, st);
 }
 
 const char* adasd_strerror(int code) {

@@ -1,7 +1,6 @@
-// Generic row kernels: one thread-block cluster per logit row (draft step) or per
-// candidate position (verification).  Any V, any stride, bf16 or fp32; rows are read
-// from global memory once per pass (later passes hit L2).  These kernels are the
-// reference CUDA path and the fallback of the staged kernels.
+// Parameters of the row kernels, the kernel of the allocation-free vanilla verification (which has no context,
+// hence no tables: one thread-block cluster per candidate position, any V, any stride, bf16 or fp32, rows read
+// from global memory once per pass, the later passes from L2), and the small kernels of the state.
 #pragma once
 
 #include "adasd_device.cuh"
@@ -9,9 +8,6 @@
 #include "adasd_warp.cuh"
 
 namespace adasd {
-
-constexpr int MODE_ADASD = 0;
-constexpr int MODE_VANILLA = 1;
 
 struct Scratch {            // per-round scratch: the context's, or the fixed array of the allocation-free call
     float* H_d;             // [B,Kmax] entropies and distances of a round's candidates, for its tail
@@ -74,11 +70,10 @@ struct RowShared {
 };
 
 // ------------------------------------------------------------------------------------
-// Verification position (b,i): softmax statistics of q_i and p_i, H, D_JS, d_i, y_i ~ p_i
-// (AdaSD mode) or alpha_i and the residual sample (vanilla mode).
+// Vanilla verification of position (b,i): softmax statistics of q_i and p_i, alpha_i, the residual sample.
 // ------------------------------------------------------------------------------------
-template <typename T, bool VEC, int MODE>
-__global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
+template <typename T, bool VEC>
+__global__ void __launch_bounds__(kThreads) static_vanilla_kernel(VerifyParams p) {
     constexpr int N = Elt<T>::N;
     cg::cluster_group cluster = cg::this_cluster();
     const int CS = (int)cluster.num_blocks();
@@ -99,20 +94,17 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
     const T* rt = reinterpret_cast<const T*>(p.zt) + (long long)b * p.t_seq + (long long)i * p.t_row;
     const T* rd = bonus ? rt
                         : reinterpret_cast<const T*>(p.zd) + (long long)b * p.d_seq + (long long)i * p.d_row;
-    const RowWarp wt = {p.inv_temp, p.cut_t ? p.cut_t[(size_t)b * (Kmax + 1) + i] : -INFINITY};
-    const RowWarp wd = {p.inv_temp, (p.cut_d && !bonus) ? p.cut_d[(size_t)b * Kmax + i] : -INFINITY};
 
-    // pass A: maxima, NaN flag, "rows differ" flag
+    // pass A: maxima, NaN flag
     float vA[4] = {-INFINITY, -INFINITY, 0.f, 0.f};
     for (int u = u0 + lane; u < u1; u += 32) {
         float xt[N], xd[N];
-        load_unit_w<T, VEC>(rt, u, p.V, xt, wt);
-        if (!bonus) load_unit_w<T, VEC>(rd, u, p.V, xd, wd);
+        load_unit<T, VEC>(rt, u, p.V, xt);
+        if (!bonus) load_unit<T, VEC>(rd, u, p.V, xd);
 #pragma unroll
         for (int j = 0; j < N; ++j) {
             if (bonus) xd[j] = xt[j];
             vA[2] = (xt[j] != xt[j] || xd[j] != xd[j]) ? 1.f : vA[2];
-            vA[3] = (xt[j] != xd[j]) ? 1.f : vA[3];
             vA[0] = fmaxf(vA[0], xt[j]);
             vA[1] = fmaxf(vA[1], xd[j]);
         }
@@ -120,15 +112,14 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
     cluster_allreduce<4, true>(vA, sh.warp, sh.xA, CS, rank, cluster);
     const bool bad = (vA[2] > 0.f) || !(vA[0] > kFloor) || !(vA[1] > kFloor) ||
                      (vA[0] == INFINITY) || (vA[1] == INFINITY);
-    const bool differ = vA[3] > 0.f;
     const float mt = vA[0], md = vA[1];
 
     // pass B: S_t, S_d; per-warp S_t for sampling y_i
     float vB[2] = {0.f, 0.f};
     for (int u = u0 + lane; u < u1; u += 32) {
         float xt[N], xd[N];
-        load_unit_w<T, VEC>(rt, u, p.V, xt, wt);
-        if (!bonus) load_unit_w<T, VEC>(rd, u, p.V, xd, wd);
+        load_unit<T, VEC>(rt, u, p.V, xt);
+        if (!bonus) load_unit<T, VEC>(rd, u, p.V, xd);
 #pragma unroll
         for (int j = 0; j < N; ++j) {
             vB[0] += ex2((fmaxf(xt[j], kFloor) - mt) * kLog2e);
@@ -148,11 +139,11 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
     // vanilla: alpha_i at the draft token, known to every thread
     bool van_accept = true;
     float alpha = 1.f;
-    if (MODE == MODE_VANILLA && !bonus && !bad) {
+    if (!bonus && !bad) {
         const int xi = p.x[(size_t)b * Kmax + i];
         if (xi >= 0 && xi < p.V) {
-            float a = fmaf(fmaxf(apply_warp(to_f32(rt[xi]), wt), kFloor) - mt, kLog2e, -lSt);
-            float q = fmaf(fmaxf(apply_warp(to_f32(rd[xi]), wd), kFloor) - md, kLog2e, -lSd);
+            float a = fmaf(fmaxf(to_f32(rt[xi]), kFloor) - mt, kLog2e, -lSt);
+            float q = fmaf(fmaxf(to_f32(rd[xi]), kFloor) - md, kLog2e, -lSd);
             alpha = fminf(1.f, ex2(a - q));
             if (!(ex2(q) > 0.f)) alpha = 1.f;   // q(x) = 0 cannot have been drafted
         } else {
@@ -161,68 +152,34 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
         van_accept = p.u_accept[(size_t)b * Kmax + i] < alpha;
     }
 
-    // pass C: sum p a', sum q b' (entropies: a' = log2 p, b' = log2 q), sum p q (== 0 means disjoint
-    // supports, where D_JS is ln 2 exactly) and the divergence itself from non-negative terms,
-    //   D_JS = 1/4 sum s phi(u),  s = p + q,  u = (q - p) / s,  phi(u) = (1-u) ln(1-u) + (1+u) ln(1+u):
-    // for |u| < 1/2 the series u^2 + u^4/6 + u^6/15 + u^8/28 + u^10/45, else the two logarithms.
-    // Nothing cancels however close the rows are (Sec. 2.2, first printed form, term by term).
-    // vanilla on a rejected row: residual mass max(0, p - q), per warp and in total.
-    float vC[4] = {0.f, 0.f, 0.f, 0.f};
-    const bool need_resid = (MODE == MODE_VANILLA) && !bonus && !van_accept;
-    if (MODE == MODE_ADASD || need_resid) {
+    // pass C, on a rejected row: residual mass max(0, p - q), per warp and in total
+    float vC[2] = {0.f, 0.f};
+    const bool need_resid = !bonus && !van_accept;
+    if (need_resid) {
         for (int u = u0 + lane; u < u1; u += 32) {
             float xt[N], xd[N];
-            load_unit_w<T, VEC>(rt, u, p.V, xt, wt);
-            if (!bonus) load_unit_w<T, VEC>(rd, u, p.V, xd, wd);
+            load_unit<T, VEC>(rt, u, p.V, xt);
+            load_unit<T, VEC>(rd, u, p.V, xd);
 #pragma unroll
             for (int j = 0; j < N; ++j) {
-                float a = fmaf(fmaxf(xt[j], kFloor) - mt, kLog2e, -lSt);
-                float pp = ex2(a);
-                if (MODE == MODE_ADASD) vC[0] = fmaf(pp, a, vC[0]);
-                if (!bonus) {
-                    float bq = fmaf(fmaxf(xd[j], kFloor) - md, kLog2e, -lSd);
-                    float qq = ex2(bq);
-                    if (MODE == MODE_ADASD) {
-                        vC[1] = fmaf(qq, bq, vC[1]);
-                        const float s = pp + qq;
-                        if (s > 0.f) {
-                            const float rs = __fdividef(1.f, s), uu = (qq - pp) * rs, w = uu * uu;
-                            float ph;
-                            if (w < 0.25f) {
-                                ph = fmaf(w, 1.f / 45.f, 1.f / 28.f);
-                                ph = fmaf(ph, w, 1.f / 15.f);
-                                ph = fmaf(ph, w, 1.f / 6.f);
-                                ph = fmaf(ph, w, 1.f);
-                                ph *= w;
-                            } else {
-                                const float lo = 2.f * pp * rs, hi = 2.f * qq * rs;     // 1 - u and 1 + u, each to full relative accuracy
-                                ph = kLn2 * ((lo > 0.f ? lo * lg2(lo) : 0.f) + (hi > 0.f ? hi * lg2(hi) : 0.f));
-                            }
-                            vC[2] = fmaf(s, ph, vC[2]);
-                        }
-                        vC[3] = fmaf(pp, qq, vC[3]);
-                    } else {
-                        vC[3] += fmaxf(pp - qq, 0.f);
-                    }
-                }
+                const float pp = ex2(fmaf(fmaxf(xt[j], kFloor) - mt, kLog2e, -lSt));
+                const float qq = ex2(fmaf(fmaxf(xd[j], kFloor) - md, kLog2e, -lSd));
+                vC[0] += fmaxf(pp - qq, 0.f);
             }
         }
-        if (MODE == MODE_VANILLA) {
-            float ws = warp_sum(vC[3]);
-            if (lane == 0)
-                for (int r = 0; r < CS; ++r) cluster.map_shared_rank(sh.wtab2, r)[gw] = ws;
-        }
+        const float ws = warp_sum(vC[0]);
+        if (lane == 0)
+            for (int r = 0; r < CS; ++r) cluster.map_shared_rank(sh.wtab2, r)[gw] = ws;
     }
-    cluster_allreduce<4, false>(vC, sh.warp, sh.xC, CS, rank, cluster);
+    cluster_allreduce<2, false>(vC, sh.warp, sh.xC, CS, rank, cluster);
 
-    // sampling: y_i ~ p_i (AdaSD: every row; vanilla: bonus row, or residual-less fallback)
+    // sampling: bonus row, or rejected row (the target row itself where the residual has no mass)
     const size_t it = (size_t)b * (Kmax + 1) + i;
     const size_t id = (size_t)b * Kmax + i;
     if (!bad) {
-        bool from_resid = need_resid && (vC[3] > 0.f);
-        bool do_sample = (MODE == MODE_ADASD) || bonus || need_resid;
-        if (do_sample) {
-            float uu = (MODE == MODE_ADASD) ? p.u_target[it] : p.u_resample[b];
+        const bool from_resid = need_resid && (vC[0] > 0.f);
+        if (bonus || need_resid) {
+            const float uu = p.u_resample[b];
             float base = 0.f, target = 0.f;
             int chosen = select_warp(from_resid ? sh.wtab2 : sh.wtab, GW, uu, base, target);
             if (chosen == gw) {
@@ -230,8 +187,8 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
                 if (from_resid) {
                     tok = warp_scan_select<N>(u0, u1, p.V, base, target, [&](int u, float(&w)[N]) {
                         float xt[N], xd[N];
-                        load_unit_w<T, VEC>(rt, u, p.V, xt, wt);
-                        load_unit_w<T, VEC>(rd, u, p.V, xd, wd);
+                        load_unit<T, VEC>(rt, u, p.V, xt);
+                        load_unit<T, VEC>(rd, u, p.V, xd);
 #pragma unroll
                         for (int j = 0; j < N; ++j) {
                             float pp = ex2(fmaf(fmaxf(xt[j], kFloor) - mt, kLog2e, -lSt));
@@ -242,20 +199,13 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
                 } else {
                     tok = warp_scan_select<N>(u0, u1, p.V, base, target, [&](int u, float(&w)[N]) {
                         float xt[N];
-                        load_unit_w<T, VEC>(rt, u, p.V, xt, wt);
+                        load_unit<T, VEC>(rt, u, p.V, xt);
 #pragma unroll
                         for (int j = 0; j < N; ++j)
                             w[j] = ex2((fmaxf(xt[j], kFloor) - mt) * kLog2e);
                     });
                 }
-                if (lane == 0) {
-                    if (MODE == MODE_ADASD) {
-                        p.sc.y[it] = tok;
-                        if (p.user.y) p.user.y[it] = tok;
-                    } else {
-                        p.sc.van_tok[it] = tok;
-                    }
-                }
+                if (lane == 0) p.sc.van_tok[it] = tok;
             }
         }
     }
@@ -263,43 +213,17 @@ __global__ void __launch_bounds__(kThreads) verify_kernel(VerifyParams p) {
     // publish this position's scalars
     if (rank == 0 && threadIdx.x == 0) {
         if (bad) atomicOr(p.st.status, ADASD_STATUS_NAN);
-        if (MODE == MODE_ADASD) {
-            float Ht = -kLn2 * vC[0], lse_t = fmaf(kLn2, lSt, mt);
-            if (bad) {
-                Ht = lse_t = NAN;
-                p.sc.y[it] = -1;
-                if (p.user.y) p.user.y[it] = -1;
-            }
-            if (p.user.H_t) p.user.H_t[it] = Ht;
-            if (p.user.lse_t) p.user.lse_t[it] = lse_t;
-            if (!bonus) {
-                float Hd = -kLn2 * vC[1], lse_d = fmaf(kLn2, lSd, md);
-                float jsd = 0.25f * vC[2];
-                jsd = differ ? fminf(fmaxf(jsd, 0.f), kLn2) : 0.f;   // identical rows: exactly 0
-                if (!(vC[3] > 0.f)) jsd = kLn2;                      // disjoint supports: exactly ln 2
-                float dist = sqrtf(jsd / kLn2);
-                dist = fminf(dist, 1.f);
-                if (bad) Hd = lse_d = jsd = dist = NAN;
-                p.sc.H_d[id] = Hd;
-                p.sc.dist[id] = dist;
-                if (p.user.H_d) p.user.H_d[id] = Hd;
-                if (p.user.lse_d) p.user.lse_d[id] = lse_d;
-                if (p.user.jsd) p.user.jsd[id] = jsd;
-                if (p.user.dist) p.user.dist[id] = dist;
-            }
-        } else {
-            if (!bonus) {
-                p.sc.van_flag[id] = (van_accept && !bad) ? 1 : 0;
-                if (p.alpha_out) p.alpha_out[id] = bad ? NAN : alpha;
-            }
-            if (bad) p.sc.van_tok[it] = -1;
+        if (!bonus) {
+            p.sc.van_flag[id] = (van_accept && !bad) ? 1 : 0;
+            if (p.alpha_out) p.alpha_out[id] = bad ? NAN : alpha;
         }
+        if (bad) p.sc.van_tok[it] = -1;
     }
 
     // all writes of this cluster are done once every CTA has passed this barrier
     cluster.sync();
-    if (MODE == MODE_ADASD || rank != 0 || threadIdx.x != 0) return;
-    // vanilla: the cluster that publishes the last position of a sequence finds its longest accepted prefix
+    if (rank != 0 || threadIdx.x != 0) return;
+    // the cluster that publishes the last position of a sequence finds its longest accepted prefix
     __threadfence();
     if (atomicAdd(p.sc.ticket + b, 1u) != (unsigned)K_t) return;
     p.sc.ticket[b] = 0u;    // ready for the next round

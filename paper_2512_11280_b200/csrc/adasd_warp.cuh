@@ -35,19 +35,6 @@ struct RowWarp {
 __device__ __forceinline__ float apply_warp(float z, const RowWarp& w) {
     return (z < w.cut) ? -INFINITY : z * w.inv_t;
 }
-template <int N>
-__device__ __forceinline__ void apply_warp(float (&x)[N], const RowWarp& w) {
-#pragma unroll
-    for (int j = 0; j < N; ++j) x[j] = apply_warp(x[j], w);
-}
-
-// load_unit with the row's adjustment applied
-template <typename T, bool VEC>
-__device__ __forceinline__ void load_unit_w(const T* __restrict__ row, int u, int V, float (&x)[Elt<T>::N],
-                                            const RowWarp& w) {
-    load_unit<T, VEC>(row, u, V, x);
-    apply_warp(x, w);
-}
 
 struct CutParams {
     const void* z;
