@@ -133,12 +133,21 @@ def cuts_on(args, wl) -> bool:
     return (0 < k < wl.V) or p < 1.0
 
 
-def vanilla_launches(wl, sm_count: int) -> int:
-    """Kernels one adasd_vanilla_verify call launches: with enough bf16 rows to fill the GPU
-    it runs three (log-sum-exps of all rows, accept test, sampling of one
-    position per sequence), else one."""
-    streaming = wl.dtype == synth.BF16 and wl.V % 8 == 0 and wl.V >= 8192
-    return 3 if streaming and wl.B * (2 * wl.K + 1) >= 2 * sm_count else 1
+def verify_launches(wl) -> int:
+    """Kernels one adasd_verify call launches: aligned bf16 rows one and the sequences' tails, other rows
+    two sweeps and the tails."""
+    return 2 if wl.dtype == synth.BF16 and wl.V % 8 == 0 and wl.V >= 8192 else 3
+
+
+VANILLA_LAUNCHES = 2    # adasd_vanilla_verify: the rows' log-sum-exps, accept test with sampling
+
+
+def cutoff_launches(args, rounds: bool) -> int:
+    """Kernels that find the cutoffs of a draft call's rows or of a round's (target and draft rows): with top-k
+    a selection over all rows at once, else a histogram per set of rows; then a radix kernel per set for
+    the rows they hand over."""
+    top_k = args.warpers[1] > 0
+    return (3 if top_k else 4) if rounds else 2
 
 
 # ------------------------------------------------------------------------------ N ranks
@@ -334,7 +343,7 @@ def run_ours(args) -> dict:
                    "warpers": None if not args.warpers else
                    {"temperature": args.warpers[0], "top_k": args.warpers[1], "top_p": args.warpers[2],
                     "note": "with top-k / top-p on, every call first finds one cutoff logit per row "
-                            "(row_cutoff_kernel): the times include it, the bytes count the rows once"},
+                            "(the cutoff kernels): the times include it, the bytes count the rows once"},
                    "draft_entropy": {"us_per_call": 1e3 * draft_ms, "bytes_per_call": B * row_bytes,
                                      "gbs": B * row_bytes / (draft_ms * 1e-3) / 1e9,
                                      "frac_of_peak": B * row_bytes / (draft_ms * 1e-3) / 1e9 / peak,
@@ -344,10 +353,8 @@ def run_ours(args) -> dict:
                 "what": "pinned host logits -> device, adasd_verify through the C ABI, results -> host",
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": h_out.numel() * 4,
                 "steps": e2e_steps, "ms_per_step": e2e_ms / e2e_steps},
-        # with a top-k / top-p cut every draft call adds two launches (the one-pass cutoff kernel and the
-        # radix kernel for the rows it hands over), verify and vanilla verify four each (target and draft rows)
-        "gpu_launches": args.steps * (K + 1 + vanilla_launches(wl, torch.cuda.get_device_properties(dev).multi_processor_count)
-                                      + (2 * K + 8 if cuts_on(args, wl) else 0)),
+        "gpu_launches": args.steps * (K + verify_launches(wl) + VANILLA_LAUNCHES
+                                      + (K * cutoff_launches(args, False) + 2 * cutoff_launches(args, True) if cuts_on(args, wl) else 0)),
         "clocks": clocks,
         "roofline": {"bound": "hbm", "kernel": "adasd_verify", "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
@@ -526,7 +533,7 @@ def run_single_stream(args, torch, adasd, wl, rank, world, local, dev, dist) -> 
            "steps": n_e2e, "ms_per_step": e2e_ms,
            "what": "pinned host logits -> device, adasd_verify through the C ABI, results -> host"}
     out = common_fields(args, world, wl, f"{args.workload}: B={B} K={K} V={V} single stream, graph replays", extra,
-                        world * vrows / (ms_v * 1e-3), ms_r, ms_v, vrows, reps * nset * (K + 2), clocks, e2e)
+                        world * vrows / (ms_v * 1e-3), ms_r, ms_v, vrows, reps * nset * (K + verify_launches(wl)), clocks, e2e)
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         out["cpu_baseline"] = oracle_sample(synth.WORKLOADS[args.workload], args.cpu_seconds, max_rounds=64)
     if dist is not None:
@@ -683,7 +690,7 @@ def run_adaptive_graph(args, torch, adasd, wl, rank, world, local, dev, dist) ->
            "steps": 3, "ms_per_step": e2e_ms,
            "what": "pinned host logits -> device, adasd_verify through the C ABI, results -> host"}
     out = common_fields(args, world, wl, f"C5: B={B} Kmax={K} V={V} adaptive windows, {R} rounds in one replayed graph",
-                        extra, world * vrows / (verify_ms * 1e-3), ms_round, verify_ms, vrows, R * (K + 1), clocks, e2e)
+                        extra, world * vrows / (verify_ms * 1e-3), ms_round, verify_ms, vrows, R * (K + verify_launches(wl)), clocks, e2e)
     out["steps"] = R
     if rank == 0 and world == 1 and not args.no_cpu_baseline:
         out["cpu_baseline"] = oracle_sample(synth.WORKLOADS["C5"], args.cpu_seconds)
