@@ -12,11 +12,12 @@
 // and the last warp of a position (a counter in device memory) publishes its distance.  Nothing in
 // a launch waits for anything but its own copies.
 //
-// What bounds them: sweep 1 HBM, sweep 2 L2 or HBM (fp32) and the special-function pipe (bf16), for few rows
-// the latency of two launches.  (One launch in which sweep 2 follows sweep 1 at a distance that keeps the
-// rows in L2 was measured slower, 84 to 110 against 61 us for the fp32 case below: warps in different sweeps
-// evict one another's instructions, and those that wait hold up items that others wait for.)
-// Measured: see launch_sweep in adasd_api.cu.
+// What bounds them: sweep 1 HBM, sweep 2 issue slots and the special-function pipe, for few rows the latency of
+// two launches and the tail's.  adasd_verify, three-pass cluster kernel before -> now: fp32 V=128256
+// B=16 K=5 125 -> 51 us (90 MB), B=64 K=4 356 -> 132 (297 MB), fp32 V=32000 B=1 K=5 24.6 -> 17.5,
+// bf16 V=50257 B=8 K=5 59.7 -> 26.9, B=64 160 -> 68.  (One launch in which sweep 2 follows sweep 1 at a distance
+// that keeps the rows in L2 was slower, 84 to 110 us for the first: warps in different sweeps evict one
+// another's instructions, and those that wait hold up items that others wait for.)
 #pragma once
 
 #include "adasd_async.cuh"
