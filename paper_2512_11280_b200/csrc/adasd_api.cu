@@ -116,10 +116,6 @@ int launch_cluster(void (*kernel)(P), const P& params, long long clusters, int c
 // ---- warp-specialised verification kernel: configuration and launch ----------------------
 template <typename K>
 int kernel_occupancy(K kern, int threads, int cs, int smem) {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
     lc.gridDim = dim3((unsigned)(cs * 64), 1, 1);
@@ -150,8 +146,21 @@ int kernel_static_smem(K kern) {
     return (int)fa.sharedSizeBytes;
 }
 
+// The limit on dynamic shared memory is one value per function and device, not per context: it is set to the
+// most any vocabulary of this ITER can ask for, so that no context lowers it under another's launches.
+template <int ITER, bool WARPED>
+cudaError_t fast_allow(int smem_optin) {
+    const int st = kernel_static_smem(spec_verify_kernel<ITER, WARPED>);
+    if (st < 0) return cudaErrorInvalidDeviceFunction;
+    return cudaFuncSetAttribute(spec_verify_kernel<ITER, WARPED>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                std::min(kSW * ITER * kSIterBytes, smem_optin - st));
+}
 template <int ITER>
-int fast_occupancy(int cs, int smem) {
+int fast_occupancy(int cs, int smem, int smem_optin) {
+    if (fast_allow<ITER, false>(smem_optin) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
     return kernel_occupancy(spec_verify_kernel<ITER>, kSThreads, cs, smem);
 }
 template <int ITER>
@@ -174,9 +183,14 @@ int fast_static_smem() {
         default: return fail;                \
     }
 
-int fast_occupancy_iter(int iter, int cs, int smem) {
-#define CALL(I) fast_occupancy<I>(cs, smem)
+int fast_occupancy_iter(int iter, int cs, int smem, int smem_optin) {
+#define CALL(I) fast_occupancy<I>(cs, smem, smem_optin)
     ADASD_ITER_SWITCH(iter, CALL, 0)
+#undef CALL
+}
+cudaError_t fast_allow_warped_iter(int iter, int smem_optin) {
+#define CALL(I) fast_allow<I, true>(smem_optin)
+    ADASD_ITER_SWITCH(iter, CALL, cudaErrorInvalidValue)
 #undef CALL
 }
 int fast_static_smem_iter(int iter) {
@@ -203,9 +217,9 @@ void fast_setup(adasd_ctx* c, size_t smem_optin) {
         if (iter < 1 || iter > kSMaxIter) continue;
         const int st = fast_static_smem_iter(iter);
         if (st < 0) continue;
-        const int smem = nwi * 2048;      // two position buffers: 512 bytes per row and warp-iteration
+        const int smem = nwi * kSIterBytes;
         if (smem > (int)smem_optin - st - 1024) continue;
-        const int ncl = fast_occupancy_iter(iter, cs, smem);
+        const int ncl = fast_occupancy_iter(iter, cs, smem, (int)smem_optin);
         const int score = ncl * cs;
         if (score > best_score) {
             best_score = score;
@@ -214,6 +228,10 @@ void fast_setup(adasd_ctx* c, size_t smem_optin) {
             f.smem = smem;
             f.geom.ncl = ncl;
         }
+    }
+    if (f.iter > 0 && fast_allow_warped_iter(f.iter, (int)smem_optin) != cudaSuccess) {
+        cudaGetLastError();
+        f.iter = 0;
     }
 }
 void cutoff_setup(adasd_ctx* c) {
@@ -364,10 +382,6 @@ int fast_launch(adasd_ctx* c, const VerifyParams& p, cudaStream_t stream) {
     const adasd_ctx::Fast& f = c->fast;
     ClusterGeom gq = f.geom;
     if (positions < gq.ncl) gq.ncl = (int)positions;
-    if (WARPED) {
-        // the instantiation for adjusted distributions: same footprint, its own attribute
-        CUDA_TRY(cudaFuncSetAttribute(spec_verify_kernel<ITER, WARPED>, cudaFuncAttributeMaxDynamicSharedMemorySize, f.smem));
-    }
     return launch_pdl(spec_verify_kernel<ITER, WARPED>, gq.ncl * f.cs, kSThreads, f.smem, f.cs, stream, p, gq);
 }
 

@@ -51,6 +51,7 @@ constexpr int kSThreads = (kSW + 4) * 32;        // 512: three warpgroups of com
 constexpr int kSHead = 5;                        // iterations whose 2^t values wait in tensor memory
 constexpr int kSRegIter = 5;                     // ... and in registers, at most
 constexpr int kSMaxIter = kSHead + kSRegIter;    // largest number of iterations per warp and row
+constexpr int kSIterBytes = 2048;                // of a warp's buffers and iteration: two positions, both rows, 512 bytes each
 constexpr int kSTmemCols = 512;                  // columns allocated (all of them: one CTA per SM)
 constexpr int kSTmemHalf = kSHead * 16;          // columns of one position's head: 16 per iteration
 constexpr int kSTmemWarp = 2 * kSTmemHalf;       // columns of one compute warp: two positions in flight
@@ -374,7 +375,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
         // values the buffer is refilled with position n + 2, one whole position before that is
         // needed.
         const int kRowB = I_w * 512;              // bytes of one row in this warp's buffers
-        unsigned char* const bufs = dyn_smem + (size_t)wi0 * 2048;
+        unsigned char* const bufs = dyn_smem + (size_t)wi0 * kSIterBytes;
         auto buf_of = [&](int n) -> unsigned char* { return bufs + (size_t)(n & 1) * (2 * kRowB) + (size_t)lane * 16; };
         auto bar_of = [&](int n) -> uint64_t* { return reinterpret_cast<uint64_t*>(&sh.bar[warp][n & 1]); };
         auto pcx = [&](int n) -> const PosCtx& { return sh.pc[n & (kSPosRing - 1)]; };
