@@ -38,7 +38,8 @@ template <int NW>
 struct __align__(16) DraftShared {
     float2 run[kDMaxEntries][kDRuns];          // rank 0: (shift, sum of 2^t under it) of every run, by warp of the cluster
     float4 wpart[kDMaxEntries];                // rank 0: every warp's (largest logit, S, T, flags)
-    int32_t widx[kDMaxEntries];                // rank 0: index of every warp's largest logit (greedy drafting)
+    float wtop[kDMaxEntries];                  // rank 0, greedy drafting: every warp's largest logit,
+    int32_t widx[kDMaxEntries];                // its index
     unsigned long long bar[NW][kDMaxRing];
 };
 
@@ -114,7 +115,8 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
     // v: the largest logit so far (kFloorL while there is none): t = (z - v) log2 e is exactly 0 for it, so
     // that a one-hot row gets S = 1, T = 0 and H = 0 exactly
     float v = kFloorL;
-    int vi = -1;
+    float top = -INFINITY;                                  // greedy drafting: the largest logit, finite but perhaps without
+    int vi = -1;                                            // probability (a mask of the type's lowest value), and its index
     float2 S2 = make_float2(0.f, 0.f), T2 = S2, R2 = S2;    // lane partials under v; R2: S of the current run, not yet in S2
     uint32_t bad = 0u;
     const float2 L2 = pair2(c1);
@@ -157,7 +159,8 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
         const float lm = U::max_val(mx, bad);
         const float x = warp_max_f32(lm);
         if (x == INFINITY) bad = 1u;
-        if (greedy && x > v && x > floor_v) {               // the lowest index of the chunk that has it
+        if (greedy && x > top) {                            // the lowest index of the chunk that has it
+            top = x;
             int first = 0x7FFFFFFF;
             if (lm == x) {
 #pragma unroll 1
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
                     uint4 w = load(k);
                     mask(w, k);
                     float2 z[NP];
-                    U::unpack(w, z);
+                    U::unpack_raw(w, z);
 #pragma unroll
                     for (int j = NP - 1; j >= 0; --j) {
                         const int e = (32 * (ci + k) + lane) * N + 2 * j;
@@ -227,6 +230,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
     if (lane >= run && lane < kDRuns) r0->run[g][lane] = make_float2(kFloorL, 0.f);      // runs this warp does not have
     if (lane == 0) {
         r0->wpart[g] = make_float4(v, Sw, Tw, __uint_as_float(bad));
+        r0->wtop[g] = top;
         r0->widx[g] = vi;
     }
     // totals and tables of every CTA are in rank 0's shared memory
@@ -251,10 +255,12 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
 
     int tok = -1;
     const bool sampling = !greedy && p.u != nullptr && p.token_out != nullptr;
-    if (greedy && !rowbad) {
+    if (greedy && !(fl & 1u)) {
         // shares are in index order: the lowest index of those that have the maximum
-        const int i0 = lane < G && e0.x == Mr ? sh.widx[lane] : 0x7FFFFFFF, i1 = lane + 32 < G && e1.x == Mr ? sh.widx[lane + 32] : 0x7FFFFFFF;
-        tok = __reduce_min_sync(0xFFFFFFFFu, min(i0, i1));
+        const float t0 = lane < G ? sh.wtop[lane] : -INFINITY, t1 = lane + 32 < G ? sh.wtop[lane + 32] : -INFINITY;
+        const float t = warp_max_f32(fmaxf(t0, t1));
+        const int i0 = lane < G && t0 == t ? sh.widx[lane] : 0x7FFFFFFF, i1 = lane + 32 < G && t1 == t ? sh.widx[lane + 32] : 0x7FFFFFFF;
+        tok = t > -INFINITY ? __reduce_min_sync(0xFFFFFFFFu, min(i0, i1)) : -1;
     } else if (sampling && !rowbad) {
         // x ~ q: the crossing of u S in index order: first the share that holds it, then the run in it
         float target = u_row * S;

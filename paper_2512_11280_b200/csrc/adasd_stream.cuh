@@ -187,7 +187,9 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
     for (int n = 0;; ++n) {
         const StreamItem c = items[warp][n & (kRItems - 1)];
         if (c.slot < 0) break;
-        float v = kFloorL;                       // argmax: largest logit so far; else its shift fl(z log2 e / T) (kFloorL: nothing finite)
+        // argmax: the largest logit so far, any finite one (also a mask of the type's lowest value, which has no
+        // probability); else its shift fl(z log2 e / T) (kFloorL: nothing finite)
+        float v = OP == OP_ARGMAX ? -INFINITY : kFloorL;
         float2 S2 = make_float2(0.f, 0.f);
         int idx = -1;                            // its index
         uint32_t bad = 0u;
@@ -215,7 +217,7 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
             if (x == INFINITY) bad = 1u;
             if (OP == OP_ARGMAX) {
                 // a larger maximum: the lowest index of the chunk that has it
-                if (x > v && x > floor_v) {
+                if (x > v) {
                     v = x;
                     int first = 0x7FFFFFFF;
                     if (lm == x) {
@@ -301,16 +303,17 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
 struct SegPair {
     float4 a, b;
 };
-__device__ __forceinline__ SegPair load_segments(const float4* seg, int segs, bool on) {
+// (v_none: the maximum of a segment that does not exist)
+__device__ __forceinline__ SegPair load_segments(const float4* seg, int segs, bool on, float v_none) {
     const int lane = threadIdx.x & 31;
-    const float4 none = make_float4(kFloorL, 0.f, __int_as_float(-1), 0.f);
+    const float4 none = make_float4(v_none, 0.f, __int_as_float(-1), 0.f);
     SegPair r;
     r.a = on && lane < segs ? __ldcg(seg + lane) : none;
     r.b = on && lane + 32 < segs ? __ldcg(seg + lane + 32) : none;
     return r;
 }
-__device__ __forceinline__ bool segments_bad(const SegPair& s, float v) {
-    return __any_sync(0xFFFFFFFFu, (__float_as_uint(s.a.w) | __float_as_uint(s.b.w)) & 1u) || !(v > kFloorL);
+__device__ __forceinline__ bool segments_bad(const SegPair& s, float v, float v_none) {
+    return __any_sync(0xFFFFFFFFu, (__float_as_uint(s.a.w) | __float_as_uint(s.b.w)) & 1u) || !(v > v_none);
 }
 
 // ---- vanilla: accept test and the one sampled position of every sequence ---------------------
@@ -383,7 +386,7 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const int r = r0 + k * kVWarps;
-            sp[k] = load_segments(q.seg + (((size_t)b * R + slot_of(r)) << q.seg_bits), segs, r < 2 * kt + 1);
+            sp[k] = load_segments(q.seg + (((size_t)b * R + slot_of(r)) << q.seg_bits), segs, r < 2 * kt + 1, kFloorL);
         }
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -391,7 +394,7 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
             if (r < 2 * kt + 1) {
                 const float v = warp_max_f32(fmaxf(sp[k].a.x, sp[k].b.x));
                 const float sum = warp_sum(ex2(sp[k].a.x - v) * sp[k].a.y + ex2(sp[k].b.x - v) * sp[k].b.y);
-                const float lse = segments_bad(sp[k], v) ? NAN : kLn2 * (v + lg2(sum));
+                const float lse = segments_bad(sp[k], v, kFloorL) ? NAN : kLn2 * (v + lg2(sum));
                 if (lane == 0) sh.lse[r <= kt ? r : ADASD_KMAX_LIMIT + 1 + (r - kt - 1)] = lse;
             }
         }
@@ -655,7 +658,7 @@ __global__ void __launch_bounds__(kGThreads) greedy_finish_kernel(GreedyParams p
         SegPair sp[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k)
-            sp[k] = load_segments(p.seg + (((size_t)b * R + i0 + k * W) << p.seg_bits), segs, i0 + k * W <= kt);
+            sp[k] = load_segments(p.seg + (((size_t)b * R + i0 + k * W) << p.seg_bits), segs, i0 + k * W <= kt, -INFINITY);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const int i = i0 + k * W;
@@ -664,7 +667,7 @@ __global__ void __launch_bounds__(kGThreads) greedy_finish_kernel(GreedyParams p
                 // segments are in index order: the lowest index of those that have the maximum
                 const int ia = sp[k].a.x == v ? __float_as_int(sp[k].a.z) : 0x7FFFFFFF, ib = sp[k].b.x == v ? __float_as_int(sp[k].b.z) : 0x7FFFFFFF;
                 int am = __reduce_min_sync(0xFFFFFFFFu, min(ia, ib));
-                if (segments_bad(sp[k], v)) am = -1;
+                if (segments_bad(sp[k], v, -INFINITY)) am = -1;
                 if (lane == 0) {
                     choice[i] = am;
                     if (p.argmax_out) p.argmax_out[(size_t)b * K1 + i] = am;
