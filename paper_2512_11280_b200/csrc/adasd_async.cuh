@@ -116,6 +116,13 @@ struct Unit<__nv_bfloat16> {
     static __device__ __forceinline__ void max_add(Max& m, const uint4& w) {
         m = bmax2(bmax2(m, w.x), bmax2(w.y, bmax2(w.z, w.w)));
     }
+    // largest element of a unit (NaN kept), and as one number (NaN dropped)
+    static __device__ __forceinline__ Max unit_max(const uint4& w) { return bmax2(bmax2(w.x, w.y), bmax2(w.z, w.w)); }
+    static __device__ __forceinline__ void max_join(Max& m, Max h) { m = bmax2(m, h); }
+    static __device__ __forceinline__ float top(Max h) {
+        const float2 v = unpack2(h);
+        return fmaxf(v.x, v.y);
+    }
     static __device__ __forceinline__ float max_val(Max m, uint32_t& bad) {
         const float2 v = unpack2(m);
         if (v.x != v.x || v.y != v.y) bad = 1u;
@@ -181,6 +188,11 @@ struct Unit<float> {
         m = fmax_nan(fmax_nan(m, __uint_as_float(w.x)),
                      fmax_nan(__uint_as_float(w.y), fmax_nan(__uint_as_float(w.z), __uint_as_float(w.w))));
     }
+    static __device__ __forceinline__ Max unit_max(const uint4& w) {
+        return fmax_nan(fmax_nan(__uint_as_float(w.x), __uint_as_float(w.y)), fmax_nan(__uint_as_float(w.z), __uint_as_float(w.w)));
+    }
+    static __device__ __forceinline__ void max_join(Max& m, Max h) { m = fmax_nan(m, h); }
+    static __device__ __forceinline__ float top(Max h) { return h; }
     static __device__ __forceinline__ float max_val(Max m, uint32_t& bad) {
         if (m != m) bad = 1u;
         return m;

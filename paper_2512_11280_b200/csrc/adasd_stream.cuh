@@ -187,11 +187,13 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
     for (int n = 0;; ++n) {
         const StreamItem c = items[warp][n & (kRItems - 1)];
         if (c.slot < 0) break;
-        // argmax: the largest logit so far, any finite one (also a mask of the type's lowest value, which has no
-        // probability); else its shift fl(z log2 e / T) (kFloorL: nothing finite)
-        float v = OP == OP_ARGMAX ? -INFINITY : kFloorL;
+        float v = kFloorL;                       // its shift fl(z log2 e / T) (kFloorL: nothing finite)
         float2 S2 = make_float2(0.f, 0.f);
-        int idx = -1;                            // its index
+        // argmax: this lane's largest logit so far, its unit (the first that has it) and what is in it.  Any finite
+        // logit counts, also one that has no probability (a mask of the type's lowest value)
+        float top = -INFINITY;
+        int top_u = -1;
+        uint4 top_w = U::none4();
         uint32_t bad = 0u;
         const typename U::Cut cut = U::make_cut(c.cut);
         // One chunk; EDGE: the last one of the row.  The maximum first, then the sum, each from shared
@@ -210,31 +212,25 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
                 return w;
             };
             typename U::Max mx = U::max0();
-#pragma unroll
-            for (int k = 0; k < IT; ++k) U::max_add(mx, load(k));
-            const float lm = U::max_val(mx, bad);
-            const float x = warp_max_f32(lm);
-            if (x == INFINITY) bad = 1u;
             if (OP == OP_ARGMAX) {
-                // a larger maximum: the lowest index of the chunk that has it
-                if (x > v) {
-                    v = x;
-                    int first = 0x7FFFFFFF;
-                    if (lm == x) {
-                        for (int k = IT - 1; k >= 0; --k) {
-                            float2 z[NP];
-                            U::unpack_raw(load(k), z);
 #pragma unroll
-                            for (int j = NP - 1; j >= 0; --j) {
-                                const int e = (32 * (ch * IT + k) + lane) * N + 2 * j;
-                                if (z[j].y == x) first = e + 1;
-                                if (z[j].x == x) first = e;
-                            }
-                        }
+                for (int k = 0; k < IT; ++k) {
+                    const uint4 w = load(k);
+                    const typename U::Max h = U::unit_max(w);
+                    U::max_join(mx, h);
+                    const float t = U::top(h);
+                    if (t > top) {
+                        top = t;
+                        top_u = 32 * (ch * IT + k) + lane;
+                        top_w = w;
                     }
-                    idx = __reduce_min_sync(0xFFFFFFFFu, first);
                 }
+                U::max_val(mx, bad);
             } else {
+#pragma unroll
+                for (int k = 0; k < IT; ++k) U::max_add(mx, load(k));
+                const float x = warp_max_f32(U::max_val(mx, bad));
+                if (x == INFINITY) bad = 1u;
                 if (x > floor_v && x * c1 > v) { // raise the shift, rescale what is summed
                     const float m = x * c1, f = ex2(v - m);
                     S2.x *= f;
@@ -279,7 +275,24 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
             else if (ch == NC - 1) chunk(std::true_type{}, ch, sb);
             else chunk(std::false_type{}, ch, sb);
         }
-        const float S = OP == OP_LSE ? warp_sum(S2.x + S2.y) : 0.f;
+        float S = 0.f;
+        int idx = 0x7FFFFFFF;
+        if (OP == OP_ARGMAX) {                   // lowest index of the largest logit: that of the lowest unit that has it
+            v = warp_max_f32(top);
+            if (v == INFINITY) bad = 1u;
+            if (top_u >= 0 && top == v) {
+                float2 z[NP];
+                U::unpack_raw(top_w, z);
+#pragma unroll
+                for (int j = NP - 1; j >= 0; --j) {
+                    if (z[j].y == v) idx = top_u * N + 2 * j + 1;
+                    if (z[j].x == v) idx = top_u * N + 2 * j;
+                }
+            }
+            idx = __reduce_min_sync(0xFFFFFFFFu, idx);
+        } else {
+            S = warp_sum(S2.x + S2.y);
+        }
         bad = __reduce_or_sync(0xFFFFFFFFu, bad);
         if (lane == 0) p.seg[((size_t)c.slot << p.seg_bits) + c.seg] = make_float4(v, S, __int_as_float(idx), __uint_as_float(bad));
         if (!alive) {
