@@ -240,20 +240,31 @@ void cutoff_setup(adasd_ctx* c) {
     if (!c->cut_hist) cudaGetLastError();
 }
 
-// Chunk length and segments of a row in the vanilla and greedy modes.  Chunks of 8 iterations (4 KB)
-// where every warp of the grid gets two of them, else of 2; segments of at least two chunks while that
-// gives the warps six items each (half as long measured 33 instead of 31.8 us on 544 rows of 128256),
-// shorter ones only where warps would have nothing to do.
+// Chunk length and segments of a row in the vanilla and greedy modes.
+// Chunks of 8 iterations (4 KB) cost a warp 0.42 us, of 2 iterations 0.33: the short ones only where a row does
+// not fill a long one, or where segments of long ones would be so few that shorter ones spread the launch over
+// more warps: less than one for four warps (vanilla, bf16 V=8200 B=8 K=5, 352 of them: 10.0 us with short chunks, 10.5
+// with long ones; V=16384, 704: 10.6 and 9.4), five where a row is a single chunk (greedy, fp32 V=1000 B=64 K=4, 576:
+// 5.4 and 4.7).
+// Segments: with four chunks or more for every warp of the grid, at least two chunks each while that gives the
+// warps six items each (half as long measured 33 instead of 31.8 us on 544 rows of 128256); with fewer long
+// chunks, as many as leave every warp with one item at most (greedy, 512 rows of 8200 bf16, 1024 / 2048 / 4096
+// items: 7.2 / 7.8 / 9.5 us); short chunks: an item for every warp at least.
 void stream_setup(adasd_ctx* c) {
     const int N = c->cfg.dtype == ADASD_BF16 ? 8 : 4, NU = (c->cfg.V + N - 1) / N;
     const long long rows = (long long)c->cfg.B * (2 * c->cfg.Kmax + 1), warps = 2LL * c->sm_count * kRW;
     const int nc8 = (NU + 255) / 256;
-    c->stream_it = rows * nc8 >= 2 * warps ? 8 : 2;
+    long long items8 = rows;
+    for (int k = 2; k <= std::min(kMaxSegs, nc8); k *= 2) items8 *= 2;
+    c->stream_it = NU >= 224 && items8 * (nc8 == 1 ? 5 : 4) >= warps ? 8 : 2;
     const int NC = c->stream_it == 8 ? nc8 : (NU + 63) / 64;
+    auto more = [&](int bits) -> bool {
+        const long long items = rows << bits;
+        if (c->stream_it == 8 && rows * nc8 < 4 * warps) return items * 2 <= warps;
+        return items < warps || (items < 6 * warps && (NC >> bits) >= 4);
+    };
     int bits = 0;
-    while ((2 << bits) <= std::min(kMaxSegs, NC) &&
-           ((rows << bits) < warps || ((rows << bits) < 6 * warps && (NC >> bits) >= 4)))
-        ++bits;
+    while ((2 << bits) <= std::min(kMaxSegs, NC) && more(bits)) ++bits;
     c->seg_bits = bits;
 }
 
