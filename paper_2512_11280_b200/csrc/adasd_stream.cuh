@@ -1,13 +1,15 @@
 // Streaming row statistics for sm_100a: what vanilla speculative sampling and greedy decoding need of
 // the rows of a round, read from HBM once.  bf16 or fp32 rows of any length, alignment and stride.
 //
-// The accept test of a vanilla candidate needs only two numbers of its two rows, the log-sum-exps:
-// alpha = min(1, exp((z_t[x] - lse_t) - (z_d[x] - lse_d))); only ONE position of a sequence needs more,
+// The accept test of a vanilla candidate needs only the softmax normalisers of its two rows,
+// alpha = min(1, p(x) / q(x)), as the largest logit m and S = sum 2^((z - m) log2 e): log2 p(x) = (z[x] - m) log2 e - log2 S
+// stays as accurate for rows whose logits share a large offset, where a log-sum-exp would round to a
+// multiple of its own last bit (logits around 5000: 4e-4 in alpha).  Only ONE position of a sequence needs more,
 // the first rejected one (its residual max(0, p - q) is sampled) or, if none is rejected, the bonus
 // row.  The greedy test needs the target rows' argmax.  So:
 //
 //  1. row_stream_kernel streams every needed row once: the row is cut into segments, a WARP takes a
-//     segment at a time and leaves (shift, sum of 2^t) or (largest logit, its index) of it in
+//     segment at a time and leaves its largest logit and the sum of 2^t under it, or its index, in
 //     a table.  No warp waits for another: the rounding of a row to warps costs nothing but its
 //     last, shorter, copy, and one row of one sequence spreads over the chip as well as a batch does.
 //  2. vanilla_finish_kernel (a cluster per sequence) folds the segments, forms the alphas, finds the
@@ -30,6 +32,7 @@ constexpr int kRRing = 3;
 constexpr int kRStage = 8 * 512 + 16;            // a chunk of 8 iterations (+ one unit: rows off a 16-byte boundary)
 constexpr int kRSmem = kRW * kRRing * kRStage;
 constexpr int kMaxSegs = 64;                     // segments of a row, at most
+constexpr float kRBig = 1e7f;                    // shifts up to it are exact to 0.5
 constexpr int kRItems = 4;                       // items of a warp that may be between their first copy and their end
 
 constexpr int OP_LSE = 0, OP_ARGMAX = 1;
@@ -61,6 +64,22 @@ struct __align__(16) StreamItem {
     int32_t pad[2];
 };
 
+// Largest logit of elements [e0, e1) of a row and the sum of 2^((z - m) log2 e / T), by a warp, element by element
+// from memory: logits or 1 / T so large (1e7 and more between them) that a shift fl(m log2 e / T) is off by whole
+// powers of two.
+template <typename T>
+__device__ __noinline__ float2 big_segment(const T* row, int e0, int e1, float c1, float cut) {
+    const int lane = threadIdx.x & 31;
+    float m = kFloorL, S = 0.f;
+    for (int e = e0 + lane; e < e1; e += 32) m = fmaxf(m, to_f32(row[e]));
+    m = warp_max_f32(m);
+    for (int e = e0 + lane; e < e1; e += 32) {
+        const float z = to_f32(row[e]);
+        if (z >= cut) S += ex2((z - m) * c1);
+    }
+    return make_float2(m, warp_sum(S));
+}
+
 // IT: 8 iterations a chunk, or 2 where the launch has too few chunks of 8 for its warps.
 // (bounds of 320 threads: at most 96 registers a thread)
 template <typename T, bool ALIGNED, int OP, bool WARPED, int IT>
@@ -76,7 +95,12 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
     const int rows_of_d = p.zd ? 1 : 0;
     const int NU = (p.V + N - 1) / N, NC = (NU + 32 * IT - 1) / (32 * IT);
     const int GW = (int)gridDim.x * kRW, gw = (int)blockIdx.x * kRW + warp;
-    const float c1 = WARPED ? p.c1 : kLog2e;
+    const float c1 = WARPED ? p.c1 : kLog2e, inv_c1 = 1.f / c1;
+    auto row_of = [&](int slot) -> const T* {    // (of the table)
+        const int b = slot / R, i = slot - b * R;
+        return i <= K ? reinterpret_cast<const T*>(p.zt) + (long long)b * p.t_seq + (long long)i * p.t_row
+                      : reinterpret_cast<const T*>(p.zd) + (long long)b * p.d_seq + (long long)(i - K1) * p.d_row;
+    };
     unsigned char* const ring = dyn_smem + (size_t)warp * (kRRing * kRStage);
     if (lane == 0) {
         for (int s = 0; s < kRRing; ++s) mbar_init(reinterpret_cast<uint64_t*>(&bars[warp][s]), 1);
@@ -187,7 +211,7 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
     for (int n = 0;; ++n) {
         const StreamItem c = items[warp][n & (kRItems - 1)];
         if (c.slot < 0) break;
-        float v = kFloorL;                       // its shift fl(z log2 e / T) (kFloorL: nothing finite)
+        float v = kFloorL;                       // the segment's shift fl(z log2 e / T), z its largest logit (kFloorL: nothing finite)
         float2 S2 = make_float2(0.f, 0.f);
         // argmax: this lane's largest logit so far, its unit (the first that has it) and what is in it.  Any finite
         // logit counts, also one that has no probability (a mask of the type's lowest value)
@@ -291,7 +315,20 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
             }
             idx = __reduce_min_sync(0xFFFFFFFFu, idx);
         } else {
+            // The table holds a logit m next to the largest and the sum under it: the exponents z log2 e / T - v are all off by
+            // the same residue m log2 e / T - v
             S = warp_sum(S2.x + S2.y);
+            if (v > kFloorL) {
+                if (fabsf(v) < kRBig) {
+                    const float m = v * inv_c1;
+                    S *= ex2(-fmaf(m, c1, -v));
+                    v = m;
+                } else {
+                    const float2 ms = big_segment(row_of(c.slot), 32 * IT * N * c.ch0, min(32 * IT * N * c.ch1, p.V), c1, c.cut);
+                    v = ms.x;
+                    S = ms.y;
+                }
+            }
         }
         bad = __reduce_or_sync(0xFFFFFFFFu, bad);
         if (lane == 0) p.seg[((size_t)c.slot << p.seg_bits) + c.seg] = make_float4(v, S, __int_as_float(idx), __uint_as_float(bad));
@@ -331,9 +368,9 @@ __device__ __forceinline__ bool segments_bad(const SegPair& s, float v, float v_
 
 // ---- vanilla: accept test and the one sampled position of every sequence ---------------------
 //
-// A cluster of S CTAs per sequence.  Each CTA folds the log-sum-exps of the round's rows and finds the
+// A cluster of S CTAs per sequence.  Each CTA folds the normalisers of the round's rows and finds the
 // first rejection for itself; the row pair of that position is then read a second time (from L2 where
-// the round is small), spread over the cluster's warps: with the log-sum-exps known, p and q are final
+// the round is small), spread over the cluster's warps: with the normalisers known, p and q are final
 // as they are read, so sums of the residual max(0, p - q) (and of p, for the bonus row and for a
 // residual without mass) over blocks of a warp's share locate the crossing of u, and rank 0 scans that
 // block again.  Latency bounds it: the caller's tokens, their logits and the uniforms are read before
@@ -351,7 +388,7 @@ struct VanillaParams {
 };
 
 struct VanillaShared {
-    float lse[2 * ADASD_KMAX_LIMIT + 1];         // log-sum-exp of the rows (NaN: unusable): target, then draft
+    float2 row[2 * ADASD_KMAX_LIMIT + 1];        // largest logit and log2 S of the rows (NaN: unusable): target, then draft
     float2 tab[kVMaxS * kVWarps * kVBlocks];     // rank 0: (residual, target) mass of every block, warp by warp of the cluster
     int32_t w;
 };
@@ -367,7 +404,7 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
     const int b = blockIdx.x / S;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int K = p.Kmax, K1 = K + 1, R = 2 * K + 1;
-    const float c1 = p.c1, floor_v = N == 8 ? ADASD_FLOOR_BF : kFloor;
+    const float c1 = p.c1;
     pdl_trigger();
 
     int kt = p.draft_len ? __ldg(p.draft_len + b) : K;
@@ -406,9 +443,9 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
             const int r = r0 + k * kVWarps;
             if (r < 2 * kt + 1) {
                 const float v = warp_max_f32(fmaxf(sp[k].a.x, sp[k].b.x));
-                const float sum = warp_sum(ex2(sp[k].a.x - v) * sp[k].a.y + ex2(sp[k].b.x - v) * sp[k].b.y);
-                const float lse = segments_bad(sp[k], v, kFloorL) ? NAN : kLn2 * (v + lg2(sum));
-                if (lane == 0) sh.lse[r <= kt ? r : ADASD_KMAX_LIMIT + 1 + (r - kt - 1)] = lse;
+                const float sum = warp_sum(ex2((sp[k].a.x - v) * c1) * sp[k].a.y + ex2((sp[k].b.x - v) * c1) * sp[k].b.y);
+                const float lS = segments_bad(sp[k], v, kFloorL) ? NAN : lg2(sum);
+                if (lane == 0) sh.row[r <= kt ? r : ADASD_KMAX_LIMIT + 1 + (r - kt - 1)] = make_float2(v, lS);
             }
         }
     }
@@ -417,26 +454,24 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
         bool reject = false, bad = false;
         if (lane < kt) {
             const size_t idd = (size_t)b * K + lane;
-            const float lt = sh.lse[lane], ld = sh.lse[ADASD_KMAX_LIMIT + 1 + lane];
-            bad = (lt != lt) || (ld != ld);
+            const float2 mt = sh.row[lane], md = sh.row[ADASD_KMAX_LIMIT + 1 + lane];
+            bad = (mt.y != mt.y) || (md.y != md.y);
             float alpha = 0.f;
             if (x_ok) {
-                // ln p(x) and ln q(x), -inf logits clamped; their difference is formed before any
-                // scaling so that identical rows give exactly 0, alpha exactly 1
-                // (logits of the adjusted distribution: scaled by 1 / T, -inf below the row's cutoff)
-                const RowWarp wt = {p.inv_temp, p.cut_t ? p.cut_t[(size_t)b * K1 + lane] : -INFINITY};
-                const RowWarp wd = {p.inv_temp, p.cut_d ? p.cut_d[idd] : -INFINITY};
-                const float lp = fmaxf(apply_warp(ztx, wt), floor_v) - lt;
-                const float lq = fmaxf(apply_warp(zdx, wd), floor_v) - ld;
-                alpha = fminf(1.f, ex2(__fmul_rn(__fsub_rn(lp, lq), kLog2e)));
-                if (!(ex2(__fmul_rn(lq, kLog2e)) > 0.f)) alpha = 1.f;       // q(x) = 0 cannot have been drafted
+                // log2 p(x) and log2 q(x): -inf for a logit below its row's cutoff; equal, and alpha exactly 1, where
+                // the rows are
+                if (p.cut_t && ztx < p.cut_t[(size_t)b * K1 + lane]) ztx = -INFINITY;
+                if (p.cut_d && zdx < p.cut_d[idd]) zdx = -INFINITY;
+                const float lp = fmaf(ztx - mt.x, c1, -mt.y), lq = fmaf(zdx - md.x, c1, -md.y);
+                alpha = fminf(1.f, ex2(lp - lq));
+                if (!(ex2(lq) > 0.f)) alpha = 1.f;       // q(x) = 0 cannot have been drafted
             }
             reject = bad || !(u_acc < alpha);
             if (rank == 0 && p.alpha_out) p.alpha_out[idd] = bad ? NAN : alpha;
         }
         const unsigned mr = __ballot_sync(0xFFFFFFFFu, reject), mb = __ballot_sync(0xFFFFFFFFu, bad);
         if (lane == 0) {
-            const float lb = sh.lse[kt];           // the bonus row
+            const float lb = sh.row[kt].y;         // the bonus row
             if (rank == 0 && (mb || lb != lb)) atomicOr(p.st.status, ADASD_STATUS_NAN);
             sh.w = mr ? (__ffs(mr) - 1) : kt;
         }
@@ -444,11 +479,11 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
     __syncthreads();
     const int i = sh.w;
     const bool bonus = (i >= kt);
-    const float lt = sh.lse[i], ld = bonus ? 0.f : sh.lse[ADASD_KMAX_LIMIT + 1 + i];
-    const bool rowbad = (lt != lt) || (ld != ld);
+    const float2 mt = sh.row[i], md = bonus ? make_float2(0.f, 0.f) : sh.row[ADASD_KMAX_LIMIT + 1 + i];
+    const bool rowbad = (mt.y != mt.y) || (md.y != md.y);
 
     // p and max(0, p - q) of unit u of the two rows
-    const float nlt = -lt * kLog2e, nld = -ld * kLog2e;
+    const float2 c2 = pair2(c1), nmt2 = pair2(-mt.x), nst2 = pair2(-mt.y), nmd2 = pair2(-md.x), nsd2 = pair2(-md.y);
     const typename U::Cut cut_t = U::make_cut(p.cut_t ? __ldg(p.cut_t + (size_t)b * K1 + i) : -INFINITY);
     const typename U::Cut cut_d = U::make_cut((p.cut_d && !bonus) ? __ldg(p.cut_d + (size_t)b * K + i) : -INFINITY);
     const int NU = (p.V + N - 1) / N, NI = (NU + 31) >> 5;
@@ -483,9 +518,10 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
         U::unpack(d, y);
 #pragma unroll
         for (int j = 0; j < NP; ++j) {
-            pv[2 * j] = ex2(fmaf(z[j].x, c1, nlt));
-            pv[2 * j + 1] = ex2(fmaf(z[j].y, c1, nlt));
-            const float q0 = bonus ? 0.f : ex2(fmaf(y[j].x, c1, nld)), q1 = bonus ? 0.f : ex2(fmaf(y[j].y, c1, nld));
+            const float2 lp = __ffma2_rn(__fadd2_rn(z[j], nmt2), c2, nst2), lq = __ffma2_rn(__fadd2_rn(y[j], nmd2), c2, nsd2);
+            pv[2 * j] = ex2(lp.x);
+            pv[2 * j + 1] = ex2(lp.y);
+            const float q0 = bonus ? 0.f : ex2(lq.x), q1 = bonus ? 0.f : ex2(lq.y);
             rv[2 * j] = fmaxf(pv[2 * j] - q0, 0.f);
             rv[2 * j + 1] = fmaxf(pv[2 * j + 1] - q1, 0.f);
         }

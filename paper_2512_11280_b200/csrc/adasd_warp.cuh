@@ -8,7 +8,7 @@
 //          of the mass of what top-k left (the smallest most-probable set whose mass reaches
 //          top_p, ties at its edge included).
 // row_cutoff_kernel finds c for every needed row; the row passes then read a logit below its
-// row's c as -inf (apply_warp below), so entropy, JS distance, the accept ratio and every sample
+// row's c as -inf, so entropy, JS distance, the accept ratio and every sample
 // are those of the adjusted distribution.
 //
 // The search is a radix descent over the order-preserving integer image of the logits (16 bits
@@ -24,17 +24,6 @@
 #include "adasd_pdl.cuh"
 
 namespace adasd {
-
-// One row's adjustment as the row passes apply it.
-struct RowWarp {
-    float inv_t;    // 1 / temperature
-    float cut;      // logits below it are cut (-inf: none)
-};
-// -inf for a cut token, z / temperature for the others; NaN stays NaN (the row is unusable);
-// {1, -inf} changes nothing, bit for bit.
-__device__ __forceinline__ float apply_warp(float z, const RowWarp& w) {
-    return (z < w.cut) ? -INFINITY : z * w.inv_t;
-}
 
 struct CutParams {
     const void* z;

@@ -64,3 +64,38 @@ def test_the_largest_logit_is_chosen_however_low_it_is(torch, adasd, V, dtype, B
         ctx.draft_entropy(z[:, i], H, token_out=tok)            # no uniform: argmax
         assert (tok.cpu().numpy() == want[:, i]).all() and torch.isnan(H).all()
     assert ctx.status() == adasd.STATUS_NAN                     # (such rows have no distribution)
+
+
+@pytest.mark.parametrize("V,dtype,B,pad", [(64, synth.FP32, 2, 0), (1003, synth.FP32, 3, 1), (32000, synth.FP32, 2, 0), (8200, synth.FP32, 150, 3),
+                                           (128256, synth.FP32, 4, 0)])
+@pytest.mark.parametrize("offset", [0.0, 300.0, -5000.0])
+def test_vanilla_alpha_of_rows_with_a_large_offset(torch, adasd, V, dtype, B, pad, offset):
+    """A constant added to a row's logits changes nothing: p(x) / q(x) has to come from differences of logits.  fp32
+    logits around an offset o are multiples of ulp(o), exactly as both sides read them; what is left are the
+    roundings of (z - m) log2 e and log2 S, of at most 2^5 here: 2 * 2^-19 each of p and q, under 1e-5 of alpha.  Tokens drawn
+    from the residual agree with float64 where u lies further than that from an edge."""
+    K = 3
+    g = torch.Generator(device="cuda").manual_seed(V + B)
+    buf_d = torch.empty(B * K * (V + pad) + pad, device="cuda")
+    buf_t = torch.empty(B * (K + 1) * (V + pad) + pad, device="cuda")
+    zd = buf_d.as_strided((B, K, V), (K * (V + pad), V + pad, 1), pad)
+    zt = buf_t.as_strided((B, K + 1, V), ((K + 1) * (V + pad), V + pad, 1), pad)
+    zt.copy_(torch.randn(B, K + 1, V, generator=g, device="cuda") * 2 + offset)
+    zd.copy_(zt[:, :K] + torch.randn(B, K, V, generator=g, device="cuda") * 0.5)
+    x = torch.multinomial(torch.softmax(zd.reshape(-1, V).double(), -1), 1, generator=g).view(B, K).to(torch.int32)
+    u, ur = torch.full((B, K), 0.9, device="cuda"), torch.rand(B, generator=g, device="cuda")
+    al, nt = torch.zeros(B, dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+    alpha = torch.zeros(B, K, device="cuda")
+    ctx = adasd.Context(B, V, K, dtype=dtype, list_capacity=8)
+    ctx.vanilla_verify(zd, zt, x, u, ur, al, nt, alpha_out=alpha)
+    p, q = torch.softmax(zt.double(), -1), torch.softmax(zd.double(), -1)
+    i = x.long()[..., None]
+    want = (p[:, :K].gather(2, i) / q.gather(2, i))[..., 0].clamp(max=1.0)
+    assert ctx.status() == 0
+    assert (alpha.double() - want).abs().max() < 1e-5
+    for b in range(B):
+        w = int(al[b])
+        r = (p[b, w] - q[b, w]).clamp(min=0) if w < K else p[b, w]
+        c = torch.cumsum(r / r.sum(), 0)
+        t = int(nt[b])
+        assert float(c[t]) > float(ur[b]) - 1e-4 and (t == 0 or float(c[t - 1]) <= float(ur[b]) + 1e-4) and float(r[t]) > 0
