@@ -94,14 +94,17 @@ __device__ __forceinline__ PosTotals fold_position(const VerifyParams& p, const 
     t.vt = warp_max_f32(fmaxf(a0.x, b0.x));
     t.vd = warp_max_f32(fmaxf(a0.w, b0.w));
     const float w0 = ex2((a0.x - t.vt) * c1) * a0.y, w1 = ex2((b0.x - t.vt) * c1) * b0.y;
-    const float wd = ex2((a0.w - t.vd) * c1) * a1.x + ex2((b0.w - t.vd) * c1) * b1.x;
+    float d0 = ex2((a0.w - t.vd) * c1) * a1.x, d1 = ex2((b0.w - t.vd) * c1) * b1.x;
     const bool bad = __any_sync(0xFFFFFFFFu, (__float_as_uint(a1.z) | __float_as_uint(b1.z)) & 1u) || !(t.vt > kFloorL) || !(t.vd > kFloorL);
-    // running weights: lane by lane over the first 32 segments, then over the others
-    float i0 = w0, i1 = w1, Sd = wd;
+    // running weights: lane by lane over the first 32 segments, then over the others.  Lane 31's prefix adds the same
+    // pairs as the exchange of the draft row's sums, so that identical rows have identical totals and a distance of
+    // exactly 0
+    float i0 = w0, i1 = w1;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const float t0 = __shfl_up_sync(0xFFFFFFFFu, i0, o), t1 = __shfl_up_sync(0xFFFFFFFFu, i1, o);
-        Sd += __shfl_xor_sync(0xFFFFFFFFu, Sd, o);
+        d0 += __shfl_xor_sync(0xFFFFFFFFu, d0, o);
+        d1 += __shfl_xor_sync(0xFFFFFFFFu, d1, o);
         if (lane >= o) {
             i0 += t0;
             i1 += t1;
@@ -109,7 +112,7 @@ __device__ __forceinline__ PosTotals fold_position(const VerifyParams& p, const 
     }
     i1 += __shfl_sync(0xFFFFFFFFu, i0, 31);
     t.St = __shfl_sync(0xFFFFFFFFu, i1, 31);
-    t.Sd = Sd;
+    t.Sd = d1 + d0;
     t.sel = -1;
     t.base = 0.f;
     t.target = u * t.St;

@@ -99,3 +99,29 @@ def test_vanilla_alpha_of_rows_with_a_large_offset(torch, adasd, V, dtype, B, pa
         c = torch.cumsum(r / r.sum(), 0)
         t = int(nt[b])
         assert float(c[t]) > float(ur[b]) - 1e-4 and (t == 0 or float(c[t - 1]) <= float(ur[b]) + 1e-4) and float(r[t]) > 0
+
+
+# from a segment of several chunks to the most segments a position has (64), bf16 and fp32, on and off 16-byte boundaries
+@pytest.mark.parametrize("V,dtype,B,pad", [(600, synth.FP32, 3, 0), (32000, synth.FP32, 1, 0), (32000, synth.FP32, 4, 1), (128256, synth.FP32, 1, 0),
+                                           (128256, synth.FP32, 4, 3), (128256, synth.FP32, 16, 0), (128256, synth.BF16, 1, 1),
+                                           (128256, synth.BF16, 5, 3), (128256, synth.BF16, 2, 0)])
+def test_identical_rows_are_exactly_0_apart(torch, adasd, V, dtype, B, pad):
+    """Sec. 4.4: a distance of exactly 0 stays out of the lists, so it has to be exactly 0."""
+    K, tdt = 5, torch.bfloat16 if dtype == synth.BF16 else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(V + B)
+
+    def rows(n):
+        return torch.zeros(B * n * (V + pad) + 16, dtype=tdt, device="cuda").as_strided((B, n, V), (n * (V + pad), V + pad, 1), pad)
+    zt, zd = rows(K + 1), rows(K)
+    zt.copy_(torch.randn(B, K + 1, V, generator=g, device="cuda") * 2)
+    zd.copy_(zt[:, :K])
+    i32 = dict(dtype=torch.int32, device="cuda")
+    ctx = adasd.Context(B, V, K, dtype=dtype, list_capacity=64)
+    for warp in ((1.0, 0, 1.0), (0.7, 0, 0.9)):
+        ctx.set_warpers(*warp)
+        rec = ctx.new_record()
+        ctx.verify(zd, zt, torch.zeros((B, K), **i32), torch.rand(B, K + 1, generator=g, device="cuda"), torch.zeros(B, K, device="cuda"),
+                   torch.zeros(B, **i32), torch.zeros(B, **i32), record=rec)
+        assert (rec["jsd"] == 0).all() and (rec["dist"] == 0).all() and torch.equal(rec["H_d"], rec["H_t"][:, :K])
+    T, nE, nA, nR = ctx.get_thresholds()
+    assert int(nA.max()) == 0 and int(nR.max()) == 0 and ctx.status() == 0
