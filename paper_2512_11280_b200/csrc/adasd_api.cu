@@ -52,6 +52,10 @@ struct adasd_ctx {
     int seg_bits, stream_it;  // ... of which there are 2^seg_bits; iterations of a chunk
     bool cuts_on() const { return (top_k > 0 && top_k < cfg.V) || top_p < 1.f; }
     bool warp_on() const { return cuts_on() || temperature != 1.f; }
+    // The two kernels of aligned bf16 rows hold shifts and 2^t t in units of 1 / T: below this temperature a shift is off by
+    // whole powers of two (logits of 10: by 8), below 4e-9 that of a masked logit overflows.  The general kernels, 7 and
+    // 15 % slower on such rows, work on differences of logits.
+    bool tiny_temperature() const { return temperature < 1e-6f; }
 };
 
 namespace {
@@ -341,7 +345,7 @@ void draft_setup(adasd_ctx* c) {
 }
 // Large batches of aligned bf16 rows: the kernel whose warps split a row to 16 bytes.
 bool draft_rows(const adasd_ctx* c) {
-    return c->cfg.dtype == ADASD_BF16 && (c->cfg.V & 7) == 0 && c->cfg.V >= 8192 && c->draft_p <= 2 &&
+    return c->cfg.dtype == ADASD_BF16 && (c->cfg.V & 7) == 0 && c->cfg.V >= 8192 && c->draft_p <= 2 && !c->tiny_temperature() &&
            c->cfg.V <= kDMaxChunks * kDChunkUnits * 8 * c->draft_p * c->draft_nw;
 }
 template <int NW>
@@ -560,7 +564,7 @@ int launch_verify(adasd_ctx* ctx, const VerifyParams& p, cudaStream_t stream) {
     const bool vec = vec_ok(p.zd, ctx->cfg.dtype, {p.d_seq, p.d_row}) &&
                      vec_ok(p.zt, ctx->cfg.dtype, {p.t_seq, p.t_row});
     if (int rc = launch_round_cutoffs(ctx, p, stream)) return rc;
-    if (vec && ctx->fast.iter > 0) return fast_launch_iter(ctx, p, stream);
+    if (vec && ctx->fast.iter > 0 && !ctx->tiny_temperature()) return fast_launch_iter(ctx, p, stream);
     return ctx->cfg.dtype == ADASD_BF16 ? launch_sweep<__nv_bfloat16>(ctx, p, vec, stream) : launch_sweep<float>(ctx, p, vec, stream);
 }
 

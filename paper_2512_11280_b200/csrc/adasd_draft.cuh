@@ -113,7 +113,8 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
     DraftShared<NW>* const r0 = P > 1 ? cluster.map_shared_rank(&sh, 0) : &sh;
 
     // v: the largest logit so far (kFloorL while there is none): t = (z - v) log2 e is exactly 0 for it, so
-    // that a one-hot row gets S = 1, T = 0 and H = 0 exactly
+    // that a one-hot row gets S = 1, T = 0 and H = 0 exactly.  Under a temperature T adds up 2^t (z - v), scaled once
+    // at the end: z - v is finite, t for small temperatures is not
     float v = kFloorL;
     float top = -INFINITY;                                  // greedy drafting: the largest logit, finite but perhaps without
     int vi = -1;                                            // probability (a mask of the type's lowest value), and its index
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
             ph ^= 1u;
         }
         if (x > v && x > floor_v) {                         // a larger maximum: rescale what is summed
-            const float d = v > kFloorL ? (v - x) * c1 : kFloorL, f = ex2(d);
+            const float dz = v > kFloorL ? v - x : kFloorL, d = WARPED ? dz : dz * c1, f = ex2(dz * c1);
             T2.x = f * fmaf(d, S2.x + R2.x, T2.x);
             T2.y = f * fmaf(d, S2.y + R2.y, T2.y);
             S2.x *= f;
@@ -204,10 +205,10 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
             U::unpack(W[k], z);
 #pragma unroll
             for (int j = 0; j < NP; ++j) {
-                const float2 t = __fmul2_rn(__fadd2_rn(z[j], nv2), L2);
+                const float2 d = __fadd2_rn(z[j], nv2), t = __fmul2_rn(d, L2);
                 const float2 e = make_float2(ex2(t.x), ex2(t.y));
                 R2 = __fadd2_rn(R2, e);
-                T2 = __ffma2_rn(e, t, T2);
+                T2 = __ffma2_rn(e, WARPED ? d : t, T2);
             }
         }
         if (++in_run == cpr || c + 1 == nch) {
@@ -225,13 +226,15 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
         for (int c = cfail; c < min(cfail + kDRing, nch); ++c)
             if (!(expiring && c == 0))
                 mbar_wait_bounded(reinterpret_cast<uint64_t*>(&sh.bar[warp][c % kDRing]), (uint32_t)(c / kDRing) & 1u);
-    const float Sw = warp_sum(S2.x + S2.y), Tw = warp_sum(T2.x + T2.y);
+    const float Sw = warp_sum(S2.x + S2.y), Tw = (WARPED ? c1 : 1.f) * warp_sum(T2.x + T2.y);
     bad = __reduce_or_sync(0xFFFFFFFFu, bad);
     if (lane >= run && lane < kDRuns) r0->run[g][lane] = make_float2(kFloorL, 0.f);      // runs this warp does not have
     if (lane == 0) {
         r0->wpart[g] = make_float4(v, Sw, Tw, __uint_as_float(bad));
-        r0->wtop[g] = top;
-        r0->widx[g] = vi;
+        if (greedy) {
+            r0->wtop[g] = top;
+            r0->widx[g] = vi;
+        }
     }
     // totals and tables of every CTA are in rank 0's shared memory
     if (P > 1) cluster.sync();
@@ -243,7 +246,11 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
     const float4 none = make_float4(kFloorL, 0.f, 0.f, 0.f);
     const float4 e0 = lane < G ? sh.wpart[lane] : none, e1 = lane + 32 < G ? sh.wpart[lane + 32] : none;
     const float Mr = warp_max_f32(fmaxf(e0.x, e1.x));
-    const float d0 = (e0.x - Mr) * c1, d1 = (e1.x - Mr) * c1;
+    float d0 = (e0.x - Mr) * c1, d1 = (e1.x - Mr) * c1;
+    if (WARPED) {                                           // (finite: 0 times it occurs)
+        d0 = fmaxf(d0, kFloor);
+        d1 = fmaxf(d1, kFloor);
+    }
     const float w0 = ex2(d0) * e0.y, w1 = ex2(d1) * e1.y;
     const float S = warp_sum(w0 + w1);
     const float Tt = warp_sum(ex2(d0) * fmaf(d0, e0.y, e0.z) + ex2(d1) * fmaf(d1, e1.y, e1.z));

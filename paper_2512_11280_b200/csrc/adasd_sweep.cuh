@@ -185,13 +185,15 @@ __device__ __forceinline__ void publish_distance(const VerifyParams& p, int pos,
     if (p.user.dist) p.user.dist[id] = dist;
 }
 
-// Row sums of sweep 1 under the running maximum v (warp-wide; kFloorL: nothing finite so far).
+// Row sums of sweep 1 under the running maximum v (warp-wide; kFloorL: nothing finite so far).  Under a temperature T
+// adds up 2^t (z - v) and is scaled once a segment: z - v is finite, t for small temperatures is not.
+template <bool WARPED>
 struct RowSums {
     float v;
     float2 S, T;
     __device__ __forceinline__ void raise(float x, float floor_v, float c1) {      // a larger maximum: rescale
         if (x > v && x > floor_v) {
-            const float d = v > kFloorL ? (v - x) * c1 : kFloorL, f = ex2(d);
+            const float dz = v > kFloorL ? v - x : kFloorL, d = WARPED ? dz : dz * c1, f = ex2(dz * c1);
             T.x = f * fmaf(d, S.x, T.x);
             T.y = f * fmaf(d, S.y, T.y);
             S.x *= f;
@@ -206,10 +208,10 @@ struct RowSums {
         U::unpack(w, z);
 #pragma unroll
         for (int j = 0; j < U::N / 2; ++j) {
-            const float2 t = __fmul2_rn(__fadd2_rn(z[j], nv2), L2);
+            const float2 d = __fadd2_rn(z[j], nv2), t = __fmul2_rn(d, L2);
             const float2 e = make_float2(ex2(t.x), ex2(t.y));
             S = __fadd2_rn(S, e);
-            T = __ffma2_rn(e, t, T);
+            T = __ffma2_rn(e, WARPED ? d : t, T);
         }
     }
 };
@@ -495,7 +497,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
         };
 
         if (!SECOND) {
-            RowSums rt = {kFloorL, make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, rd = rt;
+            RowSums<WARPED> rt = {kFloorL, make_float2(0.f, 0.f), make_float2(0.f, 0.f)}, rd = rt;
             uint32_t bad = 0u;
             auto chunk = [&](auto bonus_c, auto edge_c, int ch, const unsigned char* sb) {
                 constexpr bool BONUS = decltype(bonus_c)::value, edge = decltype(edge_c)::value;
@@ -522,12 +524,12 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
                     uint4 Tw = unit_t(sb, k);
                     if (edge) mask(Tw, ch, k);
                     if (WARPED) U::cut(Tw, cut_t);
-                    rt.add<U>(Tw, nt2, L2);
+                    rt.template add<U>(Tw, nt2, L2);
                     if (!BONUS) {
                         uint4 Dw = unit_d(sb, k);
                         if (edge) mask(Dw, ch, k);
                         if (WARPED) U::cut(Dw, cut_d);
-                        rd.add<U>(Dw, nd2, L2);
+                        rd.template add<U>(Dw, nd2, L2);
                     }
                 }
             };
@@ -545,8 +547,8 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
                 issue(false);                        // the chunk has been read, its slot is free
             }
             if (!alive) bad = 1u;
-            const float St = warp_sum(rt.S.x + rt.S.y), Tt = warp_sum(rt.T.x + rt.T.y);
-            const float Sd = bonus ? St : warp_sum(rd.S.x + rd.S.y), Td = bonus ? Tt : warp_sum(rd.T.x + rd.T.y);
+            const float sc = WARPED ? c1 : 1.f, St = warp_sum(rt.S.x + rt.S.y), Tt = sc * warp_sum(rt.T.x + rt.T.y);
+            const float Sd = bonus ? St : warp_sum(rd.S.x + rd.S.y), Td = bonus ? Tt : sc * warp_sum(rd.T.x + rd.T.y);
             bad = __reduce_or_sync(0xFFFFFFFFu, bad);
             if (lane == 0) {
                 float4* w = reinterpret_cast<float4*>(q.seg1 + (size_t)pos * q.segs + seg);

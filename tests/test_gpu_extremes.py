@@ -125,3 +125,51 @@ def test_identical_rows_are_exactly_0_apart(torch, adasd, V, dtype, B, pad):
         assert (rec["jsd"] == 0).all() and (rec["dist"] == 0).all() and torch.equal(rec["H_d"], rec["H_t"][:, :K])
     T, nE, nA, nR = ctx.get_thresholds()
     assert int(nA.max()) == 0 and int(nR.max()) == 0 and ctx.status() == 0
+
+
+@pytest.mark.parametrize("V,dtype,B,pad", [(64, synth.FP32, 2, 0), (1003, synth.FP32, 5, 1), (32000, synth.FP32, 3, 0), (128256, synth.FP32, 2, 1), (5000, synth.BF16, 3, 1),
+                                           (8200, synth.BF16, 2, 0), (32000, synth.BF16, 150, 0), (128256, synth.BF16, 3, 0)])
+@pytest.mark.parametrize("T", [1e-3, 1e-9, 1e-10])
+@pytest.mark.parametrize("mask", ["inf", "lowest"])
+def test_temperatures_that_leave_only_the_largest_logits(torch, adasd, V, dtype, B, pad, T, mask):
+    """Any positive temperature is accepted: for 1e-9, (z - max) log2 e / T of a masked logit is beyond fp32.  Rows
+    whose every other token has no probability; entropies, distances and alphas are those of a few equal logits."""
+    K, tdt = 2, torch.bfloat16 if dtype == synth.BF16 else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(V + B)
+
+    def rows(n):
+        return torch.zeros(B * n * (V + pad) + 16, dtype=tdt, device="cuda").as_strided((B, n, V), (n * (V + pad), V + pad, 1), pad)
+    zt, zd = rows(K + 1), rows(K)
+    z = torch.randn(B, K + 1, V, generator=g, device="cuda").round(decimals=1) * 8
+    z[..., : V // 3] = -np.inf if mask == "inf" else torch.finfo(tdt).min
+    zt.copy_(z)
+    zd.copy_(z[:, :K])
+    zd[:, 1] = zd[:, 1].roll(V // 2, -1)                        # another largest token
+    T = float(np.float32(T))
+    i32 = dict(dtype=torch.int32, device="cuda")
+    ctx = adasd.Context(B, V, K, dtype=dtype, list_capacity=8)
+    ctx.set_warpers(T, 0, 1.0)
+    p, q = torch.softmax(zt.double() / T, -1), torch.softmax(zd.double() / T, -1)
+    ent = lambda w: -(w * torch.log(w.clamp(min=1e-300))).sum(-1)
+    H, tok = torch.zeros(B, device="cuda"), torch.zeros(B, **i32)
+    lse = torch.zeros(B, device="cuda")
+    x = torch.zeros((B, K), **i32)
+    for i in range(K):
+        ctx.draft_entropy(zd[:, i], H, u=torch.rand(B, generator=g, device="cuda"), token_out=tok, lse_out=lse)
+        assert (H.double() - ent(q[:, i])).abs().max() < 1e-4
+        want = torch.logsumexp(zd[:, i].double() / T, -1)
+        assert ((lse.double() - want) / want.abs().clamp(min=1)).abs().max() < 1e-6
+        x[:, i] = tok
+    assert (x >= 0).all() and (q.gather(2, x.long()[..., None]) > 0).all()
+    rec, al, nt = ctx.new_record(), torch.zeros(B, **i32), torch.zeros(B, **i32)
+    ctx.verify(zd, zt, x, torch.rand(B, K + 1, generator=g, device="cuda"), torch.rand(B, K, generator=g, device="cuda"), al, nt, record=rec)
+    assert (rec["H_d"].double() - ent(q)).abs().max() < 1e-4 and (rec["H_t"].double() - ent(p)).abs().max() < 1e-4
+    m = 0.5 * (p[:, :K] + q)
+    assert (rec["jsd"].double() - (ent(m) - 0.5 * (ent(p[:, :K]) + ent(q)))).abs().max() < 1e-4
+    assert (rec["dist"][:, 0] == 0).all() and (p.gather(2, rec["y"].long()[..., None]) > 0).all()
+    alpha = torch.zeros(B, K, device="cuda")
+    ctx.vanilla_verify(zd, zt, x, torch.full((B, K), 0.5, device="cuda"), torch.rand(B, generator=g, device="cuda"), al, nt, alpha_out=alpha)
+    want = (p[:, :K].gather(2, x.long()[..., None]) / q.gather(2, x.long()[..., None]))[..., 0].clamp(max=1.0)
+    assert (alpha.double() - want).abs().max() < 1e-4
+    assert all(float(p[b, int(al[b]), int(nt[b])]) > 0 for b in range(B))
+    assert ctx.status() == 0
