@@ -218,7 +218,7 @@ class Context:
         self._draft_entropy, self._verify = L.adasd_draft_entropy, L.adasd_verify
         self._vanilla_verify, self._greedy_verify = L.adasd_vanilla_verify, L.adasd_greedy_verify
         self._raw_stream = torch._C._cuda_getCurrentRawStream
-        self._rec_key, self._rec = None, None      # the last record's addresses and their struct
+        self._rec = None                           # the last record's addresses and their struct
 
     def close(self) -> None:
         if getattr(self, "handle", None):
@@ -275,14 +275,16 @@ class Context:
             raise AdasdError(rc, "adasd_draft_entropy")
 
     def _record_ref(self, rec: Optional[dict]):
-        """The C struct of a record of device tensors; the struct of the last record is kept and
-        used again as long as the addresses are the same."""
+        """The C struct of a record of device tensors; the struct of the last record is used again
+        when the addresses are the same.  Addresses and struct are kept as one object, and the call
+        works on its own reference to it: another thread's record never gets into this call."""
         if rec is None:
             return None
         key = [(k, v.data_ptr()) if v is not None else (k, None) for k, v in rec.items()]
-        if key != self._rec_key:
-            self._rec, self._rec_key = C.byref(RoundRecord(**dict(key))), key
-        return self._rec
+        last = self._rec
+        if last is None or last[0] != key:
+            self._rec = last = (key, C.byref(RoundRecord(**dict(key))))
+        return last[1]
 
     def verify(self, draft_logits, target_logits, draft_tokens, u_target, u_accept, accept_len,
                next_token, draft_len=None, record: Optional[dict] = None,
