@@ -89,12 +89,12 @@ __device__ __forceinline__ void unpack16(const uint4& r, float (&x)[4]) {
 // Unit u of a row = elements [u*N, u*N+N).  Elements at or beyond V read as -inf.
 // VEC: the row base and stride are 16-byte aligned, so full units take one 16-byte load.
 template <typename T, bool VEC>
-__device__ __forceinline__ void load_unit(const T* __restrict__ row, int u, int V,
+__device__ __forceinline__ void load_unit(const T* row, int u, int V,
                                           float (&x)[Elt<T>::N]) {
     constexpr int N = Elt<T>::N;
     const int v0 = u * N;
     if (VEC && v0 + N <= V) {
-        uint4 r = __ldg(reinterpret_cast<const uint4*>(row + v0));
+        const uint4 r = *reinterpret_cast<const uint4*>(row + v0);
         unpack16(r, x);
     } else {
 #pragma unroll

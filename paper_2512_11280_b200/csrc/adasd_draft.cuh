@@ -102,12 +102,12 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
     float u_row = 0.f, tg_row = 0.f;
     int32_t len_row = 0;
     if (g == 0) {
-        if (p.u != nullptr) u_row = __ldg(p.u + b);
+        if (p.u != nullptr) u_row = __ldcg(p.u + b);
         tg_row = p.st.T_G[b];
         if (p.draft_len) len_row = p.draft_len[b];          // (only this row's CTA ever writes it)
     }
     const float c1 = WARPED ? p.c1 : kLog2e;                // log2 e / temperature
-    const typename U::Cut cut = U::make_cut((WARPED && p.cut) ? __ldg(p.cut + b) : -INFINITY);
+    const typename U::Cut cut = U::make_cut((WARPED && p.cut) ? __ldcg(p.cut + b) : -INFINITY);
     const bool greedy = p.argmax != 0;
     if (P > 1) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     DraftShared<NW>* const r0 = P > 1 ? cluster.map_shared_rank(&sh, 0) : &sh;
@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_step_kernel(
             uint4 W[IT + 1];
 #pragma unroll
             for (int k = 0; k < IT + (ALIGNED ? 0 : 1); ++k)
-                W[k] = ub + k < g1 ? __ldg(row + ub + k) : U::none4();
+                W[k] = ub + k < g1 ? __ldcg(row + ub + k) : U::none4();
             float e[IT][N], ls = 0.f;
 #pragma unroll
             for (int k = 0; k < IT; ++k) {

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_stream_kerne
     float u_row = 0.f, tg_row = 0.f;
     int32_t len_row = 0;
     if (active && rank == 0 && warp == 0) {
-        if (p.u != nullptr) u_row = __ldg(p.u + b);
+        if (p.u != nullptr) u_row = __ldcg(p.u + b);
         tg_row = p.st.T_G[b];
         if (p.draft_len) len_row = p.draft_len[b];          // (only this row's CTA ever writes it)
     }
@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_stream_kerne
     };
     // adjusted distribution: t = (z - max) log2 e / T, logits below the row's cutoff count as -inf
     const float c1 = WARPED ? p.c1 : kLog2e;
-    const uint32_t cut2 = (WARPED && p.cut) ? cut_pair(__ldg(p.cut + b)) : kNoCut2;
+    const uint32_t cut2 = (WARPED && p.cut) ? cut_pair(__ldcg(p.cut + b)) : kNoCut2;
     float M = kFloorL;                                   // running shift (log2 domain)
     // the largest logit so far (0 while there is none): t = (z - vM) log2 e is exactly 0 for it,
     // so that a one-hot row gets S = 1, T = 0 and H = 0 exactly
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(NW * 32, NW == kDW ? 2 : 1) draft_stream_kerne
 #pragma unroll
                     for (int i = 0; i < 8; ++i) {
                         const int u = u0 + lane * 8 + i;
-                        Wq[i] = u < u1 ? __ldg(row + u) : make_uint4(0xF149F149u, 0xF149F149u, 0xF149F149u, 0xF149F149u);
+                        Wq[i] = u < u1 ? __ldcg(row + u) : make_uint4(0xF149F149u, 0xF149F149u, 0xF149F149u, 0xF149F149u);
                         if (WARPED) bcut8(Wq[i], cut2);
                     }
                     float wt[8][8];

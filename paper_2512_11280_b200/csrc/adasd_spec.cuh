@@ -265,7 +265,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
 
     // first active position among start, start + ncl, ... (32 candidates per round)
     auto window = [&](int b) -> int {
-        int kt = p.draft_len ? __ldg(p.draft_len + b) : Kmax;
+        int kt = p.draft_len ? __ldcg(p.draft_len + b) : Kmax;
         return max(0, min(kt, Kmax));
     };
     auto scan_from = [&](int start) -> PosRef {
@@ -300,8 +300,8 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
             if (r.pos < total) {
                 const int b = r.pos / K1, i = r.pos - b * K1;
                 c.bonus = (i == r.kt) ? 1 : 0;
-                c.cut_t = (WARPED && p.cut_t) ? cut_pair(__ldg(p.cut_t + r.pos)) : kNoCut2;
-                c.cut_d = (WARPED && p.cut_d && !c.bonus) ? cut_pair(__ldg(p.cut_d + (size_t)b * Kmax + i)) : kNoCut2;
+                c.cut_t = (WARPED && p.cut_t) ? cut_pair(__ldcg(p.cut_t + r.pos)) : kNoCut2;
+                c.cut_d = (WARPED && p.cut_d && !c.bonus) ? cut_pair(__ldcg(p.cut_d + (size_t)b * Kmax + i)) : kNoCut2;
                 c.src_t = (unsigned long long)(reinterpret_cast<const __nv_bfloat16*>(p.zt) + (long long)b * p.t_seq +
                                                (long long)i * p.t_row + (size_t)cu0 * 8);
                 c.src_d = (unsigned long long)(reinterpret_cast<const __nv_bfloat16*>(p.zd) + (long long)b * p.d_seq +
@@ -809,7 +809,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
             // per-position scalars, fetched before the wait so that they are there after it
             const PosCtx& pcn = sh.pc[n & (kSPosRing - 1)];
             const bool bonus = pcn.bonus != 0;
-            const float u_samp = __ldg(p.u_target + pcn.pos);
+            const float u_samp = __ldcg(p.u_target + pcn.pos);
 
             // the CTA's totals from its compute warps, sent to every CTA of the cluster
             wait_cta(&sh.entry_bar[par], ph);

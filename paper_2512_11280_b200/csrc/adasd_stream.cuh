@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
     auto load_block = [&]() {
         const int b = blk_b + lane;
         int kt = K;
-        if (b < p.B && p.draft_len) kt = max(0, min(__ldg(p.draft_len + b), K));
+        if (b < p.B && p.draft_len) kt = max(0, min(__ldcg(p.draft_len + b), K));
         blk_cnt = b < p.B ? kt + 1 + (rows_of_d ? kt : 0) : 0;
         blk_incl = blk_cnt;
 #pragma unroll
@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(320, 2) row_stream_kernel(StreamParams p) {
             d.ch0 = ich;
             d.ch1 = ich1;
             d.cut = -INFINITY;
-            if (WARPED && p.cut_t) d.cut = tgt ? __ldg(p.cut_t + (size_t)b * K1 + i) : __ldg(p.cut_d + (size_t)b * K + i);
+            if (WARPED && p.cut_t) d.cut = tgt ? __ldcg(p.cut_t + (size_t)b * K1 + i) : __ldcg(p.cut_d + (size_t)b * K + i);
         }
         if (lane == 0) items[warp][n_items & (kRItems - 1)] = d;
         ++n_items;
@@ -407,17 +407,17 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
     const float c1 = p.c1;
     pdl_trigger();
 
-    int kt = p.draft_len ? __ldg(p.draft_len + b) : K;
+    int kt = p.draft_len ? __ldcg(p.draft_len + b) : K;
     kt = max(0, min(kt, K));
     const T* const rt = reinterpret_cast<const T*>(p.zt) + (long long)b * p.t_seq;
     const T* const rd = reinterpret_cast<const T*>(p.zd) + (long long)b * p.d_seq;
     float u_acc = 0.f, ztx = 0.f, zdx = 0.f;
     bool x_ok = false;
-    const float u_res = __ldg(p.u_resample + b);
+    const float u_res = __ldcg(p.u_resample + b);
     if (warp == 0 && lane < kt) {
         const size_t idd = (size_t)b * K + lane;
-        u_acc = __ldg(p.u_accept + idd);
-        const int xi = __ldg(p.x + idd);
+        u_acc = __ldcg(p.u_accept + idd);
+        const int xi = __ldcg(p.x + idd);
         x_ok = xi >= 0 && xi < p.V;
         if (x_ok) {
             ztx = to_f32(rt[(long long)lane * p.t_row + xi]);
@@ -484,8 +484,8 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
 
     // p and max(0, p - q) of unit u of the two rows
     const float2 c2 = pair2(c1), nmt2 = pair2(-mt.x), nst2 = pair2(-mt.y), nmd2 = pair2(-md.x), nsd2 = pair2(-md.y);
-    const typename U::Cut cut_t = U::make_cut(p.cut_t ? __ldg(p.cut_t + (size_t)b * K1 + i) : -INFINITY);
-    const typename U::Cut cut_d = U::make_cut((p.cut_d && !bonus) ? __ldg(p.cut_d + (size_t)b * K + i) : -INFINITY);
+    const typename U::Cut cut_t = U::make_cut(p.cut_t ? __ldcg(p.cut_t + (size_t)b * K1 + i) : -INFINITY);
+    const typename U::Cut cut_d = U::make_cut((p.cut_d && !bonus) ? __ldcg(p.cut_d + (size_t)b * K + i) : -INFINITY);
     const int NU = (p.V + N - 1) / N, NI = (NU + 31) >> 5;
     struct Row {
         const uint4* base;
@@ -501,8 +501,8 @@ __global__ void __launch_bounds__(kVThreads, 4) vanilla_finish_kernel(VanillaPar
     };
     const Row row_t = row_of(rt + (long long)i * p.t_row), row_d = row_of(rd + (long long)min(i, K - 1) * p.d_row);
     auto load = [&](const Row& r, int u) -> uint4 {
-        uint4 w = u < r.g1 ? __ldg(r.base + u) : U::none4();
-        if (!ALIGNED) w = U::realign(w, u + 1 < r.g1 ? __ldg(r.base + u + 1) : U::none4(), r.shift);
+        uint4 w = u < r.g1 ? r.base[u] : U::none4();
+        if (!ALIGNED) w = U::realign(w, u + 1 < r.g1 ? r.base[u + 1] : U::none4(), r.shift);
         return w;
     };
     auto weights = [&](uint4 a, uint4 d, int u, float (&pv)[N], float (&rv)[N]) {
@@ -697,9 +697,9 @@ __global__ void __launch_bounds__(kGThreads) greedy_finish_kernel(GreedyParams p
     const int b = (int)blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int K = p.Kmax, K1 = K + 1, R = 2 * K + 1, segs = 1 << p.seg_bits;
     pdl_trigger();
-    int kt = p.draft_len ? __ldg(p.draft_len + b) : K;
+    int kt = p.draft_len ? __ldcg(p.draft_len + b) : K;
     kt = max(0, min(kt, K));
-    const int x = lane < kt ? __ldg(p.x + (size_t)b * K + lane) : 0;
+    const int x = lane < kt ? __ldcg(p.x + (size_t)b * K + lane) : 0;
     pdl_wait();
     if (b == 0 && threadIdx.x == 0) *p.next = 0u;
     constexpr int W = kGThreads / 32;

@@ -281,7 +281,7 @@ __device__ __noinline__ ItemRows sweep_item(const VerifyParams& p, const SweepTa
             uint32_t blk_rank = w->blk_rank;
             int blk_b = w->blk_b, cnt, incl;
             for (;;) {
-                cnt = blk_b + lane < p.B ? max(0, min(__ldg(p.draft_len + blk_b + lane), K)) + 1 : 0;
+                cnt = blk_b + lane < p.B ? max(0, min(__ldcg(p.draft_len + blk_b + lane), K)) + 1 : 0;
                 incl = cnt;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -309,7 +309,7 @@ __device__ __noinline__ ItemRows sweep_item(const VerifyParams& p, const SweepTa
         const int pos = b * K1 + i;
         if (SECOND && bonus) {
             pdl_wait();                              // (the warp's first item is described before the wait)
-            const PosTotals t = fold_position<WARPED>(p, q, pos, __ldg(p.u_target + pos));
+            const PosTotals t = fold_position<WARPED>(p, q, pos, __ldcg(p.u_target + pos));
             const bool none = t.sel < 0;
             if (seg == 0) {
                 publish_entropies<WARPED>(p, q, pos, true, none, t.vt, t.vd);
@@ -342,8 +342,8 @@ __device__ __noinline__ ItemRows sweep_item(const VerifyParams& p, const SweepTa
         const unsigned long long qd = ad - (unsigned long long)d.mt * sizeof(T);
         const unsigned long long bd = ALIGNED ? ad : qd & ~15ull;
         d.sd = ALIGNED ? 0 : (int)((qd & 15ull) / sizeof(T));
-        d.cut_t = (WARPED && p.cut_t) ? __ldg(p.cut_t + pos) : -INFINITY;
-        d.cut_d = (WARPED && p.cut_d && !bonus) ? __ldg(p.cut_d + (size_t)b * K + i) : -INFINITY;
+        d.cut_t = (WARPED && p.cut_t) ? __ldcg(p.cut_t + pos) : -INFINITY;
+        d.cut_d = (WARPED && p.cut_d && !bonus) ? __ldcg(p.cut_d + (size_t)b * K + i) : -INFINITY;
         const int e0 = d.sd + d.mt;                  // elements between bd and the draft row
         r.src = lane == 0 ? bt : bd;
         r.glo = lane == 0 || ALIGNED ? 0 : e0 / N;
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
     // active positions of the round (i <= K_b)
     uint32_t P = 0;
     if (p.draft_len) {
-        for (int b = lane; b < p.B; b += 32) P += (uint32_t)max(0, min(__ldg(p.draft_len + b), K)) + 1u;
+        for (int b = lane; b < p.B; b += 32) P += (uint32_t)max(0, min(__ldcg(p.draft_len + b), K)) + 1u;
         P = __reduce_add_sync(0xFFFFFFFFu, P);
     } else {
         P = (uint32_t)p.B * (uint32_t)(K + 1);
@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) sweep_kernel(const __grid_co
             run = c.base;
             target = c.target;
         } else {
-            const PosTotals t = fold_position<WARPED>(p, q, pos, __ldg(p.u_target + pos));
+            const PosTotals t = fold_position<WARPED>(p, q, pos, __ldcg(p.u_target + pos));
             none = t.sel < 0;
             vt = t.vt;
             run = t.base;

@@ -102,8 +102,8 @@ __global__ void __launch_bounds__(kSelThreads, 3) row_cutoff_select_kernel(CutPa
     const int g1 = (shift + p.V + N - 1) / N;        // granules that hold elements: [0, g1)
     const int NU = (p.V + N - 1) / N, step = P * kSelThreads, u0 = rank * kSelThreads + tid;
     auto unit = [&](int u) -> uint4 {                // elements u N ..; those past the end read as -inf
-        uint4 w = __ldg(base + u);
-        if (!ALIGNED) w = U::realign(w, u + 1 < g1 ? __ldg(base + u + 1) : U::none4(), shift);
+        uint4 w = base[u];
+        if (!ALIGNED) w = U::realign(w, u + 1 < g1 ? base[u + 1] : U::none4(), shift);
         if (u == NU - 1 && u * N + N > p.V) U::mask(w, 0, p.V - u * N);
         return w;
     };

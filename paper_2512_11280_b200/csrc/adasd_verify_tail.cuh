@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(kTailThreads) verify_tail_kernel(TailParams p)
     const int Kmax = p.cfg.Kmax;
     pdl_trigger();
 
-    int K_t = p.draft_len ? __ldg(p.draft_len + b) : Kmax;
+    int K_t = p.draft_len ? __ldcg(p.draft_len + b) : Kmax;
     K_t = max(0, min(K_t, Kmax));
     const int nA0 = p.st.nA[b], nR0 = p.st.nR[b];
     double sA = 0.0, sA2 = 0.0, sE = 0.0, sR = 0.0, sR2 = 0.0;

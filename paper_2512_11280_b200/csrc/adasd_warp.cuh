@@ -311,7 +311,7 @@ __global__ void __launch_bounds__(kHistThreads, 1) row_cutoff_hist_kernel(CutPar
             for (int u0 = tid; u0 < NUF; u0 += 4 * kHistThreads) {
                 uint4 r[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) r[i] = __ldg(zq + min(u0 + i * kHistThreads, NUF - 1));
+                for (int i = 0; i < 4; ++i) r[i] = zq[min(u0 + i * kHistThreads, NUF - 1)];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     if (u0 + i * kHistThreads < NUF) {
