@@ -284,11 +284,11 @@ cudaError_t stream_prepare_it() {
 template <typename T, bool ALIGNED>
 cudaError_t stream_prepare(int it) { return it == 8 ? stream_prepare_it<T, ALIGNED, 8>() : stream_prepare_it<T, ALIGNED, 2>(); }
 
-// Launch with programmatic stream serialisation: the kernel may become resident while the one ahead of
+// early: launch with programmatic stream serialisation: the kernel may become resident while the one ahead of
 // it is still running (it waits before it reads what that one wrote).  cs: CTAs per cluster; 0: the kernel
 // uses no cluster.  (A kernel that uses cluster-scope instructions gets the attribute even for clusters of one.)
 template <typename K, typename... Args>
-int launch_pdl(K kernel, int grid, int threads, int smem, int cs, cudaStream_t stream, const Args&... args) {
+int launch_kernel(bool early, K kernel, int grid, int threads, int smem, int cs, cudaStream_t stream, const Args&... args) {
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
     lc.gridDim = dim3((unsigned)grid, 1, 1);
@@ -297,7 +297,7 @@ int launch_pdl(K kernel, int grid, int threads, int smem, int cs, cudaStream_t s
     lc.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = (unsigned)cs;
     attr[1].val.clusterDim.y = 1;
@@ -306,6 +306,10 @@ int launch_pdl(K kernel, int grid, int threads, int smem, int cs, cudaStream_t s
     lc.numAttrs = cs > 0 ? 2 : 1;
     CUDA_TRY(cudaLaunchKernelEx(&lc, kernel, args...));
     return ADASD_OK;
+}
+template <typename K, typename... Args>
+int launch_pdl(K kernel, int grid, int threads, int smem, int cs, cudaStream_t stream, const Args&... args) {
+    return launch_kernel(true, kernel, grid, threads, smem, cs, stream, args...);
 }
 
 template <typename T, bool ALIGNED, int IT>
@@ -476,11 +480,20 @@ int launch_cutoffs(adasd_ctx* ctx, CutParams c, const CutParams* second, cudaStr
     const bool vec2 = !second || vec_ok(second->z, ctx->cfg.dtype, {second->seq_stride, second->row_stride});
     CutParams c2 = second ? *second : c;
     const long long rows = (long long)c.B * (c.R + (second ? second->R : 0));
-    const bool select = c.top_k > 0 && c.top_k < c.V && c.top_k <= kSelMaxK && c.V >= kSelMinV && rows <= 0x7FFFFFFF / kSelMaxP;
+    // top-k on: selection, a row over as many CTAs as are resident at once; it flags what it cannot do
+    int P = 1;
+    while (P < kSelMaxP && rows * P * 2 <= 3LL * ctx->sm_count) P *= 2;
+    // ... up to a k where it is the faster one.  It compares its candidates, a few times k, with one another.  Against the
+    // histogram of aligned bf16 rows, us a draft call of random rows with a top-p cut behind it: V=128256, 32 rows, k=200
+    // 38 / 47, k=256 46 / 39; V=32000 k=200, 8 rows 28 / 36, 32 rows 39 / 37, 256 rows 42 / 63; and without top-p, where the
+    // histogram is a count, 32 rows k=20 23 / 22, k=100 26 / 21, 256 rows k=100 26 / 31.  Up to 200 the candidates fit the
+    // list even of a row sorted by its logits, which has the most (five times k); such rows lose (V=32000 k=64 33 / 35, k=200
+    // 129 / 36).  Against the radix descent: always, unless the few groups of a row with one CTA leave so many
+    // candidates that it hands rows over (256 rows, V=32000, k=400 66 / 146, k=512 318 / 228).
+    const bool histogram = bf && vec1 && vec2 && ctx->cut_hist;
+    const int k_most = !histogram ? std::min(kSelMaxK, 448 * P) : c.V >= 65536 || c.top_p < 1.f || P == 1 ? 200 : 64;
+    const bool select = c.top_k > 0 && c.top_k < c.V && c.top_k <= k_most && c.V >= kSelMinV && rows <= 0x7FFFFFFF / kSelMaxP;
     if (select) {
-        // top-k on: selection, a row over as many CTAs as are resident at once; it flags what it cannot do
-        int P = 1;
-        while (P < kSelMaxP && rows * P * 2 <= 3LL * ctx->sm_count) P *= 2;
         const int g = (int)(rows * P);
         const bool aligned = vec1 && vec2;
         int rc;
@@ -505,13 +518,16 @@ int launch_cutoffs(adasd_ctx* ctx, CutParams c, const CutParams* second, cudaStr
             q.only_flagged = 1;
         }
         const int grid = (int)std::min<long long>(n, 2LL * ctx->sm_count);
+        // (early only where it has next to nothing to do: 64 rows of 128256 fp32 logits took 904 instead of 400 us, packed on the
+        // SMs beside the draft step ahead)
+        const bool early = q.only_flagged != 0;
         int rc;
         if (bf)
-            rc = vec ? launch_pdl(row_cutoff_kernel<__nv_bfloat16, true>, grid, kCutThreads, 0, 0, stream, q)
-                     : launch_pdl(row_cutoff_kernel<__nv_bfloat16, false>, grid, kCutThreads, 0, 0, stream, q);
+            rc = vec ? launch_kernel(early, row_cutoff_kernel<__nv_bfloat16, true>, grid, kCutThreads, 0, 0, stream, q)
+                     : launch_kernel(early, row_cutoff_kernel<__nv_bfloat16, false>, grid, kCutThreads, 0, 0, stream, q);
         else
-            rc = vec ? launch_pdl(row_cutoff_kernel<float, true>, grid, kCutThreads, 0, 0, stream, q)
-                     : launch_pdl(row_cutoff_kernel<float, false>, grid, kCutThreads, 0, 0, stream, q);
+            rc = vec ? launch_kernel(early, row_cutoff_kernel<float, true>, grid, kCutThreads, 0, 0, stream, q)
+                     : launch_kernel(early, row_cutoff_kernel<float, false>, grid, kCutThreads, 0, 0, stream, q);
         if (rc != ADASD_OK) return rc;
     }
     return ADASD_OK;

@@ -25,7 +25,7 @@ constexpr int kSelThreads = 512;
 constexpr int kSelMaxP = 8;
 constexpr int kSelList = 1024;
 constexpr int kSelMinV = 4096;                       // shorter rows: the radix descent
-constexpr int kSelMaxK = 512;                        // at least two group maxima for each of the k
+constexpr int kSelMaxK = 512;                        // (the rule that chooses this kernel asks for less on some rows)
 
 // Whether a unit has an element at or above tau.
 template <typename T>

@@ -46,3 +46,34 @@ def test_top_k_keeps_exactly_the_k_largest_and_their_ties(torch, V, dtype, k, B)
     ent = -(q * torch.log(q.clamp(min=1e-300))).sum(-1)
     assert (lse.double() - want).abs().max() < 1e-4 and (H.double() - ent).abs().max() < 1e-4
     assert ctx.status() == 0
+
+
+# either side of the k where another kernel finds the cutoffs, on rows that keep to 16-byte boundaries and rows that do not
+@pytest.mark.parametrize("V,dtype,ks", [(8200, synth.BF16, (64, 65, 200, 201)), (65536, synth.BF16, (200, 201)), (8200, synth.FP32, (448, 449, 512, 513))])
+@pytest.mark.parametrize("top_p", [1.0, 0.9])
+@pytest.mark.parametrize("B", [2, 250])
+def test_every_route_to_a_cutoff_keeps_the_same_tokens(torch, V, dtype, ks, top_p, B):
+    import oracle
+    import paper_2512_11280_b200 as adasd
+    tdt = torch.bfloat16 if dtype == synth.BF16 else torch.float32
+    z = (torch.randn(B, V, generator=torch.Generator(device="cuda").manual_seed(V + B), device="cuda") * 2).to(tdt)
+    z[1] = z[1].sort(descending=True).values
+    off = torch.zeros(B * (V + 1) + 16, dtype=tdt, device="cuda").as_strided((B, V), (V + 1, 1), 1)
+    off.copy_(z)
+    ctx = adasd.Context(B, V, 1, dtype=dtype, list_capacity=8)
+    for k in ks:
+        ctx.set_warpers(1.0, k, top_p)
+        out = []
+        for rows in (z, off):
+            H, lse = torch.zeros(B, device="cuda"), torch.zeros(B, device="cuda")
+            ctx.draft_entropy(rows, H, lse_out=lse)
+            out.append((H, lse))
+        assert ctx.status() == 0
+        for b in (0, 1, B - 1):
+            row = z[b].view(torch.int16).cpu().numpy().view(np.uint16) if dtype == synth.BF16 else z[b].cpu().numpy()
+            zw, _, band = oracle.warp(row, 1.0, k, float(np.float32(top_p)), band=5e-7)
+            if band:                                           # a top-p decision too close to call
+                continue
+            o = oracle.draft_step(zw, 0.5, 0.0)
+            for H, lse in out:
+                assert abs(float(H[b]) - o["H"]) < 1e-4 and abs(float(lse[b]) - o["lse"]) < 1e-4, (k, b)
