@@ -142,12 +142,20 @@ def verify_launches(wl) -> int:
 VANILLA_LAUNCHES = 2    # adasd_vanilla_verify: the rows' log-sum-exps, accept test with sampling
 
 
-def cutoff_launches(args, rounds: bool) -> int:
-    """Kernels that find the cutoffs of a draft call's rows or of a round's (target and draft rows): with top-k
-    a selection over all rows at once, else a histogram per set of rows; then a radix kernel per set for
-    the rows they hand over."""
-    top_k = args.warpers[1] > 0
-    return (3 if top_k else 4) if rounds else 2
+def cutoff_launches(args, wl, rounds: bool, sm_count: int = 148) -> int:
+    """Kernels that find the cutoffs of a draft call's rows or of a round's (target and draft rows): a selection over
+    all rows at once, or for aligned bf16 rows a histogram per set of rows, or nothing; then a radix kernel per set
+    for the rows that are left.  The rule is launch_cutoffs' in csrc/adasd_api.cu."""
+    _, k, p = args.warpers
+    histogram = wl.dtype == synth.BF16 and wl.V % 8 == 0
+    rows, P = wl.B * (2 * wl.K + 1 if rounds else 1), 1
+    while P < 8 and rows * P * 2 <= 3 * sm_count:
+        P *= 2
+    k_most = (200 if wl.V >= 65536 or p < 1 or P == 1 else 64) if histogram else min(512, 448 * P)
+    sets = 2 if rounds else 1
+    if 0 < k < wl.V and k <= k_most and wl.V >= 4096:
+        return 1 + sets
+    return 2 * sets if histogram else sets
 
 
 # ------------------------------------------------------------------------------ N ranks
@@ -354,7 +362,7 @@ def run_ours(args) -> dict:
                 "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": h_out.numel() * 4,
                 "steps": e2e_steps, "ms_per_step": e2e_ms / e2e_steps},
         "gpu_launches": args.steps * (K + verify_launches(wl) + VANILLA_LAUNCHES
-                                      + (K * cutoff_launches(args, False) + 2 * cutoff_launches(args, True) if cuts_on(args, wl) else 0)),
+                                      + (K * cutoff_launches(args, wl, False) + 2 * cutoff_launches(args, wl, True) if cuts_on(args, wl) else 0)),
         "clocks": clocks,
         "roofline": {"bound": "hbm", "kernel": "adasd_verify", "achieved": achieved, "peak": peak,
                      "unit": "GB/s", "frac": achieved / peak, "peak_kind": f"of {peak_kind}",
