@@ -20,9 +20,12 @@
  *     gen_only_update, get_thresholds, reset) only enqueue kernels on `stream`: they never allocate,
  *     free or synchronise.  create/destroy/state_export/state_import/status do.
  *   - Logits are row-major with contiguous vocabulary; strides are in ELEMENTS.
- *     bf16 or fp32 as fixed at create time.  Rows whose base address and stride are
- *     multiples of 16 bytes take the vectorised path; anything else still works
- *     through a scalar path.
+ *     bf16 or fp32 as fixed at create time.  Rows may start at any multiple of their element
+ *     size; they are copied by the aligned 16-byte granules that hold them, so that up to 14
+ *     bytes before a row's first element and after its last are read (never used, and never
+ *     beyond the page).  A caller who cuts buffers out of a larger one, or watches reads of
+ *     its memory, should know.  Rows whose base address and stride are multiples of 16 bytes
+ *     read nothing but themselves and the rest of the last granule, and are faster.
  *   - Uniforms are fp32 in [0,1), supplied by the caller (the library draws nothing).
  *   - Entropy, log-sum-exp and the JS divergence are in nats; the JS distance is
  *     sqrt(D_JS / ln 2), i.e. in [0,1].
@@ -72,7 +75,7 @@ extern "C" {
 #define ADASD_STATIC_MAX_POSITIONS 16384   /* B * (Kmax + 1) per call */
 
 /* flags of adasd_verify */
-#define ADASD_FUSE_UPDATE 1u     /* run the list appends and the T_G update in the same launch */
+#define ADASD_FUSE_UPDATE 1u     /* run the list appends and the T_G update in the same call */
 
 typedef struct adasd_ctx adasd_ctx; /* opaque; owns the per-sequence adaptive state */
 
@@ -85,7 +88,9 @@ typedef struct {
     int32_t kde_bandwidth;   /* 0: Silverman factor (3n/4)^(-1/5); 1: Scott n^(-1/5) */
     int32_t reject_rule;     /* 0: Bernoulli, reject iff u >= P(A|d); 1: reject iff P(A|d) < 1/2 */
     int32_t min_kde_samples; /* below this many entries in either list P(A|d) := 0 (>= 2) */
-    int32_t cluster_size;    /* 0 = choose automatically; else 1..8 CTAs per row / position */
+    int32_t cluster_size;    /* 0 = choose automatically; else 1..8 CTAs per position in adasd_verify on 16-byte
+                                aligned bf16 rows, 1, 2, 4 or 8 per row in draft steps; other kernels deal
+                                their rows out themselves and do not look at it */
     int32_t device;          /* CUDA device ordinal */
 } adasd_config;
 
@@ -150,7 +155,7 @@ int adasd_draft_entropy(adasd_ctx* ctx, const void* logits_dev, int64_t row_stri
  *   record            host struct of device arrays to receive per-position values
  *                     (NULL: none)
  * Candidate i is rejected iff x_i != y_i and Reject(P(A|d_i)); the scan stops at the
- * first rejection.  With ADASD_FUSE_UPDATE the same launch appends to the lists and
+ * first rejection.  With ADASD_FUSE_UPDATE the same call appends to the lists and
  * recomputes T_G = mean(L_E^R); without it the state is left unchanged and
  * adasd_update_thresholds() applies the update from a record.
  */

@@ -35,36 +35,9 @@ __device__ __forceinline__ void tmem_alloc(uint32_t* smem_dst, uint32_t ncols) {
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
-// 2 N consecutive columns of this thread's lane: a[0..N-1] then b[0..N-1]
-__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&a)[8], const float (&b)[8]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
-        ::"r"(taddr), "f"(a[0]), "f"(a[1]), "f"(a[2]), "f"(a[3]), "f"(a[4]), "f"(a[5]), "f"(a[6]), "f"(a[7]),
-          "f"(b[0]), "f"(b[1]), "f"(b[2]), "f"(b[3]), "f"(b[4]), "f"(b[5]), "f"(b[6]), "f"(b[7])
-        : "memory");
-}
-__device__ __forceinline__ void tmem_st(uint32_t taddr, const float (&a)[4], const float (&b)[4]) {
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                 ::"r"(taddr), "f"(a[0]), "f"(a[1]), "f"(a[2]), "f"(a[3]), "f"(b[0]), "f"(b[1]), "f"(b[2]), "f"(b[3])
-                 : "memory");
-}
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-// The loads are asynchronous: the registers hold the values only after tmem_wait_ld, which
+// Loads are asynchronous: the registers hold the values only after tmem_wait_ld, which
 // takes them as operands so that nothing that uses them can be scheduled ahead of the wait.
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&a)[8], float (&b)[8]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=f"(a[0]), "=f"(a[1]), "=f"(a[2]), "=f"(a[3]), "=f"(a[4]), "=f"(a[5]), "=f"(a[6]), "=f"(a[7]),
-          "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3]), "=f"(b[4]), "=f"(b[5]), "=f"(b[6]), "=f"(b[7])
-        : "r"(taddr)
-        : "memory");
-}
-__device__ __forceinline__ void tmem_ld(uint32_t taddr, float (&a)[4], float (&b)[4]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=f"(a[0]), "=f"(a[1]), "=f"(a[2]), "=f"(a[3]), "=f"(b[0]), "=f"(b[1]), "=f"(b[2]), "=f"(b[3])
-                 : "r"(taddr)
-                 : "memory");
-}
 __device__ __forceinline__ void tmem_wait_ld(float (&a)[8], float (&b)[8]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;"
                  : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]),
@@ -72,13 +45,6 @@ __device__ __forceinline__ void tmem_wait_ld(float (&a)[8], float (&b)[8]) {
                  :
                  : "memory");
 }
-__device__ __forceinline__ void tmem_wait_ld(float (&a)[4], float (&b)[4]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(b[0]), "+f"(b[1]), "+f"(b[2]), "+f"(b[3])
-                 :
-                 : "memory");
-}
-
 // {x, x} as an operand of packed arithmetic, kept in its register pair: a pair the compiler can see through
 // is made again at its uses, up to two moves for each packed instruction.
 __device__ __forceinline__ float2 pair2(float x) {
@@ -102,8 +68,7 @@ __device__ __forceinline__ double warp_sum_f64(double v) {
 // A row is cut into units of 16 bytes that are ALIGNED IN MEMORY, whatever the row's own address:
 // a row that starts m elements past a 16-byte boundary has unit u = its elements u N - m ..
 // u N - m + N - 1, and the elements before its start and past its end read as -inf.  Per type: N
-// elements a unit, packed maximum with NaN kept, the cut of an adjusted distribution (to -inf), the range
-// of the difference of two rows, unpacking to fp32 with -inf (and NaN) clamped to a finite floor
+// elements a unit, packed maximum with NaN kept, the cut of an adjusted distribution (to -inf), unpacking to fp32 with -inf (and NaN) clamped to a finite floor
 // (unpack_raw: not clamped, for sums in which no product with a -inf occurs).
 template <typename T>
 struct Unit;
@@ -129,7 +94,6 @@ struct Unit<__nv_bfloat16> {
         return fmaxf(v.x, v.y);
     }
     using Cut = uint32_t;
-    static __device__ __forceinline__ Cut no_cut() { return kNoCut2; }
     static __device__ __forceinline__ Cut make_cut(float c) { return cut_pair(c); }
     static __device__ __forceinline__ uint32_t cut2(uint32_t a, uint32_t c) {
         uint32_t m;
@@ -149,8 +113,6 @@ struct Unit<__nv_bfloat16> {
             if (2 * j + 1 < lo || 2 * j + 1 >= hi) p[j] = (p[j] & 0xFFFFu) | 0xFF800000u;
         }
     }
-    // largest and smallest z_t - z_d, packed pairs rounded to bf16 (0 only for equal values); tokens that
-    // both rows exclude (-inf - -inf) do not count
     static __device__ __forceinline__ void unpack(const uint4& w, float2 (&z)[4]) {
         z[0] = unpack2(bclamp2(w.x));
         z[1] = unpack2(bclamp2(w.y));
@@ -198,7 +160,6 @@ struct Unit<float> {
         return m;
     }
     using Cut = float;
-    static __device__ __forceinline__ Cut no_cut() { return -INFINITY; }
     static __device__ __forceinline__ Cut make_cut(float c) { return c; }
     static __device__ __forceinline__ uint32_t cut1(uint32_t w, float c) {
         return __uint_as_float(w) < c ? 0xFF800000u : w;

@@ -35,7 +35,7 @@
 // warps of a quarter split the columns: 160 each = two halves (position parity) of kSHead
 // slots of 16 columns; a slot holds one iteration's 8 target and 8 draft values per lane.
 //
-// Every wait (buffer filled, partials in, totals in, message ready, sums in, queue) is bounded:
+// Every wait (buffer filled, partials in, totals in, message ready, sums in) is bounded:
 // a warp whose wait expires sets ADASD_STATUS_TIMEOUT, stops waiting and copying, and walks
 // through the rest of the protocol, so the kernel always ends.
 #pragma once
@@ -105,16 +105,6 @@ struct __align__(16) SpecShared {
     int32_t n_final;                  // leader: number of positions of this cluster, -1 until known
     int32_t fin_done;                 // leader: positions finalised so far (written by the tail warp)
 };
-
-__device__ __forceinline__ void st_cluster_u32(uint32_t remote_addr, uint32_t v) {
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote_addr), "r"(v) : "memory");
-}
-__device__ __forceinline__ uint32_t ld_cluster_u32(uint32_t remote_addr) {
-    uint32_t v;
-    asm volatile("ld.volatile.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(remote_addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void fence_cluster() { asm volatile("fence.acq_rel.cluster;" ::: "memory"); }
 
 // ---- tensor memory as a scratchpad ---------------------------------------------------------
 // 16 consecutive columns of this thread's lane: a[0..7] then b[0..7]
@@ -335,9 +325,9 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
     // thread to the three compute warpgroups (8 each): setmaxnreg draws on what the CTA was launched
     // with, so what one side gains the other must have given up first.  With the head of a position
     // in tensor memory the compute warps keep at most 80 registers of 2^t values, and 136 leave
-    // them without spills; the tail warp's float64 finalisation and the queue workers' KDE loop get
-    // by on 104 (measured on one GPU: 144 / 80, 136 / 104, 128 / 128 and 152 / 56 give 0.4933,
-    // 0.4898, 0.4937 and 0.4955 ms on the largest workload).
+    // them without spills; the tail warp's float64 finalisation gets by on 104 (128 sequences of 16
+    // candidates, 151936 tokens, measured while the service warps also ran the sequences' tails: 144 / 80, 136 / 104,
+    // 128 / 128 and 152 / 56 gave 0.4933, 0.4898, 0.4937 and 0.4955 ms).
     if (warp < kSW) asm volatile("setmaxnreg.inc.sync.aligned.u32 136;");
     else asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
     bool alive = true;         // false after a wait expired: this warp stops waiting and copying
@@ -570,7 +560,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
         };
 
         // The 2^t values of iteration k (compile-time k after unrolling): out of tensor memory
-        // (synchronously; the sampling scans and the vanilla residual use this) or from registers.
+        // (synchronously; the sampling scan uses this) or from registers.
         auto load_kept = [&](int k, int n, bool with_d, float (&a)[8], float (&b)[8]) {
             if (k < KH) {
                 if (with_d) {
@@ -661,7 +651,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
             return lastp;
         };
 
-        // ---- pass C (AdaSD mode) over the kept values of position n ---------------------------
+        // ---- pass C over the kept values of position n ---------------------------
         // NEAR == false: A = sum (p+q) log2 (p+q) and the overlap indicator sum 2^t_p 2^t_q.
         // NEAR == true (no logit of the two rows differs by more than kSNearDz): the divergence
         // itself from non-negative terms, D_JS = 1/4 sum s phi(u) with s = p + q, u = (q - p) / s and
@@ -864,7 +854,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
 
             const uint32_t fl = __reduce_or_sync(0xFFFFFFFFu, __float_as_uint(e1.z));
             const bool bad = (fl & 1u) || !(Mt > kFloorL) || !(Md > kFloorL);
-            // AdaSD: the two rows are nearly equal everywhere -> pass C in its well-conditioned form
+            // the two rows are nearly equal everywhere -> pass C in its well-conditioned form
             const bool near = !bonus && !bad && (fl & 2u) && warp_max_f32(e1.w) * inv_temp <= kSNearDz;
             const int act = near ? 5 : 1;
 
@@ -963,7 +953,7 @@ spec_verify_kernel(VerifyParams p, ClusterGeom gq) {
     } else if (warp == kSTail) {
         // ================================ tail warp =======================================
         // Leader CTA only: finalises every position of the cluster, in order, as soon as its sums
-        // are in, and runs the tail of each sequence whose last position that was.
+        // are in.
         if (leader) {
             // leader: the published scalars of position number m, once every compute warp of the
             // cluster has sent its pass-C sums (they did before publishing their next partials)

@@ -219,7 +219,7 @@ struct RowSums {
 // Sweep-2 terms of one unit of both rows: the overlap indicator PQ += 2^t_p 2^t_q, and the divergence from
 // non-negative terms, D_JS = 1/4 sum s phi(u) with s = p + q, u = |q - p| / s and
 // phi(u) = (1-u) ln(1-u) + (1+u) ln(1+u), which do not cancel however close the rows are:
-//   u < 1/2: u^2 + u^4/6 + u^6/15 + u^8/28 + u^10/45 (good to 1e-5 of phi there);
+//   u < 1/2: u^2 + u^4/6 + u^6/15 + u^8/28 + u^10/45 (low by at most 1.7e-5 of phi, at u = 1/2);
 //   else   : 2 ln(1+u) - (1-u) |ln(p / q)|, the logarithm of p / q from the logits and 1 - u = 2 min(p,q) / s.
 // Four special-function results a pair.
 struct PairConsts {

@@ -50,8 +50,8 @@ def test_lockstep_rounds_under_warpers(torch, V, dtype, warpers):
 
 
 def test_many_rows_take_the_three_kernel_vanilla_path_under_warpers(torch):
-    """352 rows a round: adasd_vanilla_verify runs row_lse_kernel, vanilla_accept_kernel and
-    vanilla_sample_kernel, adasd_verify the warp-specialised kernel, all on the adjusted rows."""
+    """352 rows a round: adasd_vanilla_verify streams the rows and finishes each sequence, adasd_verify runs the
+    warp-specialised kernel, all on the adjusted rows."""
     from tests.lockstep import Lockstep
     wl = synth.WORKLOADS["C3"].scaled(name="warp_manyrows", B=32, K=5, V=8200, rounds=8)
     rep = Lockstep(wl, follow=[0, 7, 13, 21, 30, 31], min_kde_samples=3, check_lists_every=4,
