@@ -47,9 +47,9 @@ import synth  # noqa: E402
 METRIC = "verify_logit_rows_per_s"
 UNIT = "rows/s"
 # DRAM bytes of one verify launch (dram__bytes_read.sum + dram__bytes_write.sum) per algorithmic
-# byte, from the ncu capture of workload C3 summarised under profiles/ (144.14 MB against
+# byte, from the ncu capture of workload C3 summarised under profiles/ (143.31 MB against
 # 139.54 MB); traffic grows in proportion to the rows read, so other workloads scale by it.
-NCU_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.033
+NCU_TRAFFIC_PER_ALGORITHMIC_BYTE = 1.027
 
 
 def measured_peak_gbs():
