@@ -22,7 +22,6 @@
 namespace adasd {
 
 constexpr int kSelThreads = 512;
-constexpr int kSelWarps = kSelThreads / 32;
 constexpr int kSelMaxP = 8;
 constexpr int kSelList = 1024;
 constexpr int kSelMinV = 4096;                       // shorter rows: the radix descent
@@ -57,16 +56,13 @@ struct SelShared {
         struct {
             unsigned long long w[kSelList];          // everybody's candidates and their masses
             float all[kSelList];
-            float part[kSelList];                    // the candidates as they come in: kSelList / P places for every CTA,
-            float more[kSelList];                    // and those beyond them
         };
     };
     float list[kSelList];                            // this CTA's candidates
-    uint32_t cnt[2][kSelWarps];                      // counts of the bisection steps, by warp
-    uint32_t big[kSelWarps], small[kSelWarps];
+    uint32_t cnt[32];                                // counts of the bisection steps
+    uint32_t big, small;
     int32_t n, n_eq;                                 // candidates, elements equal to tau (of this CTA)
-    int32_t at, n_more;                              // where this CTA's surplus goes; rank 0: the length of more
-    int32_t ns[kSelMaxP], eqs[kSelMaxP];             // rank 0: n and n_eq of all CTAs
+    int32_t at, total, eq;                           // where this CTA's go; rank 0: of all CTAs
     uint32_t bad;
     uint32_t tau;                                    // key
     uint32_t key_k, key_p;
@@ -82,7 +78,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) row_cutoff_select_kernel(CutPa
     __shared__ SelShared sh;
     cg::cluster_group cluster = cg::this_cluster();
     const int P = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     // (a verification round: the target rows, then the draft rows)
     int row = blockIdx.x / P;
     if (row >= p.B * p.R) {
@@ -111,10 +107,14 @@ __global__ void __launch_bounds__(kSelThreads, 3) row_cutoff_select_kernel(CutPa
         if (u == NU - 1 && u * N + N > p.V) U::mask(w, 0, p.V - u * N);
         return w;
     };
+    if (tid < 32) sh.cnt[tid] = 0u;
     if (tid == 0) {
+        sh.big = 0u;
+        sh.small = 0xFFFFFFFFu;
         sh.n = 0;
         sh.n_eq = 0;
-        sh.n_more = 0;
+        sh.total = 0;
+        sh.eq = 0;
         sh.bad = 0u;
         sh.key_k = 0u;
         sh.key_p = 0xFFFFFFFFu;
@@ -177,13 +177,11 @@ __global__ void __launch_bounds__(kSelThreads, 3) row_cutoff_select_kernel(CutPa
         big = __reduce_max_sync(0xFFFFFFFFu, big);
         small = __reduce_min_sync(0xFFFFFFFFu, small);
         if (lane == 0) {
-            sh.big[warp] = big;
-            sh.small[warp] = small;
+            atomicMax(&sh.big, big);
+            atomicMin(&sh.small, small);
         }
         __syncthreads();
-        // (every warp folds what the sixteen left: one barrier a step, and no atomic that they would queue at)
-        big = __reduce_max_sync(0xFFFFFFFFu, sh.big[lane & (kSelWarps - 1)]);
-        uint32_t lo = __reduce_min_sync(0xFFFFFFFFu, sh.small[lane & (kSelWarps - 1)]), hi = big;      // at least k keys at or above lo
+        uint32_t lo = sh.small, hi = sh.big;         // at least k keys at or above lo
         const uint32_t need = (uint32_t)p.top_k, enough = need + max(16u, need / 4u);
         for (int it = 0; lo < hi; ++it) {            // (halves hi - lo: at most 32 times)
             const uint32_t mid = lo + (hi - lo + 1u) / 2u;
@@ -191,9 +189,9 @@ __global__ void __launch_bounds__(kSelThreads, 3) row_cutoff_select_kernel(CutPa
 #pragma unroll
             for (int q = 0; q < 2 * kSelMaxP; ++q) c += key[q] >= mid ? 1u : 0u;
             c = __reduce_add_sync(0xFFFFFFFFu, c);
-            if (lane == 0) sh.cnt[it & 1][warp] = c;
+            if (lane == 0 && c) atomicAdd(&sh.cnt[it & 31], c);
             __syncthreads();
-            c = __reduce_add_sync(0xFFFFFFFFu, lane < kSelWarps ? sh.cnt[it & 1][lane] : 0u);
+            c = sh.cnt[it & 31];
             if (c < need) {
                 hi = mid - 1u;
             } else {
@@ -203,7 +201,7 @@ __global__ void __launch_bounds__(kSelThreads, 3) row_cutoff_select_kernel(CutPa
         }
         if (tid == 0) {
             sh.tau = value(lo);
-            sh.m = K32::value(value(big));
+            sh.m = K32::value(value(sh.big));
         }
     }
     cluster.sync();
@@ -241,118 +239,62 @@ __global__ void __launch_bounds__(kSelThreads, 3) row_cutoff_select_kernel(CutPa
         }
     }
     __syncthreads();
-    // everybody's candidates to rank 0: to the CTA's own places, so that nobody asks where they go, but for a surplus
-    const int mine = min(sh.n, kSelList + 1), cap = kSelList / P;
+    // everybody's candidates into rank 0's list
+    const int mine = sh.n;
     if (tid == 0) {
-        r0->ns[rank] = mine;
-        r0->eqs[rank] = sh.n_eq;
+        sh.at = atomicAdd(&r0->total, mine);
+        atomicAdd(&r0->eq, sh.n_eq);
     }
-    for (int i = tid; i < min(mine, cap); i += kSelThreads) r0->part[rank * cap + i] = sh.list[i];
-    if (mine > cap) {                                // (the same for the whole CTA)
-        if (tid == 0) sh.at = atomicAdd(&r0->n_more, mine - cap);
-        __syncthreads();
-        if (mine <= kSelList && sh.at + mine - cap <= kSelList)
-            for (int i = cap + tid; i < mine; i += kSelThreads) r0->more[sh.at + i - cap] = sh.list[i];
-    }
+    __syncthreads();
+    if (mine <= kSelList && sh.at + mine <= kSelList)
+        for (int i = tid; i < mine; i += kSelThreads) r0->all[sh.at + i] = sh.list[i];
     cluster.sync();                                  // (nobody writes to rank 0 any more)
     if (rank != 0) return;
-    int n = 0, n_eq = 0;
-    for (int r = 0; r < P; ++r) {
-        n += sh.ns[r];
-        n_eq += sh.eqs[r];
-    }
+    const int n = sh.total, n_eq = sh.eq;
     if (bad || n > kSelList) {
         if (tid == 0) *out = bad ? -INFINITY : __int_as_float(0x7FC00000);
         return;
     }
 
-    {                                                // one list, whole trips of 8 to walk it in
-        int at = 0;
-        for (int r = 0; r < P; ++r) {
-            const int c = min(sh.ns[r], cap);
-            for (int i = tid; i < c; i += kSelThreads) sh.all[at + i] = sh.part[r * cap + i];
-            at += c;
-        }
-        for (int i = tid; at + i < n; i += kSelThreads) sh.all[at + i] = sh.more[i];
-        if (tid < 8 && n + tid < kSelList) {
-            sh.all[n + tid] = -INFINITY;
-            sh.w[n + tid] = 0ull;
-        }
-    }
-    __syncthreads();
-    const bool use_p = p.top_p < 1.f;
-    constexpr int kMine = kSelList / kSelThreads;
-    float mv[kMine];                                 // this thread's candidates
-#pragma unroll
-    for (int j = 0; j < kMine; ++j) {
-        const int i = tid + j * kSelThreads;
-        mv[j] = i < n ? sh.all[i] : -INFINITY;
-        if (use_p && i < n) sh.w[i] = (unsigned long long)__double2ll_rn(exp2((double)(fmaxf(mv[j], kFloor) - m) * p.c1) * kCutFix);
-    }
-    if (use_p) __syncthreads();
-
     // 3. the k-th largest: the value with fewer than k above it and k at or above it (tau itself when the list
-    // is shorter than k); in the same walk the masses above and at or above every candidate.
-    // (entries of -inf at the end of the list are above nothing and weigh nothing)
-    unsigned long long above[kMine];
-#pragma unroll
-    for (int j = 0; j < kMine; ++j) {
-        above[j] = 0ull;
-        if (tid + j * kSelThreads >= n) continue;
-        const float v = mv[j];
+    // is shorter than k)
+    for (int i = tid; i < n; i += kSelThreads) {
+        const float v = sh.all[i];
         int gt = 0, ge = 0;
-        unsigned long long most = 0ull;
-        if (use_p) {
-#pragma unroll 1
-            for (int q0 = 0; q0 < n; q0 += 8) {
-#pragma unroll
-                for (int q = q0; q < q0 + 8; ++q) {
-                    const float x = sh.all[q];
-                    const unsigned long long w = sh.w[q];
-                    gt += x > v;
-                    ge += x >= v;
-                    above[j] += x > v ? w : 0ull;
-                    most += x >= v ? w : 0ull;
-                }
-            }
-        } else {
-#pragma unroll 1
-            for (int q0 = 0; q0 < n; q0 += 8) {
-#pragma unroll
-                for (int q = q0; q < q0 + 8; ++q) {
-                    const float x = sh.all[q];
-                    gt += x > v;
-                    ge += x >= v;
-                }
-            }
+        for (int q = 0; q < n; ++q) {
+            gt += sh.all[q] > v;
+            ge += sh.all[q] >= v;
         }
-        // (one value, perhaps several threads)
-        if (gt < p.top_k && ge >= p.top_k) {
-            sh.key_k = K32::of(v);
-            sh.S = most;
-        } else if (n < p.top_k && ge >= n) {         // the smallest: all of the list
-            sh.S = most;
-        }
+        if (gt < p.top_k && ge >= p.top_k) sh.key_k = K32::of(v);            // (one value, perhaps several threads)
+        sh.w[i] = (unsigned long long)__double2ll_rn(exp2((double)(fmaxf(v, kFloor) - m) * p.c1) * kCutFix);
     }
     __syncthreads();
     const uint32_t key_tau = sh.tau, key_k = n < p.top_k ? key_tau : sh.key_k;
-    if (!use_p) {
+    if (!(p.top_p < 1.f)) {
         if (tid == 0) *out = K32::value(key_k);
         return;
     }
     // top-p of what is left: the smallest value with less than top_p of the mass strictly above it
     const bool with_tau = key_k == key_tau && n < p.top_k;
     const unsigned long long w_tau = (unsigned long long)__double2ll_rn(exp2((double)(fmaxf(tau, kFloor) - m) * p.c1) * kCutFix);
+    unsigned long long part = 0ull;
+    for (int i = tid; i < n; i += kSelThreads)
+        if (K32::of(sh.all[i]) >= key_k) part += sh.w[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(0xFFFFFFFFu, part, o);
+    if (lane == 0 && part) atomicAdd(&sh.S, part);
+    __syncthreads();
     const unsigned long long list_mass = sh.S, S = list_mass + (with_tau ? (unsigned long long)n_eq * w_tau : 0ull);
     const double thr = (double)p.top_p * (double)S;
-    uint32_t key_p = 0xFFFFFFFFu;
-#pragma unroll
-    for (int j = 0; j < kMine; ++j) {
-        const uint32_t k = K32::of(mv[j]);
-        if (tid + j * kSelThreads < n && k >= key_k && (double)above[j] < thr) key_p = min(key_p, k);
+    for (int i = tid; i < n; i += kSelThreads) {
+        const float v = sh.all[i];
+        const uint32_t k = K32::of(v);
+        if (k < key_k) continue;
+        unsigned long long above = 0ull;
+        for (int q = 0; q < n; ++q)
+            if (sh.all[q] > v) above += sh.w[q];
+        if ((double)above < thr) atomicMin(&sh.key_p, k);
     }
-    key_p = __reduce_min_sync(0xFFFFFFFFu, key_p);
-    if (lane == 0 && key_p != 0xFFFFFFFFu) atomicMin(&sh.key_p, key_p);
     if (tid == 0 && with_tau && (double)list_mass < thr) atomicMin(&sh.key_p, key_tau);
     __syncthreads();
     if (tid == 0) *out = K32::value(max(key_k, sh.key_p));
