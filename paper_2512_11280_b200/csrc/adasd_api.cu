@@ -483,13 +483,20 @@ int launch_cutoffs(adasd_ctx* ctx, CutParams c, const CutParams* second, cudaStr
     // top-k on: selection, a row over as many CTAs as are resident at once; it flags what it cannot do
     int P = 1;
     while (P < kSelMaxP && rows * P * 2 <= 3LL * ctx->sm_count) P *= 2;
-    // ... up to a k where it is the faster one.  It compares its candidates, a few times k, with one another.  Against the
-    // histogram of aligned bf16 rows, us a draft call of random rows with a top-p cut behind it: V=128256, 32 rows, k=200
-    // 38 / 47, k=256 46 / 39; V=32000 k=200, 8 rows 28 / 36, 32 rows 39 / 37, 256 rows 42 / 63; and without top-p, where the
-    // histogram is a count, 32 rows k=20 23 / 22, k=100 26 / 21, 256 rows k=100 26 / 31.  Up to 200 the candidates fit the
-    // list even of a row sorted by its logits, which has the most (five times k); such rows lose (V=32000 k=64 33 / 35, k=200
-    // 129 / 36).  Against the radix descent: always, unless the few groups of a row with one CTA leave so many
-    // candidates that it hands rows over (256 rows, V=32000, k=400 66 / 146, k=512 318 / 228).
+    // ... up to a k where it is the faster one.  It compares its candidates, a few times k, with one another; the histogram of
+    // aligned bf16 rows depends little on k, but takes a CTA a row and a launch an array.  Selection / histogram, us a call,
+    // temperature 0.8, rows of s N(0, 1) - ln(rank), inputs beyond L2:
+    // - a top-p cut behind it, draft calls: V=128256, 32 rows, k=200 41 / 46; V=32000, 8 rows k=200 28 / 34, 32 rows k=100
+    //   28 / 34 and k=200 37 / 36, 256 rows k=200 46 / 67 (the worst: V=8192, 111 rows, k=200 41 / 36);
+    // - verification of 16 sequences, K=5: V=32000, with top-p k=200 59 / 84, without it k=64 42 / 50;
+    // - draft calls without top-p, where the histogram is a count: V=128256, 32 rows k=100 27 / 30, 256 rows k=100 54 / 62;
+    //   V=32000, 8 rows k=64 18 / 18, 256 rows k=64 29 / 35.  Here the limits are beyond the crossing while the histogram is
+    //   one wave of more than 16 rows: V=8192, 55 rows, k=40 24 / 17; V=32000, 32 rows, k=40 23 / 19; V=128256, 111 rows,
+    //   k=200 47 / 36.  A line through that range is not drawn yet.
+    // Up to 200 the candidates fit the list even of a row sorted by its logits, which has the most (five times k); such rows
+    // lose (2 N(0, 1), V=32000, 8 rows, top-p, k=64 32 / 31, k=200 124 / 32).  Against the radix descent: always, unless the
+    // few groups of a row with one CTA leave so many candidates that it hands rows over (the same, 256 fp32 rows, not sorted,
+    // k=400 114 / 221, k=448 140 / 222, k=512 293 / 225).
     const bool histogram = bf && vec1 && vec2 && ctx->cut_hist;
     const int k_most = !histogram ? std::min(kSelMaxK, 448 * P) : c.V >= 65536 || c.top_p < 1.f || P == 1 ? 200 : 64;
     const bool select = c.top_k > 0 && c.top_k < c.V && c.top_k <= k_most && c.V >= kSelMinV && rows <= 0x7FFFFFFF / kSelMaxP;
